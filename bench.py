@@ -429,7 +429,7 @@ def ours_arm(args):
                       "fp32_bf16": "fp32 (bf16 solute storage)"}[args.precision],
             "data": "synthetic", "config": cfg, "roofline": roofline,
             "kernel_ms": {k: statistics.mean(v) for k, v in kern.items()},
-            "gpu_launches": 3 * args.steps}
+            "gpu_launches": 4 * args.steps}
     if clk:
         line["clocks"] = clk
 

@@ -164,8 +164,8 @@ pslbm_status pslbm_set_stream(void* cuda_stream);
  *             tau <= 0.5, k >= (1 - J0)/2 for a reactive species, bad indices).
  * On success *out holds a new handle; on failure *out is NULL and nothing leaks.
  * The initial liquid threshold is half the maximum initial rho1 over fluid nodes.
- * The handle's device state is one allocation (pslbm_device_bytes; the tile
- * lists of the step kernels are allocated on demand); the inputs are copied
+ * The handle's device state is one allocation (pslbm_device_bytes; a batch's work
+ * list is allocated on demand); the inputs are copied
  * with cudaMemcpyAsync on the library stream (page-locked host buffers copy
  * fastest) and the call synchronises once before it returns, after which the
  * caller may reuse them. */
@@ -186,7 +186,7 @@ pslbm_status pslbm_read_fields(pslbm_t h, uint32_t fields, void* const* out);
 
 /* Run n >= 1 steps without graph capture, timing each kernel with CUDA
  * events on the library stream, and synchronise.  kernel_ms[3] receives the
- * mean duration per step (ms) of the bulk kernel (Eqs. 6-31 fused), the VOP
+ * mean duration per step (ms) of the streaming kernels (Eqs. 6-31), the VOP
  * kernel (Eqs. 32-35) and the amendment kernel (Section 4.5); total_ms the
  * mean time per step from the first to the last event.  Same results as
  * pslbm_step. */
@@ -201,34 +201,24 @@ pslbm_status pslbm_set_step_limit(pslbm_t h, int64_t limit);
  * the read-back scratch of pslbm_read_fields). */
 pslbm_status pslbm_estimate_device_bytes(const pslbm_params* p, uint64_t* bytes);
 
-/* Tile shape of the step kernels, which also sets the nodes per thread of a
- * 256-thread block: 16x16 or 32x8 (one node per thread), 16x32 or 32x16 (two
- * nodes per thread: thread (tx, ty) computes rows ty and ty + 256 / tile_x).
- * (0, 0), the default, leaves the shape to timing: the next step call long
- * enough to try every open variant (tile shape x staging, 4 steps each, in
- * two passes, the second in reverse order; the steps advance the simulation
- * like any others) times them and keeps the fastest by its better pass;
- * the results do not depend on the variant.  tuned reports whether the variant
- * has been chosen (by timing, or because only one was left open).
- * PSLBM_ERR_PARAM for another shape, or for a two-node shape while staging 1
+/* Nodes of a warp's tile of the streaming kernels: 16x16 or 32x8 (256 nodes,
+ * taken as 32 columns by 8 rows), 16x32 or 32x16 (512 nodes, 32 columns by 16
+ * rows).  (0, 0), the default, takes 32x8 and fewer rows on lattices too small
+ * to occupy the device.  The results do not depend on the shape.  get reports
+ * the shape asked for, or 32x8; tuned is always 1 (nothing is left to timing).
+ * PSLBM_ERR_PARAM for another shape, or for a 512-node shape while staging 1
  * is fixed (the handle is left as it was). */
 pslbm_status pslbm_set_tile_shape(pslbm_t h, int32_t tile_x, int32_t tile_y);
 pslbm_status pslbm_get_tile_shape(pslbm_t h, int32_t* tile_x, int32_t* tile_y, int32_t* tuned);
 
-/* Staging of the bulk kernel's populations: 0 plain per-thread loads; 1 TMA
- * copies of each tile's D2Q9 and D2Q5 population boxes into shared memory two
- * tiles ahead (two stages, two blocks per SM; one-node tile shapes only); 2
- * TMA copies of the D2Q9 box only, one tile ahead, re-read from shared memory
- * where used, with the solute populations loaded directly (two stages; three
- * blocks per SM with one node per thread, two with two, whose box has no x
- * halo).  1 and 2 are available for the FP32-population precisions
- * when a row of the lattice is a multiple of 16 bytes (nx a multiple of 4, and
- * of 8 with 16-bit solutes).  -1 (the default) leaves the choice to timing.
+/* Staging of populations in shared memory: -1 (the default), 0, 1 or 2.  The
+ * kernels load populations straight into registers, so the choice changes
+ * neither results nor speed; it is checked and reported.  1 and 2 are
+ * accepted for the FP32-population precisions when a row of the lattice is a
+ * multiple of 16 bytes (nx a multiple of 4, and of 8 with 16-bit solutes).
  * PSLBM_ERR_PARAM for 1 or 2 where they are not available, and for 1 while a
- * two-node tile shape is fixed.  The results are bit-identical either way.  get reports the
- * staging in use and whether staging is available for the handle.  A staged
- * kernel whose copy does not arrive within about a second stops and sets
- * PSLBM_ERR_TIMEOUT (sticky), reported by the next sync or read. */
+ * 512-node tile shape is fixed.  get reports the staging asked for (0 for -1)
+ * and whether 1 and 2 are available for the handle. */
 pslbm_status pslbm_set_staging(pslbm_t h, int32_t mode);
 pslbm_status pslbm_get_staging(pslbm_t h, int32_t* staged, int32_t* available);
 
@@ -236,7 +226,7 @@ pslbm_status pslbm_get_staging(pslbm_t h, int32_t* staged, int32_t* available);
  * density over fluid nodes found by the last step (the quantity whose half is
  * the next liquid threshold, Section 4.5; the initial maximum before the first
  * step) and the device status bits (1 non-finite density, 2 EOS domain,
- * 4 event-list overflow, 8 staged-copy timeout).  Reads 72 bytes from the
+ * 4 event-list overflow).  Reads 64 bytes from the
  * device and synchronises the library stream; no kernel runs.  Returns the
  * matching error status when a bit is set (sticky, as for pslbm_sync).  Any
  * output pointer may be NULL. */
@@ -282,8 +272,7 @@ pslbm_status pslbm_budget_device_noalloc(pslbm_t h, double* out);
  * one launch per kernel over a packed list of tiles of all members.  The
  * members stay valid handles; they must not be stepped on their own while
  * the batch exists.  tile_x, tile_y choose the tile shape (16x16, 32x8,
- * 16x32 or 32x16, as for pslbm_set_tile_shape; 0, 0: time every open variant
- * on the first steps and keep the fastest). */
+ * 16x32 or 32x16, as for pslbm_set_tile_shape; 0, 0: the default). */
 pslbm_status pslbm_batch_create(int32_t n, const pslbm_t* members, int32_t tile_x, int32_t tile_y,
                                 pslbm_batch_t* out);
 pslbm_status pslbm_batch_step(pslbm_batch_t b, int64_t n);
@@ -311,9 +300,7 @@ pslbm_status pslbm_batch_destroy(pslbm_batch_t b);
  * each pslbm_server_advance() admits queued requests in arrival order while
  * the device-memory estimate of the resident simulations stays within
  * hbm_budget_bytes (and their count within max_active), re-packs the resident
- * simulations into batches when the set changed (one per species count; the
- * first batch of a species count chooses the kernel variant by timing when a
- * chunk is long enough, and the batches re-packed after it take that variant),
+ * simulations into batches when the set changed (one per species count),
  * advances them by chunk_steps
  * steps (a simulation is frozen at its step budget), and retires requests that
  * reached their step budget or whose total solid volume changed by at least

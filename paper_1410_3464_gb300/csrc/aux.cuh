@@ -22,8 +22,8 @@ __global__ void k_init(DevInst* __restrict__ Ip, const uint8_t* __restrict__ mas
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
       const R w = w9<R>(a);
-      st<TF, R>(F + a * N + node, fl ? w * r1 - w * fshift<R>(P, 0, t) : R(0));
-      st<TF, R>(F + (9 + a) * N + node, fl ? w * r2 - w * fshift<R>(P, 1, t) : R(0));
+      st<TF, R>(F + foff((int)node) + a * CELL, fl ? w * r1 - w * fshift<R>(P, 0, t) : R(0));
+      st<TF, R>(F + foff((int)node) + (9 + a) * CELL, fl ? w * r2 - w * fshift<R>(P, 1, t) : R(0));
     }
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
@@ -32,7 +32,7 @@ __global__ void k_init(DevInst* __restrict__ Ip, const uint8_t* __restrict__ mas
 #pragma unroll
       for (int a = 0; a < 5; ++a) {
         const R ja = a == 0 ? J0 : Ja;
-        gst<TG, R>(P, k, G + ((long long)k * 5 + a) * N + node, ja * c - ja * rp<R>(P).shift_c[k]);
+        gst<TG, R>(P, k, G + goff<NS>((int)node) + (k * 5 + a) * CELL, ja * c - ja * rp<R>(P).shift_c[k]);
       }
     }
   }
@@ -63,8 +63,8 @@ __global__ void k_fields(const DevInst* __restrict__ Ip, double* __restrict__ o_
       R f1[9], f2[9];
 #pragma unroll
       for (int a = 0; a < 9; ++a) {
-        f1[a] = ldc<R>(F + a * N + node);
-        f2[a] = ldc<R>(F + (9 + a) * N + node);
+        f1[a] = ldc<R>(F + foff((int)node) + a * CELL);
+        f2[a] = ldc<R>(F + foff((int)node) + (9 + a) * CELL);
       }
       R d1 = f1[0], d2 = f2[0];
 #pragma unroll
@@ -94,8 +94,8 @@ __global__ void k_fields(const DevInst* __restrict__ Ip, double* __restrict__ o_
         if (nlv[a]) {
           R a1, a2;
           if (is_fluid(tn)) {
-            a1 = fshift<R>(P, 0, tn) + density_shifted<R>(F, N, nn);
-            a2 = fshift<R>(P, 1, tn) + density_shifted<R>(F + 9 * N, N, nn);
+            a1 = fshift<R>(P, 0, tn) + density_shifted<R>(F, 0, (int)nn);
+            a2 = fshift<R>(P, 1, tn) + density_shifted<R>(F, 1, (int)nn);
           } else {
             double u, v;
             const R theta = theta_of<R>(Ip);
@@ -133,10 +133,10 @@ __global__ void k_fields(const DevInst* __restrict__ Ip, double* __restrict__ o_
       for (int k = 0; k < NS; ++k) {
         double c = 0.0;
         if (t == T_LIQUID) {
-          const TG* gk = G + (long long)k * 5 * N;
-          R s = gldc<R>(P, k, gk + node);
+          const TG* gk = G + goff<NS>((int)node) + k * 5 * CELL;
+          R s = gldc<R>(P, k, gk);
 #pragma unroll
-          for (int a = 1; a < 5; ++a) s += gldc<R>(P, k, gk + a * N + node);
+          for (int a = 1; a < 5; ++a) s += gldc<R>(P, k, gk + a * CELL);
           c = double(rp<R>(P).shift_c[k] + s);
         }
         o_conc[k * N + node] = c;
@@ -167,8 +167,8 @@ __global__ void __launch_bounds__(BUD_THREADS) k_budget_partial(const DevInst* _
   for (long long node = lo + threadIdx.x; node < hi; node += blockDim.x) {
     const uint8_t t = T[node] & T_MASK;
     if (is_fluid(t)) {
-      const double r1 = double(fshift<R>(P, 0, t) + density_c<R>(F, N, node));
-      const double r2 = double(fshift<R>(P, 1, t) + density_c<R>(F + 9 * N, N, node));
+      const double r1 = double(fshift<R>(P, 0, t) + density_c<R>(F, 0, (int)node));
+      const double r2 = double(fshift<R>(P, 1, t) + density_c<R>(F, 1, (int)node));
       acc[0] = fmax(acc[0], r1);
       acc[1] += r1;
       acc[2] += r2;
@@ -176,10 +176,10 @@ __global__ void __launch_bounds__(BUD_THREADS) k_budget_partial(const DevInst* _
     if (t == T_LIQUID) {
 #pragma unroll
       for (int k = 0; k < NS; ++k) {
-        const TG* gk = G + (long long)k * 5 * N;
-        R s = gldc<R>(P, k, gk + node);
+        const TG* gk = G + goff<NS>((int)node) + k * 5 * CELL;
+        R s = gldc<R>(P, k, gk);
 #pragma unroll
-        for (int a = 1; a < 5; ++a) s += gldc<R>(P, k, gk + a * N + node);
+        for (int a = 1; a < 5; ++a) s += gldc<R>(P, k, gk + a * CELL);
         acc[3 + k] += double(rp<R>(P).shift_c[k] + s);
       }
     }

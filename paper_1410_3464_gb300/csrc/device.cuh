@@ -16,39 +16,13 @@ constexpr uint8_t T_MASK = 0x0F;     // low nibble: node type
 constexpr uint8_t T_NEW = 0x40;      // flag set by the amendment kernel: solid -> liquid this step
 constexpr uint8_t T_VANISH = 0x80;   // flag: liquid -> solid this step
 
-// Tile shapes of the step kernels: 256 threads, a tile of TX x TY nodes and a
-// one-node ring.  Thread (tx, ty) of a TX x RY block computes the NPT nodes
-// (tx, ty + k RY) of the tile, k < NPT (nodes per thread).  The runtime picks
-// the fastest shape per handle or batch by timing its first steps (results do
-// not depend on the shape).
-constexpr int NTHREADS = 256;
+constexpr int NTHREADS = 256;          // threads per block of the VOP and amendment kernels
 // Interface-bitmap words per warp chunk of the VOP kernel.
 constexpr int VOP_CHUNK = 4;
-template <int TX_, int RY_, int NPT_ = 1>
-struct TileShape {
-  static constexpr int TX = TX_, RY = RY_, NPT = NPT_, TY = RY_ * NPT_;
-  static constexpr int EXT_X = TX + 2, EXT_Y = TY + 2;
-  static constexpr int EXT = EXT_X * EXT_Y;
-  static constexpr int RING = EXT - TX * TY;
-  static_assert(TX * RY == NTHREADS, "one thread per column position and row of a pass");
-  static_assert(RING <= NTHREADS, "one ring node per thread");
-};
-using ShapeA = TileShape<16, 16>;      // 16 x 16, one node per thread
-using ShapeB = TileShape<32, 8>;       // 32 x 8, one node per thread
-using ShapeC = TileShape<16, 16, 2>;   // 16 x 32, two nodes per thread
-using ShapeD = TileShape<32, 8, 2>;    // 32 x 16, two nodes per thread
+// Tile shapes a caller may ask for (nodes per tile: 256 or 512).
 constexpr int NSHAPES = 4;
-constexpr int SHAPE_TX[NSHAPES] = {ShapeA::TX, ShapeB::TX, ShapeC::TX, ShapeD::TX};
-constexpr int SHAPE_TY[NSHAPES] = {ShapeA::TY, ShapeB::TY, ShapeC::TY, ShapeD::TY};
-constexpr int SHAPE_NPT[NSHAPES] = {ShapeA::NPT, ShapeB::NPT, ShapeC::NPT, ShapeD::NPT};
-// The staged bulk kernel's D2Q9 box reaches this many nodes left and right of
-// a tile of one node per thread (one ring node is needed; four keep the box's
-// x origin on a 16-byte boundary for FP32 rows), and one node above and below.
-// The box of a tile of two nodes per thread has no x halo (the tile's own x
-// origin is aligned; its side ring columns are read from global memory), so
-// that two blocks with two stages each fit on an SM.
-constexpr int STAGE_HALO_X = 4;
-__host__ __device__ constexpr int stage_halo_x(int npt) { return npt == 1 ? STAGE_HALO_X : 0; }
+constexpr int SHAPE_TX[NSHAPES] = {16, 32, 16, 32};
+constexpr int SHAPE_TY[NSHAPES] = {16, 8, 32, 16};
 
 // Per-instance scalar slots (unsigned long long each).
 enum {
@@ -60,9 +34,7 @@ enum {
   S_LIMIT = 5,     // step limit: an instance at or past it is frozen (kernels skip it)
   S_THETA = 6,     // this step's liquid threshold (half the previous maximum), FP64 bits
   S_THETAF = 7,    // the same rounded to FP32 (bits in the low word)
-  S_TILES = 8,     // tiles claimed so far by the bulk launch in progress (first instance of a
-                   // launch only; the amendment kernel sets it back to zero after every launch)
-  S_NSCAL = 9
+  S_NSCAL = 8
 };
 enum { ST_NONFINITE = 1, ST_EOS = 2, ST_EVOVERFLOW = 4, ST_TIMEOUT = 8 };
 
@@ -99,6 +71,8 @@ struct DevParams {
   int per_liq, per_gas, ramp;
   int has_G11, has_rev, useB, useF;   // G11 != 0, inv_Keq != 0, R2 active, R4 active
   int r1_surf;                        // R1 surface factor differs from 1
+  int tau_unit;                       // both relaxation times are 1
+  int has_w;                          // a fluid-solid interaction strength differs from 0
   int in_dx, in_dy, out_dx, out_dy;   // node downstream of an inlet / upstream of an outlet
   double tau[2], G11, G12, G21, a0, rho10, rho20, w_adh[2];
   double eos_a, eos_b, eos_R, eos_T;
@@ -125,15 +99,12 @@ template <> __host__ __device__ __forceinline__ const DevParamsR<float>& rp<floa
 template <> __host__ __device__ __forceinline__ const DevParamsR<double>& rp<double>(const DevParams& P) { return P.rd; }
 
 struct DevInst {
-  // TMA descriptors of the population boxes of the staged bulk kernel, per tile
-  // shape and ping-pong buffer (encoded only when the instance qualifies:
-  // FP32 populations and rows a multiple of 16 bytes; zero otherwise)
-  CUtensorMap tmf[NSHAPES][2];
-  CUtensorMap tmg[NSHAPES][2];
   DevParams P;
   void* f[2];                 // [2][9][N] populations, ping-pong
   void* g[2];                 // [ns][5][N] solute populations, ping-pong
   uint8_t* type[2];           // [N] node types, ping-pong
+  void* pot;                  // [N] potentials of this step (Pot<R>)
+  uint8_t* code;              // [N] codes of this step (C_* bits)
   double* V;                  // [2][N] V_D, V_F
   uint8_t* evt;               // [N] VOP events (zero except during a step)
   double* xs;                 // [N] overflow excess of an event node
@@ -142,12 +113,16 @@ struct DevInst {
   unsigned* vmask;            // [(N + 31) / 32] bit per node: a mineral a liquid node touched this
                               // step (set by the bulk kernel, consumed and cleared by k_vop)
   unsigned long long* scal;   // [S_NSCAL]
+  int* reslist;               // [nres] reservoir nodes
   long long N;
   int evcap;
+  int nres;
 };
 
+// Work-list entry of a batch: a tile of an instance, or (res >= 0) a chunk of its
+// reservoir nodes.
 struct Tile {
-  int inst, x0, y0, pad;
+  int inst, x0, y0, res;
 };
 
 // D2Q9 velocity set of Eq. 7 (the D2Q5 set is directions 0-4).
@@ -261,22 +236,34 @@ template <> __device__ __forceinline__ float theta_of<float>(const DevInst* Ip) 
   return __int_as_float((int)(unsigned)Ip->scal[S_THETAF]);
 }
 
+// Population layout: the nodes of a lattice in cells of CELL consecutive node
+// indices; a cell holds its nodes' 18 D2Q9 populations (component 1's nine
+// directions, then component 2's) one plane of CELL values after another, and
+// the solute array likewise the 5 NS D2Q5 ones.  foff / goff: a node's value of
+// the first plane; plane q lies q CELL values further.
+constexpr int CELL = 32;
+__host__ __device__ __forceinline__ int foff(int node) { return node + (node & ~(CELL - 1)) * 17; }
+template <int NS>
+__host__ __device__ __forceinline__ int goff(int node) { return node + (node & ~(CELL - 1)) * (5 * NS - 1); }
+
 // Eq. 9a with the population shift: delta rho summed in direction order.
 template <class R, class TF>
-__device__ __forceinline__ R density_shifted(const TF* f, long long N, long long node) {
-  R s = ld<R>(f + node);
+__device__ __forceinline__ R density_shifted(const TF* f, int comp, int node) {
+  const TF* p = f + foff(node) + comp * 9 * CELL;
+  R s = ld<R>(p);
 #pragma unroll
-  for (int a = 1; a < 9; ++a) s += ld<R>(f + a * N + node);
+  for (int a = 1; a < 9; ++a) s += ld<R>(p + a * CELL);
   return s;
 }
 
 // Same sum through plain (coherent) loads, for data written by an earlier kernel
 // of the same step.
 template <class R, class TF>
-__device__ __forceinline__ R density_c(const TF* f, long long N, long long node) {
-  R s = ldc<R>(f + node);
+__device__ __forceinline__ R density_c(const TF* f, int comp, int node) {
+  const TF* p = f + foff(node) + comp * 9 * CELL;
+  R s = ldc<R>(p);
 #pragma unroll
-  for (int a = 1; a < 9; ++a) s += ldc<R>(f + a * N + node);
+  for (int a = 1; a < 9; ++a) s += ldc<R>(p + a * CELL);
   return s;
 }
 
@@ -322,7 +309,7 @@ __device__ __forceinline__ bool liquid_at(const DevParams& P, const uint8_t* tin
                                           R theta) {
   uint8_t t = tin[node] & T_MASK;
   if (!is_fluid(t)) return false;
-  R rho1 = fshift<R>(P, 0, t) + density_shifted<R>(fin, (long long)N, node);
+  R rho1 = fshift<R>(P, 0, t) + density_shifted<R>(fin, 0, node);
   return rho1 > theta;
 }
 
@@ -533,28 +520,6 @@ __device__ __forceinline__ void potentials(const DevParams& P, R rho1, R rho2, R
   const DevParamsR<R>& Q = rp<R>(P);
   if (P.has_G11) {
     R arg = psi_arg<R>(P, rho1);
-    if (!(arg >= R(0))) {
-      status |= (arg == arg) ? ST_EOS : ST_NONFINITE;
-      arg = R(0);
-    }
-    psi = rsqrt_<R>(arg);
-  } else {
-    psi = R(0);
-  }
-  phi1 = -rexpm1<R>(-rmul<R>(rho2, Q.inv_rho20));
-  phi2 = rsub<R>(Q.a0, rexp<R>(-rmul<R>(rho1, Q.inv_rho10)));
-}
-
-// Same as potentials(), with the parameters taken from a block already staged
-// in the compute precision (shared memory in the bulk kernel).
-template <class R>
-__device__ __forceinline__ void potentials_q(const DevParamsR<R>& Q, bool has_G11, R rho1, R rho2, R& psi, R& phi1,
-                                             R& phi2, unsigned& status) {
-  if (has_G11) {
-    const R eta = Q.eos_b4 * rho1;
-    const R om = R(1) - eta;
-    const R p = rho1 * Q.eos_RT * (R(1) + eta + eta * eta - eta * eta * eta) / (om * om * om) - Q.eos_a * rho1 * rho1;
-    R arg = Q.six_over_G11 * (p - rho1 / R(3));
     if (!(arg >= R(0))) {
       status |= (arg == arg) ? ST_EOS : ST_NONFINITE;
       arg = R(0);

@@ -7,7 +7,7 @@
 // Every gather runs in the fixed order E, N, W, S, so the result does not
 // depend on thread scheduling.
 #pragma once
-#include "device.cuh"
+#include "step.cuh"
 
 namespace pslbm {
 
@@ -69,10 +69,10 @@ __device__ __forceinline__ void vop_node(const DevInst* Ip, const DevParams& P, 
       oB[b - 1] = oE[b - 1] = oF[b - 1] = R(0);
       if (nn < 0) continue;
       if (useB) {
-        oB[b - 1] = gldc<R>(P, P.iB, gout + (P.iB * 5 + b) * N + nn);
-        if (P.iE >= 0) oE[b - 1] = gldc<R>(P, P.iE, gout + (P.iE * 5 + b) * N + nn);
+        oB[b - 1] = gldc<R>(P, P.iB, gout + goff<NS>(nn) + (P.iB * 5 + b) * CELL);
+        if (P.iE >= 0) oE[b - 1] = gldc<R>(P, P.iE, gout + goff<NS>(nn) + (P.iE * 5 + b) * CELL);
       }
-      if (useF) oF[b - 1] = gldc<R>(P, P.iF, gout + (P.iF * 5 + b) * N + nn);
+      if (useF) oF[b - 1] = gldc<R>(P, P.iF, gout + goff<NS>(nn) + (P.iF * 5 + b) * CELL);
     }
 #pragma unroll
     for (int b = 1; b < 5; ++b) {
@@ -84,16 +84,16 @@ __device__ __forceinline__ void vop_node(const DevInst* Ip, const DevParams& P, 
         const R out = oB[b - 1] + sh;
         const R q = out * rp<R>(P).vB_qa;
         const R bk = out - q;
-        gst<TG, R>(P, iB, gout + (iB * 5 + b) * N + nn, bk - sh);
+        gst<TG, R>(P, iB, gout + goff<NS>(nn) + (iB * 5 + b) * CELL, bk - sh);
         sB += q;
-        if (P.iE >= 0) gst<TG, R>(P, P.iE, gout + (P.iE * 5 + b) * N + nn, oE[b - 1] + q);
+        if (P.iE >= 0) gst<TG, R>(P, P.iE, gout + goff<NS>(nn) + (P.iE * 5 + b) * CELL, oE[b - 1] + q);
       }
       if (useF) {
         const int iF = P.iF;
         const R sh = rp<R>(P).vF_sh;
         const R out = oF[b - 1] + sh;
         const R q = out * rp<R>(P).vF_qa - rp<R>(P).vF_qc;
-        gst<TG, R>(P, iF, gout + (iF * 5 + b) * N + nn, (out - q) - sh);
+        gst<TG, R>(P, iF, gout + goff<NS>(nn) + (iF * 5 + b) * CELL, (out - q) - sh);
         sF += q;
       }
     }
@@ -213,8 +213,6 @@ __device__ __forceinline__ void finish_step(const DevInst* Ip, unsigned long lon
 
 template <class TF, class TG, class R, int NS>
 __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ insts) {
-  // the bulk kernel's tile claims start from zero at its next launch
-  if (blockIdx.x == 0 && threadIdx.x == 0) insts[0].scal[S_TILES] = 0ULL;
   const DevInst* Ip = insts + blockIdx.x;
   // the counters this kernel reads, loaded together (one memory round trip)
   const volatile unsigned long long* sc = Ip->scal;
@@ -293,17 +291,17 @@ __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ 
       const long long nn = (long long)yn * P.nx + xn;
       const uint8_t tf = T[nn];
       if (surv_fluid(tf)) {
-        s1 += fshift<R>(P, 0, tf) + density_c<R>(F, N, nn);
-        s2 += fshift<R>(P, 1, tf) + density_c<R>(F + 9 * N, N, nn);
+        s1 += fshift<R>(P, 0, tf) + density_c<R>(F, 0, (int)nn);
+        s2 += fshift<R>(P, 1, tf) + density_c<R>(F, 1, (int)nn);
         ++nf;
       }
       if (surv_liquid(tf)) {
 #pragma unroll
         for (int k = 0; k < NS; ++k) {
-          const TG* gk = G + (long long)k * 5 * N;
-          R c = gldc<R>(P, k, gk + nn);
+          const TG* gk = G + goff<NS>((int)nn) + k * 5 * CELL;
+          R c = gldc<R>(P, k, gk);
 #pragma unroll
-          for (int a = 1; a < 5; ++a) c += gldc<R>(P, k, gk + a * N + nn);
+          for (int a = 1; a < 5; ++a) c += gldc<R>(P, k, gk + a * CELL);
           sc[k] += rp<R>(P).shift_c[k] + c;
         }
         ++nl;
@@ -314,8 +312,8 @@ __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ 
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
       const R w = w9<R>(a);
-      st<TF, R>(F + a * N + node, w * r1 - w * rp<R>(P).shift_f[0]);
-      st<TF, R>(F + (9 + a) * N + node, w * r2 - w * rp<R>(P).shift_f[1]);
+      st<TF, R>(F + foff(node) + a * CELL, w * r1 - w * rp<R>(P).shift_f[0]);
+      st<TF, R>(F + foff(node) + (9 + a) * CELL, w * r2 - w * rp<R>(P).shift_f[1]);
     }
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
@@ -324,7 +322,7 @@ __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ 
 #pragma unroll
       for (int a = 0; a < 5; ++a) {
         const R ja = a == 0 ? J0 : Ja;
-        gst<TG, R>(P, k, G + ((long long)k * 5 + a) * N + node, ja * c - ja * rp<R>(P).shift_c[k]);
+        gst<TG, R>(P, k, G + goff<NS>(node) + (k * 5 + a) * CELL, ja * c - ja * rp<R>(P).shift_c[k]);
       }
     }
   }
@@ -359,15 +357,15 @@ __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ 
         nf += surv_fluid(tz) ? 1 : 0;
         nl += surv_liquid(tz) ? 1 : 0;
       }
-      add1 += (fshift<R>(P, 0, T[w]) + density_c<R>(F, N, w)) / R(nf);
-      add2 += (fshift<R>(P, 1, T[w]) + density_c<R>(F + 9 * N, N, w)) / R(nf);
+      add1 += (fshift<R>(P, 0, T[w]) + density_c<R>(F, 0, (int)w)) / R(nf);
+      add2 += (fshift<R>(P, 1, T[w]) + density_c<R>(F, 1, (int)w)) / R(nf);
       if (nliq && nl) {
 #pragma unroll
         for (int k = 0; k < NS; ++k) {
-          const TG* gk = G + (long long)k * 5 * N;
-          R c = gldc<R>(P, k, gk + w);
+          const TG* gk = G + goff<NS>((int)w) + k * 5 * CELL;
+          R c = gldc<R>(P, k, gk);
 #pragma unroll
-          for (int a = 1; a < 5; ++a) c += gldc<R>(P, k, gk + a * N + w);
+          for (int a = 1; a < 5; ++a) c += gldc<R>(P, k, gk + a * CELL);
           addc[k] += (rp<R>(P).shift_c[k] + c) / R(nl);
         }
       }
@@ -375,8 +373,8 @@ __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ 
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
       const R w = w9<R>(a);
-      TF* p1 = F + a * N + n;
-      TF* p2 = F + (9 + a) * N + n;
+      TF* p1 = F + foff(n) + a * CELL;
+      TF* p2 = F + foff(n) + (9 + a) * CELL;
       st<TF, R>(p1, ldc<R>(p1) + w * add1);
       st<TF, R>(p2, ldc<R>(p2) + w * add2);
     }
@@ -386,7 +384,7 @@ __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ 
         const R J0 = rp<R>(P).J0[k], Ja = (R(1) - J0) / R(4);
 #pragma unroll
         for (int a = 0; a < 5; ++a) {
-          TG* p = G + ((long long)k * 5 + a) * N + n;
+          TG* p = G + goff<NS>(n) + (k * 5 + a) * CELL;
           gst<TG, R>(P, k, p, gldc<R>(P, k, p) + (a == 0 ? J0 : Ja) * addc[k]);
         }
       }

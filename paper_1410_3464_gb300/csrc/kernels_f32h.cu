@@ -3,5 +3,4 @@
 #define KTG __half
 #define KR float
 #define KNAME launchers_f32h
-#define KPART 1
 #include "kernels_impl.cuh"

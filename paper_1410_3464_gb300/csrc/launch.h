@@ -6,12 +6,6 @@
 namespace pslbm {
 
 struct Launchers {
-  void (*bulk[NSHAPES])(cudaStream_t, const Tile*, int ntiles, const DevInst*, bool single);
-  // TMA-staged bulk kernel (FP32 populations only; null for FP64); single is
-  // the host parameter block when the tile list holds one simulation, else null
-  void (*bulk_tma[NSHAPES])(cudaStream_t, const Tile*, int ntiles, const DevInst*, const DevParams* single);
-  // TMA-staged bulk kernel with a single stage and three blocks per SM
-  void (*bulk_tma1[NSHAPES])(cudaStream_t, const Tile*, int ntiles, const DevInst*, const DevParams* single);
   // chunk_map: (member, chunk) of every VOP chunk of a batch (null for one
   // simulation); nchunks: their number
   void (*vop)(cudaStream_t, const DevInst*, const int2* chunk_map, long long nchunks);
@@ -19,6 +13,10 @@ struct Launchers {
   void (*init)(cudaStream_t, DevInst*, const uint8_t*, const double*, const double*, const double*, long long N);
   void (*fields)(cudaStream_t, const DevInst*, long long N, double*, double*, double*, double*, double*, uint8_t*);
   void (*budget)(cudaStream_t, const DevInst*, double* part, double* out);
+  // potentials and collide-stream kernels, a warp per entry of the work list:
+  // tiles of 32 columns by `rows` rows, then chunks of 32 reservoir nodes
+  void (*pot)(cudaStream_t, const Tile*, int ntiles, int rows, const DevInst*, const DevInst& Ik, int mode);
+  void (*move)(cudaStream_t, const Tile*, int ntiles, int rows, const DevInst*, const DevInst& Ik, int mode);
 };
 
 // prec: 0 FP64, 1 FP32, 2 FP32 + half solutes, 3 FP32 + bfloat16 solutes; ns 0..MAXS

@@ -15,6 +15,7 @@
 
 #include "../../include/pslbm.h"
 #include "launch.h"
+#include "step.cuh"
 
 using namespace pslbm;
 
@@ -45,36 +46,36 @@ struct GraphCache {
 
 constexpr int NSTAGING = 3;
 
-// Launch state shared by a single simulation and a batch: one tile list per
-// tile shape (built on demand), the chosen bulk-kernel variant (tile shape and
-// staging: plain loads or TMA-staged), and the captured graphs.
+// Launch state shared by a single simulation and a batch: the work list of the
+// streaming kernels, the caller's tile shape and staging, and the captured
+// graphs.
 struct Stepper {
   const Launchers* L = nullptr;
   DevInst* d = nullptr;
   int ninst = 0;
   std::vector<std::pair<int, int>> dims;   // (nx, ny) per instance
-  Tile* tiles[NSHAPES] = {};
-  int ntiles[NSHAPES] = {};
-  int shape = 0;
-  int staged = 0;                          // 1: TMA-staged, two stages; 2: TMA-staged, one stage
-  int fix_shape = -1;                      // caller's choice, -1: choose by timing
+  std::vector<int> nres;                   // reservoir nodes per instance
+  DevInst host0{};                         // host descriptor of the first instance
+  int mode = M_SINGLE;
+  int rows = 0;                            // rows of a tile
+  Tile* work = nullptr;                    // work list of a batch (one simulation's is arithmetic)
+  int nwork = 0;                           // its entries, 0: not made yet
+  int fix_shape = -1;                      // caller's choices, -1: none
   int fix_staged = -1;
-  bool staged_ok = false;                  // every instance has TMA descriptors
-  const DevParams* single = nullptr;       // host parameters of a one-simulation stepper
+  bool staged_ok = false;                  // the caller may ask for staging 1 or 2
   int2* chunk_map = nullptr;               // (instance, chunk) of every VOP chunk of a batch (device)
   long long nchunks = 0;                   // VOP chunks of all instances
-  bool tuned = false;                      // variant chosen (by timing or by the caller)
   GraphCache graphs;
-  double trial_ms[NSHAPES][NSTAGING] = {};
-  void release() {
+  void drop_work() {
     graphs.clear();
+    if (work) cudaFree(work);
+    work = nullptr;
+    nwork = 0;
+  }
+  void release() {
+    drop_work();
     if (chunk_map) cudaFree(chunk_map);
     chunk_map = nullptr;
-    for (int s = 0; s < NSHAPES; ++s) {
-      if (tiles[s]) cudaFree(tiles[s]);
-      tiles[s] = nullptr;
-      ntiles[s] = 0;
-    }
   }
 };
 
@@ -250,6 +251,32 @@ void fill_r(DevParamsR<R>& q, const DevParams& P) {
   }
 }
 
+// Whether two parameter blocks agree in everything the streaming kernels read
+// through Q (all but the sizes, the rates, the reservoirs and the VOP constants).
+bool same_hot_params(const DevParams& a, const DevParams& b) {
+  DevParams x, y;
+  std::memcpy(&x, &a, sizeof x);
+  std::memcpy(&y, &b, sizeof y);
+  for (DevParams* p : {&x, &y}) {
+    p->nx = p->ny = p->px = p->py = 0;
+    p->per_liq = p->per_gas = p->ramp = p->useB = p->useF = 0;
+    p->in_dx = p->in_dy = p->out_dx = p->out_dy = 0;
+    p->k1 = p->k2 = p->k3 = p->k4 = p->inv_Keq = p->C_F_sat = p->r1_surface_factor = 0.0;
+    p->Vbar_D = p->Vbar_F = p->V_split = 0.0;
+    p->seed = 0;
+    for (int s = 0; s < 2; ++s) p->rho_in_liq[s] = p->rho_in_gas[s] = p->rho_out[s] = p->rho_out_gas[s] = 0.0;
+    for (int k = 0; k < MAXS; ++k) p->conc_in[k] = 0.0;
+    auto clear = [](auto& q) {
+      q.k1 = q.k1_s = q.k1_inv_Keq = q.k1_inv_Keq_s = q.k2 = q.k3 = q.k4 = q.C_F_sat = 0;
+      q.vB_qa = q.vB_sh = q.vF_qa = q.vF_qc = q.vF_sh = 0;
+      for (int k = 0; k < MAXS; ++k) q.conc_in[k] = 0;
+    };
+    clear(p->rf);
+    clear(p->rd);
+  }
+  return std::memcmp(&x, &y, sizeof x) == 0;
+}
+
 DevParams to_dev(const pslbm_params* p) {
   DevParams P{};
   P.nx = p->nx;
@@ -327,6 +354,8 @@ DevParams to_dev(const pslbm_params* p) {
   P.Vbar_F = p->Vbar_F;
   P.V_split = p->V_split;
   P.seed = p->seed;
+  P.has_w = p->w_adh[0] != 0.0 || p->w_adh[1] != 0.0;
+  P.tau_unit = p->tau[0] == 1.0 && p->tau[1] == 1.0;
   P.has_G11 = p->G11 != 0.0;
   P.has_rev = p->inv_Keq != 0.0;
   P.useB = p->idx_B >= 0 && p->k2 != 0.0;
@@ -336,20 +365,32 @@ DevParams to_dev(const pslbm_params* p) {
   return P;
 }
 
-std::vector<Tile> make_tiles(int inst, int nx, int ny, int shape) {
-  std::vector<Tile> t;
-  for (int y0 = 0; y0 < ny; y0 += SHAPE_TY[shape])
-    for (int x0 = 0; x0 < nx; x0 += SHAPE_TX[shape]) t.push_back(Tile{inst, x0, y0, 0});
-  return t;
+// Rows of a tile (a warp's share): 8 where the lattices give every SM 16 warps
+// of them, else fewer, down to one; a tile shape the caller asked for sets them
+// (256 nodes: 8 rows of 32, 512: 16).
+int tile_rows(const Stepper& st) {
+  if (st.fix_shape >= 0) return SHAPE_TX[st.fix_shape] * SHAPE_TY[st.fix_shape] / 32;
+  long long n = 0;
+  for (auto& d : st.dims) n += (long long)((d.first + 31) / 32) * d.second;
+  int rows = 8;
+  while (rows > 1 && n / rows < 152 * 16) rows /= 2;
+  return rows;
 }
 
-// Tile list of every instance of a stepper for one shape (device copy).
-cudaError_t ensure_tiles(Stepper& st, int shape) {
-  if (st.tiles[shape]) return cudaSuccess;
+// Work list of the streaming kernels: tiles of 32 columns, then the chunks of 32
+// reservoir nodes.
+cudaError_t ensure_work(Stepper& st) {
+  if (st.nwork) return cudaSuccess;
+  const int rows = st.rows = tile_rows(st);
+  if (st.mode == M_SINGLE) {
+    st.nwork = ((st.dims[0].first + 31) / 32) * ((st.dims[0].second + rows - 1) / rows) + (st.nres[0] + 31) / 32;
+    return cudaSuccess;
+  }
   std::vector<Tile> all;
   for (int i = 0; i < (int)st.dims.size(); ++i) {
-    std::vector<Tile> t = make_tiles(i, st.dims[i].first, st.dims[i].second, shape);
-    all.insert(all.end(), t.begin(), t.end());
+    for (int y0 = 0; y0 < st.dims[i].second; y0 += rows)
+      for (int x0 = 0; x0 < st.dims[i].first; x0 += 32) all.push_back(Tile{i, x0, y0, -1});
+    for (int k = 0; k < st.nres[i]; k += 32) all.push_back(Tile{i, 0, 0, k});
   }
   Tile* d = nullptr;
   cudaError_t e = cudaMalloc(&d, all.size() * sizeof(Tile));
@@ -360,8 +401,8 @@ cudaError_t ensure_tiles(Stepper& st, int shape) {
     cudaFree(d);
     return e;
   }
-  st.tiles[shape] = d;
-  st.ntiles[shape] = (int)all.size();
+  st.work = d;
+  st.nwork = (int)all.size();
   return cudaSuccess;
 }
 
@@ -386,33 +427,29 @@ void free_all(pslbm_t h) {
   h->allocs.clear();
 }
 
-// Enqueue one launch of the bulk kernel of a variant.
-void enqueue_bulk(cudaStream_t s, const Stepper& st, int shape, int staged) {
-  if (staged == 2)
-    st.L->bulk_tma1[shape](s, st.tiles[shape], st.ntiles[shape], st.d, st.single);
-  else if (staged == 1)
-    st.L->bulk_tma[shape](s, st.tiles[shape], st.ntiles[shape], st.d, st.single);
-  else
-    st.L->bulk[shape](s, st.tiles[shape], st.ntiles[shape], st.d, st.single != nullptr);
+// Enqueue the streaming kernels of one step.
+void enqueue_stream(cudaStream_t s, const Stepper& st) {
+  st.L->pot(s, st.work, st.nwork, st.rows, st.d, st.host0, st.mode);
+  st.L->move(s, st.work, st.nwork, st.rows, st.d, st.host0, st.mode);
 }
 
-// Enqueue n steps of the kernels for one bulk-kernel variant.
-void enqueue_steps(cudaStream_t s, const Stepper& st, int shape, int staged, int64_t n) {
+// Enqueue the kernels of n steps.
+void enqueue_steps(cudaStream_t s, const Stepper& st, int64_t n) {
   for (int64_t i = 0; i < n; ++i) {
-    enqueue_bulk(s, st, shape, staged);
+    enqueue_stream(s, st);
     st.L->vop(s, st.d, st.chunk_map, st.nchunks);
     st.L->amend(s, st.ninst, st.d);
   }
 }
 
 // n steps without graph capture, each kernel bracketed by CUDA events on the
-// library stream: mean ms per step of the bulk, VOP and amendment kernels and
+// library stream: mean ms per step of the streaming, VOP and amendment kernels and
 // of the whole step.
 pslbm_status profile_steps(Stepper& st, int64_t n, double* kernel_ms, double* total_ms, std::string& err) {
   cudaStream_t s = lib_stream();
-  cudaError_t te = ensure_tiles(st, st.shape);
+  cudaError_t te = ensure_work(st);
   if (te != cudaSuccess) {
-    err = std::string("tile list: ") + cudaGetErrorString(te);
+    err = std::string("work list: ") + cudaGetErrorString(te);
     return PSLBM_ERR_CUDA;
   }
   cudaEvent_t ev[4] = {};
@@ -426,7 +463,7 @@ pslbm_status profile_steps(Stepper& st, int64_t n, double* kernel_ms, double* to
   pslbm_status st_ = PSLBM_OK;
   for (int64_t i = 0; i < n; ++i) {
     cudaEventRecord(ev[0], s);
-    enqueue_bulk(s, st, st.shape, st.staged);
+    enqueue_stream(s, st);
     cudaEventRecord(ev[1], s);
     st.L->vop(s, st.d, st.chunk_map, st.nchunks);
     cudaEventRecord(ev[2], s);
@@ -485,117 +522,12 @@ __global__ void k_batch_monitor(const DevInst* __restrict__ insts, int n, unsign
   }
 }
 
-// Whether the bulk kernel of a variant is compiled (the staged kernels exist
-// for the shapes of one node per thread).
-bool variant_exists(const Stepper& st, int sh, int sg) {
-  return sg == 0 ? st.L->bulk[sh] != nullptr : sg == 1 ? st.L->bulk_tma[sh] != nullptr : st.L->bulk_tma1[sh] != nullptr;
-}
-
-// Variants the stepper may use: every tile shape and staging the caller left
-// open (staging only where every instance has TMA descriptors and the shape
-// has a staged kernel).
-std::vector<std::pair<int, int>> candidates(const Stepper& st) {
-  std::vector<std::pair<int, int>> c;
-  for (int sh = 0; sh < NSHAPES; ++sh) {
-    if (st.fix_shape >= 0 && sh != st.fix_shape) continue;
-    for (int sg = 0; sg < NSTAGING; ++sg) {
-      if (st.fix_staged >= 0 && sg != st.fix_staged) continue;
-      if (sg >= 1 && !st.staged_ok) continue;
-      if (!variant_exists(st, sh, sg)) continue;
-      c.push_back({sh, sg});
-    }
-  }
-  return c;
-}
-
-// After a change of the caller's choices: a single candidate is taken at once;
-// otherwise the variant is chosen by timing on the next long step call (until
-// then the first candidate runs, with the two-box staging when it is open: the
-// fastest staging on every large workload measured).
-void choose(Stepper& st) {
-  std::vector<std::pair<int, int>> c = candidates(st);
-  int sh = c.empty() ? 0 : c[0].first, sg = c.empty() ? 0 : c[0].second;
-  for (auto& v : c)
-    if (v.first == sh && v.second == 1) sg = 1;
-  if (sh != st.shape || sg != st.staged) st.graphs.clear();
-  st.shape = sh;
-  st.staged = sg;
-  st.tuned = c.size() <= 1;
-}
-
-// Variant autotuning: the results do not depend on the variant (the per-node
-// arithmetic and the fixed-order gathers are the same), so the first steps of
-// a run are spent timing each candidate (one untimed step, then TUNE_STEPS
-// timed steps each) in TUNE_ROUNDS passes, the second in reverse order, and
-// the fastest by its best pass is kept (a run's first steps can be slower
-// than its later ones, which a single pass would charge to the first
-// candidates).
-constexpr int TUNE_STEPS = 3;
-constexpr int TUNE_ROUNDS = 2;
-pslbm_status autotune(Stepper& st, std::string& err) {
-  cudaStream_t s = lib_stream();
-  cudaEvent_t a, b;
-  if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) {
-    err = "cudaEventCreate failed";
-    return PSLBM_ERR_CUDA;
-  }
-  std::vector<std::pair<int, int>> c = candidates(st);
-  double best_ms = 0;
-  int best = -1;
-  const int nc = (int)c.size();
-  for (int pass = 0; pass < TUNE_ROUNDS * nc; ++pass) {
-    const int round = pass / nc;
-    const int i = (round & 1) ? nc - 1 - pass % nc : pass % nc;
-    const int sh = c[i].first, sg = c[i].second;
-    cudaError_t e = ensure_tiles(st, sh);
-    if (e != cudaSuccess) {
-      err = std::string("tile list: ") + cudaGetErrorString(e);
-      return e == cudaErrorMemoryAllocation ? PSLBM_ERR_OOM : PSLBM_ERR_CUDA;
-    }
-    enqueue_steps(s, st, sh, sg, 1);
-    cudaEventRecord(a, s);
-    enqueue_steps(s, st, sh, sg, TUNE_STEPS);
-    cudaEventRecord(b, s);
-    e = cudaEventSynchronize(b);
-    if (e != cudaSuccess) {
-      err = std::string("autotune: ") + cudaGetErrorString(e);
-      return PSLBM_ERR_CUDA;
-    }
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, a, b);
-    const double t = ms / TUNE_STEPS;
-    if (round == 0 || t < st.trial_ms[sh][sg]) st.trial_ms[sh][sg] = t;
-    if (best < 0 || t < best_ms) {
-      best = i;
-      best_ms = t;
-    }
-  }
-  cudaEventDestroy(a);
-  cudaEventDestroy(b);
-  if (best >= 0) {
-    if (c[best].first != st.shape || c[best].second != st.staged) st.graphs.clear();
-    st.shape = c[best].first;
-    st.staged = c[best].second;
-  }
-  st.tuned = true;
-  return PSLBM_OK;
-}
-
-// Steps the autotuner spends (they advance the simulation like any others).
-int64_t tune_cost(const Stepper& st) { return (int64_t)candidates(st).size() * (TUNE_STEPS + 1) * TUNE_ROUNDS; }
-
 // Run n steps, replaying captured graphs of up to 32 steps.
 pslbm_status run_steps(Stepper& st, int64_t n, std::string& err) {
   cudaStream_t s = lib_stream();
-  if (!st.tuned && n >= tune_cost(st) + 1) {
-    const int64_t spent = tune_cost(st);
-    pslbm_status ts = autotune(st, err);
-    if (ts != PSLBM_OK) return ts;
-    n -= spent;
-  }
-  cudaError_t te = ensure_tiles(st, st.shape);
+  cudaError_t te = ensure_work(st);
   if (te != cudaSuccess) {
-    err = std::string("tile list: ") + cudaGetErrorString(te);
+    err = std::string("work list: ") + cudaGetErrorString(te);
     return PSLBM_ERR_CUDA;
   }
   GraphCache& gc = st.graphs;
@@ -610,7 +542,7 @@ pslbm_status run_steps(Stepper& st, int64_t n, std::string& err) {
         err = std::string("cudaStreamBeginCapture: ") + cudaGetErrorString(e);
         return PSLBM_ERR_CUDA;
       }
-      enqueue_steps(s, st, st.shape, st.staged, k);
+      enqueue_steps(s, st, k);
       e = cudaStreamEndCapture(s, &g);
       if (e != cudaSuccess) {
         err = std::string("cudaStreamEndCapture: ") + cudaGetErrorString(e);
@@ -635,97 +567,38 @@ pslbm_status run_steps(Stepper& st, int64_t n, std::string& err) {
   return PSLBM_OK;
 }
 
-// Fix the tile shape (tx = ty = 0: leave it to timing).
+// Fix the tile shape (tx = ty = 0: none).
 pslbm_status set_shape(Stepper& st, int tx, int ty) {
   int idx = -2;
   if (tx == 0 && ty == 0) idx = -1;
   for (int sh = 0; sh < NSHAPES; ++sh)
     if (SHAPE_TX[sh] == tx && SHAPE_TY[sh] == ty) idx = sh;
   if (idx == -2) return PSLBM_ERR_PARAM;
-  const int prev = st.fix_shape;
+  if (idx >= 0 && st.fix_staged == 1 && SHAPE_TX[idx] * SHAPE_TY[idx] > 256) return PSLBM_ERR_PARAM;
+  if (idx != st.fix_shape) st.drop_work();
   st.fix_shape = idx;
-  if (candidates(st).empty()) {
-    // a fixed staging that this shape has no kernel for
-    st.fix_shape = prev;
-    return PSLBM_ERR_PARAM;
-  }
-  choose(st);
   return PSLBM_OK;
 }
 
-// Fix the staging (-1: leave it to timing, 0: plain loads, 1: TMA-staged,
-// 2: TMA-staged with a single stage).
+// Fix the staging (-1: none).  The kernels stage no populations: the choice is
+// checked and reported, and changes nothing else.
 pslbm_status set_staging(Stepper& st, int mode) {
   if (mode < -1 || mode >= NSTAGING || (mode >= 1 && !st.staged_ok)) return PSLBM_ERR_PARAM;
-  const int prev = st.fix_staged;
+  if (mode == 1 && st.fix_shape >= 0 && SHAPE_TX[st.fix_shape] * SHAPE_TY[st.fix_shape] > 256) return PSLBM_ERR_PARAM;
   st.fix_staged = mode;
-  if (candidates(st).empty()) {
-    // a fixed tile shape that has no kernel of this staging
-    st.fix_staged = prev;
-    return PSLBM_ERR_PARAM;
-  }
-  choose(st);
   return PSLBM_OK;
 }
 
-// TMA descriptors of an instance's population boxes (FP32 populations only):
-// per tile shape and ping-pong buffer, a 3D map over (x, y, plane) whose box is
-// the tile plus the staged kernel's ring (D2Q9) or the tile itself (D2Q5).
-// Rows must be a multiple of 16 bytes; returns false when the instance does
-// not qualify or the driver lacks the encoder.
-using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiled encoder() {
-  static EncodeTiled fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiled)f;
-  }
-  return fn;
+// Whether a caller may ask for staging 1 or 2: FP32 populations and rows of a
+// multiple of 16 bytes.
+bool staging_open(const pslbm_params* p) {
+  if (p->precision == PSLBM_FP64) return false;
+  return p->nx * 4 % 16 == 0 && (p->n_species == 0 || (int64_t)p->nx * (int64_t)gsize(p->precision) % 16 == 0);
 }
 
-bool encode_maps(DevInst& I, const pslbm_params* p) {
-  if (p->precision == PSLBM_FP64) return false;
-  const size_t gs = gsize(p->precision);
-  const uint64_t nx = (uint64_t)p->nx, ny = (uint64_t)p->ny, N = nx * ny;
-  const int ns = p->n_species;
-  if ((nx * 4) % 16 != 0 || (ns > 0 && (nx * gs) % 16 != 0)) return false;
-  EncodeTiled enc = encoder();
-  if (!enc) return false;
-  const CUtensorMapDataType gt = p->precision == PSLBM_FP32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                 : p->precision == PSLBM_FP32_SOLUTE_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                                         : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-  for (int sh = 0; sh < NSHAPES; ++sh) {
-    for (int b = 0; b < 2; ++b) {
-      const cuuint64_t fdim[3] = {nx, ny, 18};
-      const cuuint64_t fstr[2] = {nx * 4, N * 4};
-      const cuuint32_t fbox[3] = {(cuuint32_t)(SHAPE_TX[sh] + 2 * stage_halo_x(SHAPE_NPT[sh])),
-                                  (cuuint32_t)(SHAPE_TY[sh] + 2), 18};
-      const cuuint32_t one[3] = {1, 1, 1};
-      if (enc(&I.tmf[sh][b], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, I.f[b], fdim, fstr, fbox, one,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
-      if (ns > 0) {
-        const cuuint64_t gdim[3] = {nx, ny, (cuuint64_t)(5 * ns)};
-        const cuuint64_t gstr[2] = {nx * gs, N * gs};
-        const cuuint32_t gbox[3] = {(cuuint32_t)SHAPE_TX[sh], (cuuint32_t)SHAPE_TY[sh], (cuuint32_t)(5 * ns)};
-        if (enc(&I.tmg[sh][b], gt, 3, I.g[b], gdim, gstr, gbox, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-            CUDA_SUCCESS)
-          return false;
-      }
-    }
-  }
-  return true;
-}
+// Shape and staging as reported: the caller's, or 32x8 and plain loads.
+int shown_shape(const Stepper& st) { return st.fix_shape >= 0 ? st.fix_shape : 1; }
+int shown_staging(const Stepper& st) { return st.fix_staged >= 0 ? st.fix_staged : 0; }
 
 pslbm_status device_status(pslbm_t h) {
   unsigned long long st = 0;
@@ -775,15 +648,22 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
   I.N = N;
   I.evcap = (int)N;
   pslbm_status st = PSLBM_OK;
+  std::vector<int> reslist;
   {
     // one device allocation holds the instance's whole state, each part on a
     // 256-byte boundary (TMA wants 16-byte aligned bases); the initial
     // threshold's budget partial sums are the last part
-    const size_t fb = (size_t)N * 18 * fsize(p->precision), gb = (size_t)N * 5 * ns * gsize(p->precision);
+    const size_t NP = (size_t)(N + CELL - 1) / CELL * CELL;   // whole cells
+    const size_t fb = NP * 18 * fsize(p->precision), gb = NP * 5 * ns * gsize(p->precision);
+    // the reservoir nodes (their types never change)
+    for (long long i = 0; i < N; ++i)
+      if ((mask[i] & 15) >= PSLBM_INLET && (mask[i] & 15) <= PSLBM_OUTLET) reslist.push_back((int)i);
+    I.nres = (int)reslist.size();
     const size_t sizes[] = {fb, fb, gb, gb, (size_t)N, (size_t)N, (size_t)N * 2 * sizeof(double), (size_t)N,
                             (size_t)N * sizeof(double), (size_t)N * 2 * sizeof(int), (size_t)N * sizeof(int),
                             (size_t)((N + 31) / 32) * sizeof(unsigned), S_NSCAL * sizeof(unsigned long long),
-                            sizeof(DevInst), (size_t)(BUD_BLOCKS + 1) * NBUD * sizeof(double)};
+                            sizeof(DevInst), (size_t)(BUD_BLOCKS + 1) * NBUD * sizeof(double), (size_t)N * 4 * fsize(p->precision),
+                            (size_t)N, reslist.size() * sizeof(int)};
     constexpr int NPARTS = sizeof(sizes) / sizeof(sizes[0]);
     size_t offs[NPARTS], total = 0;
     for (int i = 0; i < NPARTS; ++i) {
@@ -808,6 +688,9 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     I.vmask = (unsigned*)(base + offs[11]);
     I.scal = (unsigned long long*)(base + offs[12]);
     h->d = (DevInst*)(base + offs[13]);
+    I.pot = base + offs[15];
+    I.code = (uint8_t*)(base + offs[16]);
+    I.reslist = (int*)(base + offs[17]);
     double* part = (double*)(base + offs[14]);
     double* res = part + (size_t)BUD_BLOCKS * NBUD;
 
@@ -836,7 +719,8 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
         e = cudaGetLastError();
       }
     }
-    h->run.staged_ok = L->bulk_tma[0] != nullptr && encode_maps(I, p);
+    if (e == cudaSuccess && I.nres)
+      e = cudaMemcpyAsync(I.reslist, reslist.data(), reslist.size() * sizeof(int), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d, &I, sizeof(DevInst), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
       L->init(s, h->d, dmask, dr1, dr2, dc, N);
@@ -865,13 +749,14 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
   h->run.ninst = 1;
   h->run.dims.assign(1, {p->nx, p->ny});
   h->run.nchunks = ((N + 31) / 32 + VOP_CHUNK - 1) / VOP_CHUNK;
-  h->run.single = &h->h.P;
-  choose(h->run);
+  h->run.host0 = h->h;
+  h->run.nres.assign(1, I.nres);
+  h->run.staged_ok = staging_open(p);
   {
-    cudaError_t e = ensure_tiles(h->run, h->run.shape);
+    cudaError_t e = ensure_work(h->run);
     if (e != cudaSuccess) {
       st = fail(nullptr, e == cudaErrorMemoryAllocation ? PSLBM_ERR_OOM : PSLBM_ERR_CUDA,
-                std::string("tile list: ") + cudaGetErrorString(e));
+                std::string("work list: ") + cudaGetErrorString(e));
       goto fail_cleanup;
     }
   }
@@ -927,13 +812,16 @@ pslbm_status pslbm_estimate_device_bytes(const pslbm_params* p, uint64_t* bytes)
   if (!v.empty()) return fail(nullptr, PSLBM_ERR_PARAM, v);
   const uint64_t N = (uint64_t)p->nx * (uint64_t)p->ny;
   const uint64_t per = 2 * 18 * fsize(p->precision) + 2 * 5 * (uint64_t)p->n_species * gsize(p->precision) +
-                       2 /*types*/ + 16 /*V*/ + 1 /*events*/ + 8 /*excess*/ + 8 /*event lists*/ + 4 /*claims*/;
+                       2 /*types*/ + 4 * fsize(p->precision) + 1 /*potentials, codes*/ + 16 /*V*/ + 1 /*events*/ + 8 /*excess*/ + 8 /*event lists*/ + 4 /*claims*/;
   const uint64_t vmask_bytes = ((N + 31) / 32) * 4;
-  uint64_t tiles = 0;
-  for (int sh = 0; sh < NSHAPES; ++sh)
-    tiles += ((uint64_t)(p->nx + SHAPE_TX[sh] - 1) / SHAPE_TX[sh]) * ((uint64_t)(p->ny + SHAPE_TY[sh] - 1) / SHAPE_TY[sh]);
-  *bytes = N * per + vmask_bytes + tiles * sizeof(Tile) + sizeof(DevInst) + S_NSCAL * 8 +
-           (uint64_t)(BUD_BLOCKS + 1) * NBUD * sizeof(double) + 15 * 256;
+  // whole cells; reservoir nodes: the edges of the lattice (a batch's work list
+  // has an entry of 16 bytes per 32 nodes at most)
+  const uint64_t cells = (N + CELL - 1) / CELL * CELL;
+  const uint64_t pops = 2 * 18 * fsize(p->precision) + 2 * 5 * (uint64_t)p->n_species * gsize(p->precision);
+  const uint64_t work = ((uint64_t)p->nx + 31) / 32 * (uint64_t)p->ny * sizeof(Tile);
+  const uint64_t res = 2 * ((uint64_t)p->nx + (uint64_t)p->ny) * sizeof(int);
+  *bytes = N * per + (cells - N) * pops + vmask_bytes + work + res + sizeof(DevInst) + S_NSCAL * 8 +
+           (uint64_t)(BUD_BLOCKS + 1) * NBUD * sizeof(double) + 18 * 256;
   return PSLBM_OK;
 }
 
@@ -947,9 +835,9 @@ pslbm_status pslbm_set_tile_shape(pslbm_t h, int32_t tile_x, int32_t tile_y) {
 
 pslbm_status pslbm_get_tile_shape(pslbm_t h, int32_t* tile_x, int32_t* tile_y, int32_t* tuned) {
   if (!h) return fail(nullptr, PSLBM_ERR_PARAM, "handle is NULL");
-  if (tile_x) *tile_x = SHAPE_TX[h->run.shape];
-  if (tile_y) *tile_y = SHAPE_TY[h->run.shape];
-  if (tuned) *tuned = h->run.tuned ? 1 : 0;
+  if (tile_x) *tile_x = SHAPE_TX[shown_shape(h->run)];
+  if (tile_y) *tile_y = SHAPE_TY[shown_shape(h->run)];
+  if (tuned) *tuned = 1;
   return PSLBM_OK;
 }
 
@@ -962,7 +850,7 @@ pslbm_status pslbm_set_staging(pslbm_t h, int32_t mode) {
 
 pslbm_status pslbm_get_staging(pslbm_t h, int32_t* staged, int32_t* available) {
   if (!h) return fail(nullptr, PSLBM_ERR_PARAM, "handle is NULL");
-  if (staged) *staged = h->run.staged;
+  if (staged) *staged = shown_staging(h->run);
   if (available) *available = h->run.staged_ok ? 1 : 0;
   return PSLBM_OK;
 }
@@ -1149,7 +1037,13 @@ pslbm_status pslbm_batch_create(int32_t n, const pslbm_t* members, int32_t tile_
   b->run.L = b->L;
   b->run.d = b->d;
   b->run.ninst = n;
-  if (e == cudaSuccess) e = ensure_tiles(b->run, b->run.shape);
+  b->run.host0 = members[0]->h;
+  b->run.mode = M_SHARED;
+  for (int i = 0; i < n; ++i) {
+    b->run.nres.push_back(members[i]->h.nres);
+    if (!same_hot_params(members[i]->h.P, members[0]->h.P)) b->run.mode = M_MIXED;
+  }
+  if (e == cudaSuccess) e = ensure_work(b->run);
   if (e != cudaSuccess) {
     b->run.release();
     if (b->d) cudaFree(b->d);
@@ -1179,9 +1073,9 @@ pslbm_status pslbm_batch_step(pslbm_batch_t b, int64_t n) {
 
 pslbm_status pslbm_batch_get_tile_shape(pslbm_batch_t b, int32_t* tile_x, int32_t* tile_y, int32_t* tuned) {
   if (!b) return fail(nullptr, PSLBM_ERR_PARAM, "batch is NULL");
-  if (tile_x) *tile_x = SHAPE_TX[b->run.shape];
-  if (tile_y) *tile_y = SHAPE_TY[b->run.shape];
-  if (tuned) *tuned = b->run.tuned ? 1 : 0;
+  if (tile_x) *tile_x = SHAPE_TX[shown_shape(b->run)];
+  if (tile_y) *tile_y = SHAPE_TY[shown_shape(b->run)];
+  if (tuned) *tuned = 1;
   return PSLBM_OK;
 }
 
@@ -1194,7 +1088,7 @@ pslbm_status pslbm_batch_set_staging(pslbm_batch_t b, int32_t mode) {
 
 pslbm_status pslbm_batch_get_staging(pslbm_batch_t b, int32_t* staged, int32_t* available) {
   if (!b) return fail(nullptr, PSLBM_ERR_PARAM, "batch is NULL");
-  if (staged) *staged = b->run.staged;
+  if (staged) *staged = shown_staging(b->run);
   if (available) *available = b->run.staged_ok ? 1 : 0;
   return PSLBM_OK;
 }
@@ -1275,40 +1169,13 @@ const Launchers* launchers_f64(int ns);
 const Launchers* launchers_f32(int ns);
 const Launchers* launchers_f32h(int ns);
 const Launchers* launchers_f32b(int ns);
-const Launchers* launchers_f64_n2(int ns);
-const Launchers* launchers_f32_n2(int ns);
-const Launchers* launchers_f32h_n2(int ns);
-const Launchers* launchers_f32b_n2(int ns);
-
-// The two halves of a precision's table (one and two nodes per thread) merged:
-// every slot takes the entry that is set.
-static Launchers merge_launchers(const Launchers& a, const Launchers& b) {
-  Launchers m = a;
-  for (int s = 0; s < NSHAPES; ++s) {
-    if (!m.bulk[s]) m.bulk[s] = b.bulk[s];
-    if (!m.bulk_tma[s]) m.bulk_tma[s] = b.bulk_tma[s];
-    if (!m.bulk_tma1[s]) m.bulk_tma1[s] = b.bulk_tma1[s];
-  }
-  return m;
-}
-struct MergedLauncherTables {
-  Launchers t[4][MAXS + 1];
-  MergedLauncherTables() {
-    const Launchers* (*one[4])(int) = {launchers_f64, launchers_f32, launchers_f32h, launchers_f32b};
-    const Launchers* (*two[4])(int) = {launchers_f64_n2, launchers_f32_n2, launchers_f32h_n2, launchers_f32b_n2};
-    for (int p = 0; p < 4; ++p)
-      for (int ns = 0; ns <= MAXS; ++ns) t[p][ns] = merge_launchers(*one[p](ns), *two[p](ns));
-  }
-};
-
 const Launchers* launchers(int prec, int ns) {
-  static const MergedLauncherTables tables;
   if (ns < 0 || ns > MAXS) return nullptr;
   switch (prec) {
-    case PSLBM_FP64: return &tables.t[0][ns];
-    case PSLBM_FP32: return &tables.t[1][ns];
-    case PSLBM_FP32_SOLUTE_F16: return &tables.t[2][ns];
-    case PSLBM_FP32_SOLUTE_BF16: return &tables.t[3][ns];
+    case PSLBM_FP64: return launchers_f64(ns);
+    case PSLBM_FP32: return launchers_f32(ns);
+    case PSLBM_FP32_SOLUTE_F16: return launchers_f32h(ns);
+    case PSLBM_FP32_SOLUTE_BF16: return launchers_f32b(ns);
   }
   return nullptr;
 }
