@@ -201,13 +201,13 @@ pslbm_status pslbm_set_step_limit(pslbm_t h, int64_t limit);
  * the read-back scratch of pslbm_read_fields). */
 pslbm_status pslbm_estimate_device_bytes(const pslbm_params* p, uint64_t* bytes);
 
-/* Nodes of a warp's tile of the streaming kernels: 16x16 or 32x8 (256 nodes,
- * taken as 32 columns by 8 rows), 16x32 or 32x16 (512 nodes, 32 columns by 16
- * rows).  (0, 0), the default, takes 32x8 and fewer rows on lattices too small
- * to occupy the device.  The results do not depend on the shape.  get reports
- * the shape asked for, or 32x8; tuned is always 1 (nothing is left to timing).
- * PSLBM_ERR_PARAM for another shape, or for a 512-node shape while staging 1
- * is fixed (the handle is left as it was). */
+/* Nodes a warp of the streaming kernels works through: 16x16 or 32x8 (256 nodes
+ * of the lattice: four turns of 32 fluid nodes) or 16x32 or 32x16 (512: eight
+ * turns).  (0, 0), the default, goes by the size of the lattices.  The results
+ * do not depend on the choice.  get reports the shape asked for, or 32x8; tuned
+ * is always 1 (nothing is left to timing).  PSLBM_ERR_PARAM for another shape,
+ * or for a 512-node shape while staging 1 is fixed (the handle is left as it
+ * was). */
 pslbm_status pslbm_set_tile_shape(pslbm_t h, int32_t tile_x, int32_t tile_y);
 pslbm_status pslbm_get_tile_shape(pslbm_t h, int32_t* tile_x, int32_t* tile_y, int32_t* tuned);
 
@@ -226,7 +226,7 @@ pslbm_status pslbm_get_staging(pslbm_t h, int32_t* staged, int32_t* available);
  * density over fluid nodes found by the last step (the quantity whose half is
  * the next liquid threshold, Section 4.5; the initial maximum before the first
  * step) and the device status bits (1 non-finite density, 2 EOS domain,
- * 4 event-list overflow).  Reads 64 bytes from the
+ * 4 event-list overflow).  Reads 80 bytes from the
  * device and synchronises the library stream; no kernel runs.  Returns the
  * matching error status when a bit is set (sticky, as for pslbm_sync).  Any
  * output pointer may be NULL. */

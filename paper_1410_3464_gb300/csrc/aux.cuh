@@ -1,6 +1,6 @@
 // Initialisation, field read-out and deterministic budget reduction.
 #pragma once
-#include "device.cuh"
+#include "step.cuh"
 
 namespace pslbm {
 
@@ -15,6 +15,7 @@ __global__ void k_init(DevInst* __restrict__ Ip, const uint8_t* __restrict__ mas
     const uint8_t t = mask[node] & T_MASK;
     Ip->type[0][node] = t;
     Ip->type[1][node] = t;
+    Ip->code[node] = (uint8_t)type_code(t);
     TF* F = (TF*)Ip->f[0];
     TG* G = (TG*)Ip->g[0];
     const bool fl = is_fluid(t);

@@ -17,8 +17,6 @@ constexpr uint8_t T_NEW = 0x40;      // flag set by the amendment kernel: solid 
 constexpr uint8_t T_VANISH = 0x80;   // flag: liquid -> solid this step
 
 constexpr int NTHREADS = 256;          // threads per block of the VOP and amendment kernels
-// Interface-bitmap words per warp chunk of the VOP kernel.
-constexpr int VOP_CHUNK = 4;
 // Tile shapes a caller may ask for (nodes per tile: 256 or 512).
 constexpr int NSHAPES = 4;
 constexpr int SHAPE_TX[NSHAPES] = {16, 32, 16, 32};
@@ -34,7 +32,9 @@ enum {
   S_LIMIT = 5,     // step limit: an instance at or past it is frozen (kernels skip it)
   S_THETA = 6,     // this step's liquid threshold (half the previous maximum), FP64 bits
   S_THETAF = 7,    // the same rounded to FP32 (bits in the low word)
-  S_NSCAL = 8
+  S_NFLUID = 8,    // entries of the fluid list
+  S_NFACE = 9,     // entries of the list of minerals facing fluid
+  S_NSCAL = 10
 };
 enum { ST_NONFINITE = 1, ST_EOS = 2, ST_EVOVERFLOW = 4, ST_TIMEOUT = 8 };
 
@@ -67,6 +67,8 @@ struct DevParamsR {
 
 struct DevParams {
   int nx, ny, px, py, ns;
+  int row_shift;                      // node / nx == node * row_mul >> row_shift for every node index
+  unsigned row_mul;
   int iA, iB, iE, iF;
   int per_liq, per_gas, ramp;
   int has_G11, has_rev, useB, useF;   // G11 != 0, inv_Keq != 0, R2 active, R4 active
@@ -110,8 +112,11 @@ struct DevInst {
   double* xs;                 // [N] overflow excess of an event node
   int* evlist;                // [evcap] event node indices
   int* claim;                 // [N] zero except while the amendment kernel runs
-  unsigned* vmask;            // [(N + 31) / 32] bit per node: a mineral a liquid node touched this
-                              // step (set by the bulk kernel, consumed and cleared by k_vop)
+  int* flist;                 // [N] fluid nodes (S_NFLUID entries; an entry may have filled since)
+  int* mlist;                 // [N] minerals with a fluid axis neighbour (S_NFACE entries; an entry may
+                              // have lost its fluid neighbours, or dissolved, since)
+  unsigned* fbits;            // [(N + 31) / 32] bit per node: listed in flist
+  unsigned* mbits;            // [(N + 31) / 32] bit per node: listed in mlist
   unsigned long long* scal;   // [S_NSCAL]
   int* reslist;               // [nres] reservoir nodes
   long long N;
@@ -119,10 +124,10 @@ struct DevInst {
   int nres;
 };
 
-// Work-list entry of a batch: a tile of an instance, or (res >= 0) a chunk of its
-// reservoir nodes.
-struct Tile {
-  int inst, x0, y0, res;
+// A warp's work: 32 entries of an instance's list from entry `first` on, and
+// again every `stride` entries; or (res >= 0) reservoir nodes from entry res on.
+struct Work {
+  int inst, first, stride, res;
 };
 
 // D2Q9 velocity set of Eq. 7 (the D2Q5 set is directions 0-4).
@@ -195,6 +200,11 @@ template <class TG, class R>
 __device__ __forceinline__ void gst(const DevParams& P, int k, TG* p, R v) {
   if constexpr (Is16<TG>::value) st<TG, R>(p, v * rp<R>(P).gs_mul[k]);
   else st<TG, R>(p, v);
+}
+
+// Row of a node index (node / nx without the division).
+__device__ __forceinline__ int node_row(const DevParams& P, int node) {
+  return (int)((unsigned long long)(unsigned)node * P.row_mul >> P.row_shift);
 }
 
 // Neighbour coordinate with periodic wrap; false outside a non-periodic edge.

@@ -23,35 +23,43 @@ namespace pslbm {
 // sum q_B, V_F += Vbar_F sum q_F, and the node dissolves, overflows or changes
 // between D(s) and F(s).
 //
-// The bulk kernel sets a bit for every mineral node a liquid node touched in
-// the step (the only nodes this kernel changes).  Each warp takes a chunk of
-// VOP_CHUNK consecutive words of that bitmap, clears them, and deals the set
-// bits of the chunk out to its lanes in node order (32 nodes per round), so
-// that every lane of a round has a node to update.
+// Only minerals with a liquid axis neighbour change.  The kernel runs over the
+// instance's list of minerals that face fluid, a lane a mineral, and sees from
+// the codes of this step which of the neighbours are liquid.
 template <class TF, class TG, class R, int NS>
 __device__ __forceinline__ void vop_node(const DevInst* Ip, const DevParams& P, int N, int cur,
                                          unsigned long long step, int node) {
-  uint8_t* __restrict__ tnew = Ip->type[cur ^ 1];
   double* __restrict__ V = Ip->V;
-  // independent loads first: own type, volumes, the four neighbour types
-  const uint8_t t = tnew[node] & T_MASK;
+  uint8_t* __restrict__ code = Ip->code;
+  // independent loads first: own code, volumes, the four neighbour codes
+  const int c0 = code[node];
   double VD = V[node], VF = V[N + node];
-  const int x = node % P.nx, y = node / P.nx;
+  const int y = node_row(P, node), x = node - y * P.nx;
   int nbx[4];
 #pragma unroll
   for (int b = 1; b < 5; ++b) {
-    int xn, yn;
-    nbx[b - 1] = nbr(P, x, y, EX(b), EY(b), xn, yn) ? yn * P.nx + xn : -1;
+    int xn = x + EX(b), yn = y + EY(b);
+    bool in = true;
+    if (xn < 0 || xn >= P.nx) {
+      in = P.px != 0;
+      xn = xn < 0 ? P.nx - 1 : 0;
+    }
+    if (yn < 0 || yn >= P.ny) {
+      in = in && P.py != 0;
+      yn = yn < 0 ? P.ny - 1 : 0;
+    }
+    nbx[b - 1] = in ? yn * P.nx + xn : -1;
   }
-  uint8_t tn[4];
+  int cn[4];
 #pragma unroll
-  for (int b = 0; b < 4; ++b) tn[b] = nbx[b] >= 0 ? (tnew[nbx[b]] & T_MASK) : T_WALL;
-  if (!is_mineral(t)) return;
+  for (int b = 0; b < 4; ++b) cn[b] = nbx[b] >= 0 ? code[nbx[b]] : 0;
+  if (!(c0 & C_MIN)) return;      // dissolved since it was listed
+  const uint8_t t = (c0 & C_SOLD) ? T_SOLID_D : T_SOLID_F;
   int nl = 0;
   int dirs[4];
 #pragma unroll
   for (int b = 1; b < 5; ++b) {
-    if (tn[b - 1] != T_LIQUID) nbx[b - 1] = -1;
+    if (!(cn[b - 1] & C_FLIQ)) nbx[b - 1] = -1;
     else dirs[nl++] = b;
   }
   if (nl == 0) return;
@@ -103,26 +111,32 @@ __device__ __forceinline__ void vop_node(const DevInst* Ip, const DevParams& P, 
   VF = VF + P.Vbar_F * double(sF);                        // Eq. 35 (precipitation adds volume)
   if (VD < 0.0) VD = 0.0;
   const double total = VD + VF;
-  int code = EV_NONE;
+  int ev = EV_NONE;
   if (total <= 0.0) {
     VD = 0.0;
     VF = 0.0;
-    code = EV_DISSOLVE;
+    ev = EV_DISSOLVE;
   } else {
-    tnew[node] = VD > 0.0 ? T_SOLID_D : T_SOLID_F;
+    const bool sd = VD > 0.0;
+    if (sd != (t == T_SOLID_D)) {
+      // a solid's type and code change here and in the amendment kernel only, in
+      // both type buffers
+      Ip->type[0][node] = Ip->type[1][node] = sd ? T_SOLID_D : T_SOLID_F;
+      code[node] = (uint8_t)(sd ? C_MIN | C_SOLD : C_MIN);
+    }
     if (total >= P.V_split) {
       const double excess = total - 1.0;
       VF = VF - excess;
       const unsigned long long key = P.seed ^ (step << 40) ^ (unsigned long long)node;
       const int pick = int(splitmix64(key) % (unsigned long long)nl);
-      code = EV_OVERFLOW | (dirs[pick] << 4);
+      ev = EV_OVERFLOW | (dirs[pick] << 4);
       Ip->xs[node] = excess;
     }
   }
   V[node] = VD;
   V[N + node] = VF;
-  if (code != EV_NONE) {
-    Ip->evt[node] = (uint8_t)code;
+  if (ev != EV_NONE) {
+    Ip->evt[node] = (uint8_t)ev;
     const unsigned long long slot = atomicAdd(&Ip->scal[S_NEVENT], 1ULL);
     if (slot < (unsigned long long)Ip->evcap)
       Ip->evlist[slot] = node;
@@ -139,59 +153,29 @@ constexpr int vop_min_blocks() {
   return sizeof(R) == 8 ? 4 : 5;
 }
 
-// chunk_map: (instance, chunk within it) of every chunk of a batch, in
-// instance order, or null for one simulation (instance 0, chunk g); nchunks:
-// the number of chunks.  Warps take chunks with a grid stride, so every
-// member's chunks are spread over the whole grid.
+// A warp per work entry: work[w] of a batch, or the w-th 32 entries of the only
+// instance's list; both again every `stride` entries as far as the list goes.
 template <class TF, class TG, class R, int NS>
 __global__ void __launch_bounds__(NTHREADS, vop_min_blocks<R>())
-    k_vop(const DevInst* __restrict__ insts, const int2* __restrict__ chunk_map, long long nchunks) {
-  const unsigned FULL = 0xffffffffu;
+    k_vop(const DevInst* __restrict__ insts, const Work* __restrict__ work, int nwork) {
   const int lane = threadIdx.x & 31;
-  const long long c0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const long long cs = (gridDim.x * (long long)blockDim.x) >> 5;
-  for (long long g = c0; g < nchunks; g += cs) {
-    const int2 ic = chunk_map ? chunk_map[g] : make_int2(0, (int)g);
-    const DevInst* Ip = insts + ic.x;
-    const int c = ic.y;
-    const unsigned long long step = Ip->scal[S_STEP];
-    if (step >= Ip->scal[S_LIMIT]) continue;   // frozen instance
-    const int N = (int)Ip->N;
-    const int nw = (N + 31) >> 5;
-    const int cur = int(step & 1ULL);
-    unsigned* vmask = Ip->vmask;
-    // lane j < VOP_CHUNK holds word c VOP_CHUNK + j, and the number of set
-    // bits before it in the chunk
-    const int wj = c * VOP_CHUNK + lane;
-    const unsigned m = (lane < VOP_CHUNK && wj < nw) ? vmask[wj] : 0u;
-    if (m) vmask[wj] = 0u;
-    const int cnt = __popc(m);
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < VOP_CHUNK; o <<= 1) {
-      const int v = __shfl_up_sync(FULL, incl, o);
-      if (lane >= o) incl += v;
-    }
-    const int total = __shfl_sync(FULL, incl, VOP_CHUNK - 1);
-    const int excl = incl - cnt;
-    for (int r = 0; r < total; r += 32) {
-      // the k-th set bit of the chunk: its word j and its rank within it
-      const int k = r + lane;
-      int node = -1;
-#pragma unroll
-      for (int j = 0; j < VOP_CHUNK; ++j) {
-        const int ej = __shfl_sync(FULL, excl, j);
-        const int nj = __shfl_sync(FULL, cnt, j);
-        const unsigned mj = __shfl_sync(FULL, m, j);
-        if (k >= ej && k < ej + nj) {
-          unsigned mm = mj;
-          for (int i = k - ej; i > 0; --i) mm &= mm - 1u;   // drop the lower set bits
-          node = (c * VOP_CHUNK + j) * 32 + (__ffs(mm) - 1);
-        }
-      }
-      if (node >= 0) vop_node<TF, TG, R, NS>(Ip, Ip->P, N, cur, step, node);
-    }
-  }
+  const int w = (blockIdx.x * (int)blockDim.x + threadIdx.x) >> 5;
+  if (w >= nwork) return;
+  const Work wk = work ? work[w] : Work{0, w * 32, nwork * 32, -1};
+  const DevInst* Ip = insts + wk.inst;
+  const unsigned long long step = Ip->scal[S_STEP];
+  if (step >= Ip->scal[S_LIMIT]) return;   // frozen instance
+  const int n = (int)Ip->scal[S_NFACE];
+  for (int first = wk.first; first < n; first += wk.stride)
+    if (first + lane < n)
+      vop_node<TF, TG, R, NS>(Ip, Ip->P, (int)Ip->N, int(step & 1ULL), step, Ip->mlist[first + lane]);
+}
+
+// Append a node to a list unless it is listed (bits).
+__device__ __forceinline__ void list_node(unsigned* bits, int* list, unsigned long long* count, int node) {
+  const unsigned bit = 1u << (node & 31);
+  if (atomicOr(&bits[node >> 5], bit) & bit) return;
+  list[(int)atomicAdd(count, 1ULL)] = node;
 }
 
 __device__ __forceinline__ bool surv_fluid(uint8_t tf) { return (tf & (T_NEW | T_VANISH)) == 0 && is_fluid(tf & T_MASK); }
@@ -392,7 +376,34 @@ __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ 
   }
   __syncthreads();
 
-  // phase 4: clear the scratch state used by this step
+  // phase 4: lists, and the solids' types (both buffers) and codes
+  for (int i = threadIdx.x; i < nev; i += blockDim.x) {
+    const int node = Ip->evlist[i];
+    if ((Ip->evt[node] & 15) != EV_DISSOLVE) continue;
+    const int x = node % P.nx, y = node / P.nx;
+    list_node(Ip->fbits, Ip->flist, Ip->scal + S_NFLUID, node);
+#pragma unroll
+    for (int b = 1; b < 5; ++b) {
+      int xn, yn;
+      if (nbr(P, x, y, EX(b), EY(b), xn, yn) && is_mineral(T[yn * P.nx + xn] & T_MASK))
+        list_node(Ip->mbits, Ip->mlist, Ip->scal + S_NFACE, yn * P.nx + xn);
+    }
+  }
+  for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+    const int v = vlist[i];
+    list_node(Ip->mbits, Ip->mlist, Ip->scal + S_NFACE, v);
+    Ip->code[v] = (uint8_t)C_MIN;
+    Ip->type[cur ^ 1][v] = T_SOLID_F;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nv; i += blockDim.x) T[vlist[i]] = T_SOLID_F;
+  for (int i = threadIdx.x; i < nev; i += blockDim.x) {
+    const int node = Ip->evlist[i];
+    if ((Ip->evt[node] & 15) == EV_DISSOLVE) T[node] = T_LIQUID;
+  }
+  __syncthreads();
+
+  // phase 5: clear the scratch state used by this step
   for (int i = threadIdx.x; i < nv * 4; i += blockDim.x) {
     const int v = vlist[i >> 2];
     int xr, yr;

@@ -9,39 +9,29 @@
 namespace pslbm {
 namespace {
 
-// Streaming kernels over ntiles warps; Ik: the descriptor of a single simulation
+// Streaming kernels over nwork warps; Ik: the descriptor of a single simulation
 // (mode M_SINGLE), or of a batch's first member (M_SHARED: all members have its
 // hot parameters).
 template <int NS>
-void pot_l(cudaStream_t s, const Tile* tiles, int ntiles, int rows, const DevInst* insts, const DevInst& Ik, int mode) {
-  const int blocks = (ntiles + ST_WARPS - 1) / ST_WARPS;
-  if (mode == M_SINGLE) k_pot<KTF, KR, M_SINGLE><<<blocks, ST_THREADS, 0, s>>>(tiles, ntiles, rows, insts, Ik);
-  else if (mode == M_SHARED) k_pot<KTF, KR, M_SHARED><<<blocks, ST_THREADS, 0, s>>>(tiles, ntiles, rows, insts, Ik);
-  else k_pot<KTF, KR, M_MIXED><<<blocks, ST_THREADS, 0, s>>>(tiles, ntiles, rows, insts, Ik);
+void pot_l(cudaStream_t s, const Work* work, int nwork, int nstream, const DevInst* insts, const DevInst& Ik, int mode) {
+  if (nwork <= 0) return;
+  const int blocks = (nwork + ST_WARPS - 1) / ST_WARPS;
+  if (mode == M_SINGLE) k_pot<KTF, KR, M_SINGLE><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
+  else if (mode == M_SHARED) k_pot<KTF, KR, M_SHARED><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
+  else k_pot<KTF, KR, M_MIXED><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
 }
 template <int NS>
-void move_l(cudaStream_t s, const Tile* tiles, int ntiles, int rows, const DevInst* insts, const DevInst& Ik, int mode) {
-  const int blocks = (ntiles + ST_WARPS - 1) / ST_WARPS;
-  if (mode == M_SINGLE) k_move<KTF, KTG, KR, NS, M_SINGLE><<<blocks, ST_THREADS, 0, s>>>(tiles, ntiles, rows, insts, Ik);
-  else if (mode == M_SHARED) k_move<KTF, KTG, KR, NS, M_SHARED><<<blocks, ST_THREADS, 0, s>>>(tiles, ntiles, rows, insts, Ik);
-  else k_move<KTF, KTG, KR, NS, M_MIXED><<<blocks, ST_THREADS, 0, s>>>(tiles, ntiles, rows, insts, Ik);
+void move_l(cudaStream_t s, const Work* work, int nwork, int nstream, const DevInst* insts, const DevInst& Ik, int mode) {
+  if (nwork <= 0) return;
+  const int blocks = (nwork + ST_WARPS - 1) / ST_WARPS;
+  if (mode == M_SINGLE) k_move<KTF, KTG, KR, NS, M_SINGLE><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
+  else if (mode == M_SHARED) k_move<KTF, KTG, KR, NS, M_SHARED><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
+  else k_move<KTF, KTG, KR, NS, M_MIXED><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
 }
-// Grid over the chunks of VOP_CHUNK interface-bitmap words of all members
-// (one chunk per warp), capped at one wave of resident blocks (warps then
-// stride).
 template <int NS>
-void vop_l(cudaStream_t s, const DevInst* insts, const int2* chunk_map, long long nchunks) {
-  if (nchunks <= 0) return;
-  static int cap = 0;
-  if (cap == 0) {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_vop<KTF, KTG, KR, NS>, NTHREADS, 0);
-    cap = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
-  }
-  const long long need = (nchunks * 32 + NTHREADS - 1) / NTHREADS;
-  k_vop<KTF, KTG, KR, NS><<<int(need < cap ? need : cap), NTHREADS, 0, s>>>(insts, chunk_map, nchunks);
+void vop_l(cudaStream_t s, const DevInst* insts, const Work* work, int nwork) {
+  if (nwork <= 0) return;
+  k_vop<KTF, KTG, KR, NS><<<(nwork + NTHREADS / 32 - 1) / (NTHREADS / 32), NTHREADS, 0, s>>>(insts, work, nwork);
 }
 template <int NS>
 void amend_l(cudaStream_t s, int ninst, const DevInst* insts) {

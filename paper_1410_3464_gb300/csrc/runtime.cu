@@ -54,17 +54,15 @@ struct Stepper {
   DevInst* d = nullptr;
   int ninst = 0;
   std::vector<std::pair<int, int>> dims;   // (nx, ny) per instance
-  std::vector<int> nres;                   // reservoir nodes per instance
+  std::vector<int> nfluid, nface, nres;    // listed nodes and reservoirs per instance, as created
   DevInst host0{};                         // host descriptor of the first instance
   int mode = M_SINGLE;
-  int rows = 0;                            // rows of a tile
-  Tile* work = nullptr;                    // work list of a batch (one simulation's is arithmetic)
-  int nwork = 0;                           // its entries, 0: not made yet
+  bool fp64 = false;
+  Work* work = nullptr;                    // a batch's work entries: streaming kernels, then VOP kernel
+  int nwork = 0, nstream = 0, nvop = 0;    // their numbers (nwork 0: not made yet)
   int fix_shape = -1;                      // caller's choices, -1: none
   int fix_staged = -1;
   bool staged_ok = false;                  // the caller may ask for staging 1 or 2
-  int2* chunk_map = nullptr;               // (instance, chunk) of every VOP chunk of a batch (device)
-  long long nchunks = 0;                   // VOP chunks of all instances
   GraphCache graphs;
   void drop_work() {
     graphs.clear();
@@ -72,11 +70,7 @@ struct Stepper {
     work = nullptr;
     nwork = 0;
   }
-  void release() {
-    drop_work();
-    if (chunk_map) cudaFree(chunk_map);
-    chunk_map = nullptr;
-  }
+  void release() { drop_work(); }
 };
 
 }  // namespace
@@ -258,7 +252,8 @@ bool same_hot_params(const DevParams& a, const DevParams& b) {
   std::memcpy(&x, &a, sizeof x);
   std::memcpy(&y, &b, sizeof y);
   for (DevParams* p : {&x, &y}) {
-    p->nx = p->ny = p->px = p->py = 0;
+    p->nx = p->ny = p->px = p->py = p->row_shift = 0;
+    p->row_mul = 0;
     p->per_liq = p->per_gas = p->ramp = p->useB = p->useF = 0;
     p->in_dx = p->in_dy = p->out_dx = p->out_dy = 0;
     p->k1 = p->k2 = p->k3 = p->k4 = p->inv_Keq = p->C_F_sat = p->r1_surface_factor = 0.0;
@@ -283,6 +278,15 @@ DevParams to_dev(const pslbm_params* p) {
   P.ny = p->ny;
   P.px = p->periodic_x ? 1 : 0;
   P.py = p->periodic_y ? 1 : 0;
+  // node / nx for 0 <= node < 2^31 as a product and a shift: with l = ceil(log2 nx)
+  // and m = ceil(2^(31+l) / nx), m nx exceeds 2^(31+l) by less than 2^l, so the
+  // quotient's error stays below 1 / nx; m fits 32 bits
+  {
+    int l = 0;
+    while ((1LL << l) < p->nx) ++l;
+    P.row_shift = 31 + l;
+    P.row_mul = (unsigned)(((1ULL << (31 + l)) + (unsigned)p->nx - 1) / (unsigned)p->nx);
+  }
   P.ns = p->n_species;
   P.iA = p->idx_A;
   P.iB = p->idx_B;
@@ -365,44 +369,65 @@ DevParams to_dev(const pslbm_params* p) {
   return P;
 }
 
-// Rows of a tile (a warp's share): 8 where the lattices give every SM 16 warps
-// of them, else fewer, down to one; a tile shape the caller asked for sets them
-// (256 nodes: 8 rows of 32, 512: 16).
-int tile_rows(const Stepper& st) {
-  if (st.fix_shape >= 0) return SHAPE_TX[st.fix_shape] * SHAPE_TY[st.fix_shape] / 32;
-  long long n = 0;
-  for (auto& d : st.dims) n += (long long)((d.first + 31) / 32) * d.second;
-  int rows = 8;
-  while (rows > 1 && n / rows < 152 * 16) rows /= 2;
-  return rows;
+// Warps for a list of n entries now (of at most N), each taking 32 entries at a
+// time in `turns` turns.  Lists grow as nodes dissolve: a few warps more than
+// needed, so that growth does not give one warp a turn more than the others.
+int list_warps(long long n, long long N, int turns) {
+  const long long room = std::min(N, n + std::max(2048LL, n / 8));
+  return (int)std::max(1LL, (room + 32LL * turns - 1) / (32LL * turns));
 }
 
-// Work list of the streaming kernels: tiles of 32 columns, then the chunks of 32
-// reservoir nodes.
+// Turns a warp of the streaming kernels takes.  Several, because each saves a
+// start (descriptor, step count, list) and has the next turn's loads in flight,
+// as long as every SM keeps 8 warps: 1024x512 (FP32) takes 66 us a step with one
+// turn, 58 with four, 54 with eight and 64 with sixteen; 4096x2048 619, 610, 612
+// and 628; a batch of 24 members 428, 381, 386 and 404.  FP64 is bound by its
+// arithmetic units, where many short warps even out: two turns at most (1024x512
+// 334 us with one, 322 with two, 353 with four), 128x64 30 us with one, 46 with two.
+int stream_turns(const Stepper& st, bool fp64) {
+  if (st.fix_shape >= 0) return SHAPE_TX[st.fix_shape] * SHAPE_TY[st.fix_shape] / 64;
+  long long n = 0;
+  for (int f : st.nfluid) n += f;
+  int turns = fp64 ? 2 : 8;
+  while (turns > 1 && n / 32 / turns < 152 * (fp64 ? 32 : 8)) turns /= 2;
+  return turns;
+}
+
+// Work entries of the streaming kernels (parts of the fluid lists, then chunks of
+// 32 reservoir nodes) and of the VOP kernel.
 cudaError_t ensure_work(Stepper& st) {
   if (st.nwork) return cudaSuccess;
-  const int rows = st.rows = tile_rows(st);
+  const int turns = stream_turns(st, st.fp64);
+  auto nodes = [&](int i) { return (long long)st.dims[i].first * st.dims[i].second; };
   if (st.mode == M_SINGLE) {
-    st.nwork = ((st.dims[0].first + 31) / 32) * ((st.dims[0].second + rows - 1) / rows) + (st.nres[0] + 31) / 32;
+    st.nstream = list_warps(st.nfluid[0], nodes(0), turns);
+    st.nwork = st.nstream + (st.nres[0] + 31) / 32;
+    st.nvop = list_warps(st.nface[0], nodes(0), 1);
     return cudaSuccess;
   }
-  std::vector<Tile> all;
+  std::vector<Work> all;
   for (int i = 0; i < (int)st.dims.size(); ++i) {
-    for (int y0 = 0; y0 < st.dims[i].second; y0 += rows)
-      for (int x0 = 0; x0 < st.dims[i].first; x0 += 32) all.push_back(Tile{i, x0, y0, -1});
-    for (int k = 0; k < st.nres[i]; k += 32) all.push_back(Tile{i, 0, 0, k});
+    const int nw = list_warps(st.nfluid[i], nodes(i), turns);
+    for (int c = 0; c < nw; ++c) all.push_back(Work{i, c * 32, nw * 32, -1});
+    for (int k = 0; k < st.nres[i]; k += 32) all.push_back(Work{i, 0, 0, k});
   }
-  Tile* d = nullptr;
-  cudaError_t e = cudaMalloc(&d, all.size() * sizeof(Tile));
+  const int nwork = (int)all.size();
+  for (int i = 0; i < (int)st.dims.size(); ++i) {
+    const int nw = list_warps(st.nface[i], nodes(i), 1);
+    for (int c = 0; c < nw; ++c) all.push_back(Work{i, c * 32, nw * 32, -1});
+  }
+  Work* d = nullptr;
+  cudaError_t e = cudaMalloc(&d, all.size() * sizeof(Work));
   if (e != cudaSuccess) return e;
-  e = cudaMemcpyAsync(d, all.data(), all.size() * sizeof(Tile), cudaMemcpyHostToDevice, lib_stream());
+  e = cudaMemcpyAsync(d, all.data(), all.size() * sizeof(Work), cudaMemcpyHostToDevice, lib_stream());
   if (e == cudaSuccess) e = cudaStreamSynchronize(lib_stream());
   if (e != cudaSuccess) {
     cudaFree(d);
     return e;
   }
   st.work = d;
-  st.nwork = (int)all.size();
+  st.nwork = nwork;
+  st.nvop = (int)all.size() - nwork;
   return cudaSuccess;
 }
 
@@ -429,15 +454,15 @@ void free_all(pslbm_t h) {
 
 // Enqueue the streaming kernels of one step.
 void enqueue_stream(cudaStream_t s, const Stepper& st) {
-  st.L->pot(s, st.work, st.nwork, st.rows, st.d, st.host0, st.mode);
-  st.L->move(s, st.work, st.nwork, st.rows, st.d, st.host0, st.mode);
+  st.L->pot(s, st.work, st.nwork, st.nstream, st.d, st.host0, st.mode);
+  st.L->move(s, st.work, st.nwork, st.nstream, st.d, st.host0, st.mode);
 }
 
 // Enqueue the kernels of n steps.
 void enqueue_steps(cudaStream_t s, const Stepper& st, int64_t n) {
   for (int64_t i = 0; i < n; ++i) {
     enqueue_stream(s, st);
-    st.L->vop(s, st.d, st.chunk_map, st.nchunks);
+    st.L->vop(s, st.d, st.work ? st.work + st.nwork : nullptr, st.nvop);
     st.L->amend(s, st.ninst, st.d);
   }
 }
@@ -465,7 +490,7 @@ pslbm_status profile_steps(Stepper& st, int64_t n, double* kernel_ms, double* to
     cudaEventRecord(ev[0], s);
     enqueue_stream(s, st);
     cudaEventRecord(ev[1], s);
-    st.L->vop(s, st.d, st.chunk_map, st.nchunks);
+    st.L->vop(s, st.d, st.work ? st.work + st.nwork : nullptr, st.nvop);
     cudaEventRecord(ev[2], s);
     st.L->amend(s, st.ninst, st.d);
     cudaEventRecord(ev[3], s);
@@ -661,9 +686,9 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     I.nres = (int)reslist.size();
     const size_t sizes[] = {fb, fb, gb, gb, (size_t)N, (size_t)N, (size_t)N * 2 * sizeof(double), (size_t)N,
                             (size_t)N * sizeof(double), (size_t)N * 2 * sizeof(int), (size_t)N * sizeof(int),
-                            (size_t)((N + 31) / 32) * sizeof(unsigned), S_NSCAL * sizeof(unsigned long long),
+                            (size_t)((N + 31) / 32) * 2 * sizeof(unsigned), S_NSCAL * sizeof(unsigned long long),
                             sizeof(DevInst), (size_t)(BUD_BLOCKS + 1) * NBUD * sizeof(double), (size_t)N * 4 * fsize(p->precision),
-                            (size_t)N, reslist.size() * sizeof(int)};
+                            (size_t)N, reslist.size() * sizeof(int), (size_t)N * 2 * sizeof(int)};
     constexpr int NPARTS = sizeof(sizes) / sizeof(sizes[0]);
     size_t offs[NPARTS], total = 0;
     for (int i = 0; i < NPARTS; ++i) {
@@ -685,7 +710,10 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     I.xs = (double*)(base + offs[8]);
     I.evlist = (int*)(base + offs[9]);
     I.claim = (int*)(base + offs[10]);
-    I.vmask = (unsigned*)(base + offs[11]);
+    I.fbits = (unsigned*)(base + offs[11]);
+    I.mbits = I.fbits + (N + 31) / 32;
+    I.flist = (int*)(base + offs[18]);
+    I.mlist = I.flist + N;
     I.scal = (unsigned long long*)(base + offs[12]);
     h->d = (DevInst*)(base + offs[13]);
     I.pot = base + offs[15];
@@ -707,7 +735,7 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     if (e == cudaSuccess && dc) e = cudaMemcpyAsync(dc, conc, N * ns * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(I.evt, 0, (size_t)N, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(I.claim, 0, (size_t)N * sizeof(int), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(I.vmask, 0, (size_t)((N + 31) / 32) * sizeof(unsigned), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(I.fbits, 0, (size_t)((N + 31) / 32) * 2 * sizeof(unsigned), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(I.scal, 0, S_NSCAL * sizeof(unsigned long long), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(I.scal + S_LIMIT, 0xff, sizeof(unsigned long long), s);
     if (e == cudaSuccess && ns) e = cudaMemsetAsync(I.g[1], 0, gb, s);
@@ -724,6 +752,12 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d, &I, sizeof(DevInst), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
       L->init(s, h->d, dmask, dr1, dr2, dc, N);
+      // node lists (the tile counts use the event list, empty between steps)
+      const int tiles = ((p->nx + 31) / 32) * ((p->ny + 7) / 8);
+      const int blocks = (tiles + ST_WARPS - 1) / ST_WARPS;
+      k_list<false><<<blocks, ST_THREADS, 0, s>>>(I, I.evlist, tiles);
+      k_list_scan<<<1, 1024, 0, s>>>(I.evlist, tiles, I.scal);
+      k_list<true><<<blocks, ST_THREADS, 0, s>>>(I, I.evlist, tiles);
       e = cudaGetLastError();
     }
     // initial liquid threshold: half the maximum initial rho_1 over fluid
@@ -737,7 +771,13 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     // the host copy of the descriptor is read by the copy above before the
     // call returns only for pageable memory; synchronise once for it and for
     // the errors of everything above
+    unsigned long long counts[2] = {0, 0};
+    static_assert(S_NFACE == S_NFLUID + 1, "read together");
+    if (e == cudaSuccess) e = cudaMemcpyAsync(counts, I.scal + S_NFLUID, sizeof counts, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    h->run.nfluid.assign(1, (int)counts[0]);
+    h->run.nface.assign(1, (int)counts[1]);
+    h->run.nres.assign(1, I.nres);
     if (e != cudaSuccess) {
       st = fail(nullptr, e == cudaErrorMemoryAllocation ? PSLBM_ERR_OOM : PSLBM_ERR_CUDA,
                 std::string("create: ") + cudaGetErrorString(e));
@@ -748,9 +788,8 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
   h->run.d = h->d;
   h->run.ninst = 1;
   h->run.dims.assign(1, {p->nx, p->ny});
-  h->run.nchunks = ((N + 31) / 32 + VOP_CHUNK - 1) / VOP_CHUNK;
   h->run.host0 = h->h;
-  h->run.nres.assign(1, I.nres);
+  h->run.fp64 = p->precision == PSLBM_FP64;
   h->run.staged_ok = staging_open(p);
   {
     cudaError_t e = ensure_work(h->run);
@@ -812,16 +851,14 @@ pslbm_status pslbm_estimate_device_bytes(const pslbm_params* p, uint64_t* bytes)
   if (!v.empty()) return fail(nullptr, PSLBM_ERR_PARAM, v);
   const uint64_t N = (uint64_t)p->nx * (uint64_t)p->ny;
   const uint64_t per = 2 * 18 * fsize(p->precision) + 2 * 5 * (uint64_t)p->n_species * gsize(p->precision) +
-                       2 /*types*/ + 4 * fsize(p->precision) + 1 /*potentials, codes*/ + 16 /*V*/ + 1 /*events*/ + 8 /*excess*/ + 8 /*event lists*/ + 4 /*claims*/;
-  const uint64_t vmask_bytes = ((N + 31) / 32) * 4;
-  // whole cells; reservoir nodes: the edges of the lattice (a batch's work list
-  // has an entry of 16 bytes per 32 nodes at most)
+                       2 /*types*/ + 4 * fsize(p->precision) + 1 /*potentials, codes*/ + 16 /*V*/ + 1 /*events*/ + 8 /*excess*/ + 8 /*event lists*/ + 4 /*claims*/ + 8 /*node lists*/;
+  const uint64_t bits = ((N + 31) / 32) * 8;
+  // whole cells; reservoir nodes: the edges of the lattice
   const uint64_t cells = (N + CELL - 1) / CELL * CELL;
   const uint64_t pops = 2 * 18 * fsize(p->precision) + 2 * 5 * (uint64_t)p->n_species * gsize(p->precision);
-  const uint64_t work = ((uint64_t)p->nx + 31) / 32 * (uint64_t)p->ny * sizeof(Tile);
   const uint64_t res = 2 * ((uint64_t)p->nx + (uint64_t)p->ny) * sizeof(int);
-  *bytes = N * per + (cells - N) * pops + vmask_bytes + work + res + sizeof(DevInst) + S_NSCAL * 8 +
-           (uint64_t)(BUD_BLOCKS + 1) * NBUD * sizeof(double) + 18 * 256;
+  *bytes = N * per + (cells - N) * pops + bits + res + sizeof(DevInst) + S_NSCAL * 8 +
+           (uint64_t)(BUD_BLOCKS + 1) * NBUD * sizeof(double) + 19 * 256;
   return PSLBM_OK;
 }
 
@@ -1019,28 +1056,21 @@ pslbm_status pslbm_batch_create(int32_t n, const pslbm_t* members, int32_t tile_
     di.push_back(members[i]->h);
     b->run.dims.push_back({members[i]->p.nx, members[i]->p.ny});
   }
-  // VOP chunks of all members, in member order
-  std::vector<int2> cmap;
-  for (int i = 0; i < n; ++i) {
-    const long long nc = ((members[i]->N + 31) / 32 + VOP_CHUNK - 1) / VOP_CHUNK;
-    for (long long c = 0; c < nc; ++c) cmap.push_back(make_int2(i, (int)c));
-  }
-  b->run.nchunks = (long long)cmap.size();
   cudaStream_t s = lib_stream();
   cudaError_t e = cudaMalloc(&b->d, di.size() * sizeof(DevInst));
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d, di.data(), di.size() * sizeof(DevInst), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMalloc(&b->run.chunk_map, cmap.size() * sizeof(int2));
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(b->run.chunk_map, cmap.data(), cmap.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   b->L = members[0]->L;
   b->run.L = b->L;
   b->run.d = b->d;
   b->run.ninst = n;
   b->run.host0 = members[0]->h;
+  b->run.fp64 = members[0]->prec == PSLBM_FP64;
   b->run.mode = M_SHARED;
   for (int i = 0; i < n; ++i) {
-    b->run.nres.push_back(members[i]->h.nres);
+    b->run.nfluid.push_back(members[i]->run.nfluid[0]);
+    b->run.nface.push_back(members[i]->run.nface[0]);
+    b->run.nres.push_back(members[i]->run.nres[0]);
     if (!same_hot_params(members[i]->h.P, members[0]->h.P)) b->run.mode = M_MIXED;
   }
   if (e == cudaSuccess) e = ensure_work(b->run);

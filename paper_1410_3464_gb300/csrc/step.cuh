@@ -102,42 +102,102 @@ __device__ __forceinline__ Pot<double> ld_pot(const Pot<double>* p) {
   return Pot<double>{v.x, v.y, __ldg(&p->p2), 0.0};
 }
 
-// Both kernels: a warp takes a tile of 32 columns by up to ST_ROWS rows, lists
-// its fluid nodes (in shared memory, in row order) and works through the list 32
-// at a time, so that solid nodes cost no lanes.  A few warps take the reservoir
-// nodes instead, 32 of the instance's list at a time.
+// Both kernels run over the instance's list of fluid nodes (in tile order, kept
+// up to date by the amendment kernel when nodes dissolve or fill), so that solid
+// nodes cost neither lanes nor loads.  A warp takes a chunk of the list, 32 nodes
+// at a time; a few warps take the reservoir nodes instead.
 constexpr int ST_WARPS = 4;
 constexpr int ST_THREADS = 32 * ST_WARPS;
-constexpr int ST_ROWS = 16;
 // Where a launch finds its instances: one simulation, whose descriptor comes as
-// a kernel argument (constant bank), or a batch's tile list and descriptors; in
+// a kernel argument (constant bank), or a batch's work list and descriptors; in
 // a batch of equal hot parameters those come as an argument too.
 enum { M_SINGLE = 0, M_SHARED = 1, M_MIXED = 2 };
 
-struct StepTile {
-  int inst, x0, y0, res;     // res: first entry of a reservoir chunk, or -1
-};
-// Tile of warp ti: the lattice's tiles row by row, then its reservoir chunks.
-template <int MODE>
-__device__ __forceinline__ bool step_tile(const Tile* __restrict__ tiles, int ntiles, int rows, const DevInst& Ik, int ti,
-                                          StepTile& t) {
-  if (ti >= ntiles) return false;
-  if constexpr (MODE == M_SINGLE) {
-    const int ncx = (Ik.P.nx + 31) >> 5;
-    const int nt = ncx * ((Ik.P.ny + rows - 1) / rows);
-    t.inst = 0;
-    t.res = ti >= nt ? (ti - nt) * 32 : -1;
-    const int ty = ti / ncx;
-    t.y0 = ty * rows;
-    t.x0 = (ti - ty * ncx) * 32;
-  } else {
-    const Tile l = tiles[ti];
-    t.inst = l.inst;
-    t.x0 = l.x0;
-    t.y0 = l.y0;
-    t.res = l.res;
-  }
+// Work of warp w: 32 list entries from `first` on, and the same again every
+// `stride` entries as far as the list goes; or reservoir nodes from entry `res`.
+__device__ __forceinline__ bool step_work(bool single, const Work* __restrict__ work, int nwork, int nstream, int w, Work& t) {
+  if (w >= nwork) return false;
+  if (single) t = Work{0, w * 32, nstream * 32, w >= nstream ? (w - nstream) * 32 : -1};
+  else t = work[w];
   return true;
+}
+
+// The fluid list and the list of minerals with a fluid axis neighbour, from the
+// node types (creation).  Both go through the lattice by tiles of 32 columns and
+// 8 rows, row by row within a tile, so that a warp's chunk of the list stays
+// together on the lattice: k_list<false> counts a tile's nodes (a warp a tile),
+// k_list_scan turns the counts into positions, k_list<true> writes the lists.
+template <bool FILL>
+static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constant__ DevInst I, int* __restrict__ counts, int ntiles) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int nx = I.P.nx, ny = I.P.ny, ncx = (nx + 31) >> 5;
+  const int ti = blockIdx.x * ST_WARPS + (threadIdx.x >> 5);
+  if (ti >= ntiles) return;
+  const int y0 = ti / ncx * 8, x = (ti % ncx) * 32 + lane;
+  const uint8_t* type = I.type[0];
+  int bf = FILL ? counts[ti] : 0, bm = FILL ? counts[ntiles + ti] : 0;
+  const unsigned below = (1u << lane) - 1u;
+#pragma unroll 4
+  for (int r = 0; r < 8; ++r) {
+    const int y = y0 + r;
+    const int node = y * nx + x;
+    const bool in = x < nx && y < ny;
+    const int t = in ? type[node] & T_MASK : T_WALL;
+    bool face = false;
+    if (in && is_mineral(t)) {
+#pragma unroll
+      for (int a = 1; a < 5; ++a) {
+        int xn, yn;
+        if (nbr(I.P, x, y, EX(a), EY(a), xn, yn)) face = face || is_fluid(type[yn * nx + xn] & T_MASK);
+      }
+    }
+    const bool fl = in && is_fluid(t);
+    const unsigned mf = __ballot_sync(FULL, fl), mm = __ballot_sync(FULL, face);
+    if constexpr (FILL) {
+      if (fl) {
+        I.flist[bf + __popc(mf & below)] = node;
+        atomicOr(&I.fbits[node >> 5], 1u << (node & 31));
+      }
+      if (face) {
+        I.mlist[bm + __popc(mm & below)] = node;
+        atomicOr(&I.mbits[node >> 5], 1u << (node & 31));
+      }
+    }
+    bf += __popc(mf);
+    bm += __popc(mm);
+  }
+  if (!FILL && lane == 0) {
+    counts[ti] = bf;
+    counts[ntiles + ti] = bm;
+  }
+}
+// One block: exclusive sums of both count arrays in place, totals into scal.
+static __global__ void __launch_bounds__(1024) k_list_scan(int* __restrict__ counts, int ntiles, unsigned long long* scal) {
+  __shared__ int sums[1024];
+  const int per = (ntiles + 1023) / 1024;
+  for (int k = 0; k < 2; ++k) {
+    int* c = counts + k * ntiles;
+    const int lo = min(threadIdx.x * per, ntiles), hi = min(lo + per, ntiles);
+    int s = 0;
+    for (int i = lo; i < hi; ++i) s += c[i];
+    sums[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 1; o < 1024; o <<= 1) {
+      const int v = threadIdx.x >= o ? sums[threadIdx.x - o] : 0;
+      __syncthreads();
+      sums[threadIdx.x] += v;
+      __syncthreads();
+    }
+    int at = sums[threadIdx.x] - s;
+    for (int i = lo; i < hi; ++i) {
+      const int v = c[i];
+      c[i] = at;
+      at += v;
+    }
+    if (threadIdx.x == 1023) scal[S_NFLUID + k] = (unsigned long long)sums[1023];
+    __syncthreads();
+  }
 }
 
 // Reservoir nodes i .. i + 31 of an instance: densities of the step, potentials
@@ -158,7 +218,6 @@ __device__ __noinline__ void reservoir_pot(const DevInst* I, int cur, unsigned l
   potentials<R>(P, R(a), R(b), ps, p1, p2, status);
   ((Pot<R>*)I->pot)[node] = Pot<R>{ps, p1, p2, R(0)};
   I->code[node] = (uint8_t)(C_RES | (R(a) > theta ? C_MARK : 0));
-  I->type[cur ^ 1][node] = t;
   if (status) atomicOr(&I->scal[S_STATUS], (unsigned long long)status);
 }
 
@@ -167,95 +226,69 @@ __device__ __noinline__ void reservoir_pot(const DevInst* I, int cur, unsigned l
 #endif
 template <class TF, class R, int MODE>
 __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : PSLBM_POT_MINB)
-    k_pot(const Tile* __restrict__ tiles, int ntiles, int rows, const DevInst* __restrict__ insts,
+    k_pot(const Work* __restrict__ work, int nwork, int nstream, const DevInst* __restrict__ insts,
           const __grid_constant__ DevInst Ik) {
-  constexpr unsigned FULL = 0xffffffffu;
-  __shared__ uint16_t lists[ST_WARPS][32 * ST_ROWS];
-  uint16_t* list = lists[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  StepTile tl;
-  if (!step_tile<MODE>(tiles, ntiles, rows, Ik, blockIdx.x * ST_WARPS + (threadIdx.x >> 5), tl)) return;
-  const DevInst& I = MODE == M_SINGLE ? Ik : insts[tl.inst];
+  Work wk;
+  if (!step_work(MODE == M_SINGLE, work, nwork, nstream, blockIdx.x * ST_WARPS + (threadIdx.x >> 5), wk)) return;
+  const DevInst& I = MODE == M_SINGLE ? Ik : insts[wk.inst];
   const DevParams& P = I.P;
   const DevParams& Q = MODE == M_MIXED ? P : Ik.P;
   unsigned long long* scal = I.scal;
   const unsigned long long step = scal[S_STEP];
   const bool live = step < scal[S_LIMIT];   // else a frozen instance
   const int cur = int(step & 1ULL);
-  if (tl.res >= 0) {
-    if (live) reservoir_pot<TF, R>(insts + tl.inst, cur, step, tl.res);
+  if (wk.res >= 0) {
+    if (live) reservoir_pot<TF, R>(insts + wk.inst, cur, step, wk.res);
     return;
   }
   if (!live) return;
+  const int n = (int)scal[S_NFLUID];
   const R theta = theta_of<R>(&I);
   const TF* __restrict__ fin = (const TF*)I.f[cur];
   const uint8_t* __restrict__ tin = I.type[cur];
   uint8_t* __restrict__ tout = I.type[cur ^ 1];
   Pot<R>* __restrict__ pot = (Pot<R>*)I.pot;
   uint8_t* __restrict__ code = I.code;
-  const int nx = P.nx, ny = P.ny;
-  const int x = tl.x0 + lane;
+  const int* __restrict__ flist = I.flist;
   TileAcc<R> acc{R(-1.0 / 0.0), 0u};
-  unsigned status = 0;
-
-  // ---- types: list the fluid nodes, settle the others
-  int n = 0;
-  for (int r0 = 0; r0 < rows; r0 += 8) {
-    uint8_t tv[8];
+  {
+    // the next node's populations are in flight while a lane reduces one
+    R q[18];
+    int next = wk.first + lane < n ? flist[wk.first + lane] : -1;
+    uint8_t tnext = 0;
+    auto fetch = [&] {
+      if (next < 0) return;
+      tnext = tin[next] & T_MASK;
+      const TF* fi = fin + foff(next);
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
-      tv[r] = (r0 + r < rows && x < nx && tl.y0 + r0 + r < ny) ? tin[(tl.y0 + r0 + r) * nx + x] : 0xFF;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const bool in = tv[r] != 0xFF;
-      const int t = tv[r] & T_MASK;
-      const int node = (tl.y0 + r0 + r) * nx + x;
-      const bool fl = in && is_fluid(t);
-      const unsigned m = __ballot_sync(FULL, fl);
-      if (fl) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(((r0 + r) << 5) | lane | (t << 12));
-      n += __popc(m);
-      if (in && !fl && !is_res(t)) {
-        code[node] = (uint8_t)type_code(t);
-        tout[node] = (uint8_t)t;
-      }
-    }
-  }
-  __syncwarp();
-
-  // ---- the fluid nodes; the next node's populations are in flight while a lane
-  // reduces one
-  R q[18];
-  int e = lane < n ? list[lane] : -1;
-  auto fetch = [&] {
-    if (e < 0) return;
-    const TF* fi = fin + foff((tl.y0 + ((e >> 5) & 15)) * nx + tl.x0 + (e & 31));
-#pragma unroll
-    for (int a = 0; a < 18; ++a) q[a] = ld<R>(fi + a * CELL);
-  };
-  fetch();
-#pragma unroll 1
-  for (int b = lane; b < n; b += 32) {
-    const int t = e >> 12;
-    const int node = (tl.y0 + ((e >> 5) & 15)) * nx + tl.x0 + (e & 31);
-    R d1 = q[0], d2 = q[9];
-#pragma unroll
-    for (int a = 1; a < 9; ++a) {
-      d1 += q[a];
-      d2 += q[9 + a];
-    }
-    e = b + 32 < n ? list[b + 32] : -1;
+      for (int a = 0; a < 18; ++a) q[a] = ld<R>(fi + a * CELL);
+    };
     fetch();
-    const R r1 = fshift<R>(Q, 0, t) + d1, r2 = fshift<R>(Q, 1, t) + d2;
-    if (!(r1 == r1 && r2 == r2)) status |= ST_NONFINITE;
-    acc.mx = rmax<R>(acc.mx, r1);
-    R ps, p1, p2;
-    potentials<R>(Q, r1, r2, ps, p1, p2, status);
-    const bool liq = r1 > theta;
-    pot[node] = Pot<R>{ps, p1, p2, R(0)};
-    code[node] = (uint8_t)(type_code(t) | (liq ? (C_MARK | C_FLIQ) : C_FGAS));
-    tout[node] = liq ? T_LIQUID : T_GAS;
+#pragma unroll 1
+    for (int i = wk.first + lane; i < n; i += wk.stride) {
+      const int node = next;
+      const int t = tnext;
+      R d1 = q[0], d2 = q[9];
+#pragma unroll
+      for (int a = 1; a < 9; ++a) {
+        d1 += q[a];
+        d2 += q[9 + a];
+      }
+      next = i + wk.stride < n ? flist[i + wk.stride] : -1;
+      fetch();
+      if (!is_fluid(t)) continue;     // filled since it was listed
+      const R r1 = fshift<R>(Q, 0, t) + d1, r2 = fshift<R>(Q, 1, t) + d2;
+      if (!(r1 == r1 && r2 == r2)) acc.status |= ST_NONFINITE;
+      acc.mx = rmax<R>(acc.mx, r1);
+      R ps, p1, p2;
+      potentials<R>(Q, r1, r2, ps, p1, p2, acc.status);
+      const bool liq = r1 > theta;
+      pot[node] = Pot<R>{ps, p1, p2, R(0)};
+      code[node] = (uint8_t)(type_code(t) | (liq ? (C_MARK | C_FLIQ) : C_FGAS));
+      tout[node] = liq ? T_LIQUID : T_GAS;
+    }
   }
-  acc.status = status;
   __syncwarp();
   flush_acc(acc, scal, cur);
 }
@@ -370,17 +403,15 @@ __device__ __noinline__ void reservoir_push(const DevInst* I, int cur, unsigned 
 #endif
 template <class TF, class TG, class R, int NS, int MODE>
 __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MINB)
-    k_move(const Tile* __restrict__ tiles, int ntiles, int rows, const DevInst* __restrict__ insts,
+    k_move(const Work* __restrict__ work, int nwork, int nstream, const DevInst* __restrict__ insts,
            const __grid_constant__ DevInst Ik) {
   using PR = Pair<R>;
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NP = (NS + 1) / 2, NPX = NP > 0 ? NP : 1;
-  __shared__ uint16_t lists[ST_WARPS][32 * ST_ROWS];
-  uint16_t* list = lists[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  StepTile tl;
-  if (!step_tile<MODE>(tiles, ntiles, rows, Ik, blockIdx.x * ST_WARPS + (threadIdx.x >> 5), tl)) return;
-  const DevInst& I = MODE == M_SINGLE ? Ik : insts[tl.inst];
+  Work wk;
+  if (!step_work(MODE == M_SINGLE, work, nwork, nstream, blockIdx.x * ST_WARPS + (threadIdx.x >> 5), wk)) return;
+  const DevInst& I = MODE == M_SINGLE ? Ik : insts[wk.inst];
   const DevParams& P = I.P;
   const DevParams& Q = MODE == M_MIXED ? P : Ik.P;
   const DevParamsR<R>& rates = rp<R>(P);
@@ -388,55 +419,38 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
   const unsigned long long step = I.scal[S_STEP];
   const bool live = step < I.scal[S_LIMIT];   // else a frozen instance
   const int cur = int(step & 1ULL);
-  if (tl.res >= 0) {
-    if (live) reservoir_push<TF, TG, R, NS>(insts + tl.inst, cur, step, tl.res);
+  if (wk.res >= 0) {
+    if (live) reservoir_push<TF, TG, R, NS>(insts + wk.inst, cur, step, wk.res);
     return;
   }
   if (!live) return;
+  const int n = (int)I.scal[S_NFLUID];
+  const int* __restrict__ flist = I.flist;
   const TF* __restrict__ fin = (const TF*)I.f[cur];
   TF* __restrict__ fout = (TF*)I.f[cur ^ 1];
   const TG* __restrict__ gin = (const TG*)I.g[cur];
   TG* __restrict__ gout = (TG*)I.g[cur ^ 1];
   const Pot<R>* __restrict__ pot = (const Pot<R>*)I.pot;
   const uint8_t* __restrict__ code = I.code;
-  unsigned* __restrict__ vmask = I.vmask;
   const int nx = P.nx, ny = P.ny;
   const bool px = P.px != 0, py = P.py != 0;
   auto spec = [&](const R* v, int k) { return mk<R>(v[2 * k], v[2 * k + 1]); };
 
-  // ---- list the fluid nodes
-  int n = 0;
-  {
-    const int x = tl.x0 + lane;
-    for (int r0 = 0; r0 < rows; r0 += 8) {
-      uint8_t cv[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r)
-        cv[r] = (r0 + r < rows && x < nx && tl.y0 + r0 + r < ny) ? __ldg(code + (tl.y0 + r0 + r) * nx + x) : 0;
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const bool fl = (cv[r] & C_FLUID) != 0;
-        const unsigned m = __ballot_sync(FULL, fl);
-        if (fl) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(((r0 + r) << 5) | lane);
-        n += __popc(m);
-      }
-    }
-  }
-  __syncwarp();
-
+  int next = wk.first + lane < n ? flist[wk.first + lane] : -1;
 #pragma unroll 1
-  for (int b = 0; b < n; b += 32) {
-  const unsigned act = __ballot_sync(FULL, b + lane < n);
-  if (b + lane >= n) break;
-  const int e = list[b + lane];
-  const int x = tl.x0 + (e & 31), y = tl.y0 + (e >> 5);
-  const int node = y * nx + x;
+  for (int b = wk.first; b < n; b += wk.stride) {
+  const int node = next < 0 ? 0 : next;
+  const bool in_list = next >= 0;
+  next = b + wk.stride + lane < n ? flist[b + wk.stride + lane] : -1;
+  // all loads that depend on the node alone go out together
   PR F[9];      // populations of the two components
   {
     const TF* fi = fin + foff(node);
 #pragma unroll
     for (int a = 0; a < 9; ++a) F[a] = mk<R>(ld<R>(fi + a * CELL), ld<R>(fi + (9 + a) * CELL));
   }
+  const int c0 = __ldg(code + node);
+  const int y = node_row(P, node), x = node - y * nx;
   // ---- neighbours: index offsets (with periodic wrap) and codes (outside a
   // non-periodic edge a wall)
   const bool vl = x > 0 || px, vr = x + 1 < nx || px, vd = y > 0 || py, vu = y + 1 < ny || py;
@@ -444,32 +458,33 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
   const int od = y > 0 ? -nx : (ny - 1) * nx, ou = y + 1 < ny ? nx : -(ny - 1) * nx;
   int dn[9], nc[9];
   dn[0] = 0;
+  nc[0] = c0;
 #pragma unroll
-  for (int a = 0; a < 9; ++a) {
+  for (int a = 1; a < 9; ++a) {
     dn[a] = (EX(a) > 0 ? orr : EX(a) < 0 ? ol : 0) + (EY(a) > 0 ? ou : EY(a) < 0 ? od : 0);
     const bool in = (EX(a) > 0 ? vr : EX(a) < 0 ? vl : true) && (EY(a) > 0 ? vu : EY(a) < 0 ? vd : true);
     nc[a] = in ? (int)__ldg(code + node + dn[a]) : 0;
   }
-  const int c0 = nc[0];
+  PR gs[NPX][5];   // solute populations, two species a pair (unused at a node that was gas)
+  if constexpr (NS > 0) {
+    const TG* gi = gin + goff<NS>(node);
+#pragma unroll
+    for (int k = 0; k < NP; ++k)
+#pragma unroll
+      for (int a = 0; a < 5; ++a) {
+        const R ga = ld<R>(gi + (2 * k * 5 + a) * CELL);
+        const R gb = 2 * k + 1 < NS ? ld<R>(gi + ((2 * k + 1) * 5 + a) * CELL) : R(0);
+        gs[k][a] = mk<R>(ga, gb);
+        if constexpr (Is16<TG>::value) gs[k][a] = gs[k][a] * spec(rp<R>(Q).gs_div, k);
+      }
+  }
+  const bool on = in_list && (c0 & C_FLUID);      // else past the end, or filled since it was listed
+  const unsigned act = __ballot_sync(FULL, on);
+  if (!on) continue;
   const bool liq = (c0 & C_MARK) != 0, was = (c0 & C_OLDLIQ) != 0;
   const uint8_t t = was ? T_LIQUID : T_GAS;
   const int axis = nc[1] | nc[2] | nc[3] | nc[4];
   const int orc = axis | nc[5] | nc[6] | nc[7] | nc[8];
-  PR gs[NPX][5];   // solute populations, two species a pair
-  if constexpr (NS > 0) {
-    if (was) {
-      const TG* gi = gin + goff<NS>(node);
-#pragma unroll
-      for (int k = 0; k < NP; ++k)
-#pragma unroll
-        for (int a = 0; a < 5; ++a) {
-          const R ga = ld<R>(gi + (2 * k * 5 + a) * CELL);
-          const R gb = 2 * k + 1 < NS ? ld<R>(gi + ((2 * k + 1) * 5 + a) * CELL) : R(0);
-          gs[k][a] = mk<R>(ga, gb);
-          if constexpr (Is16<TG>::value) gs[k][a] = gs[k][a] * spec(rp<R>(Q).gs_div, k);
-        }
-    }
-  }
   // ---- force stencils (force_stencils): a non-live neighbour's values are read
   // at its mirror image
   PR sx, sy;      // stencil sums of (psi_1, phi_1)
@@ -560,13 +575,6 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
     ux = pfma<R>(Fx, q, mk<R>(u_common<R>(jx.a, jx.b, it1, it2, rden)));
     uy = pfma<R>(Fy, q, mk<R>(u_common<R>(jy.a, jy.b, it1, it2, rden)));
   }
-  // minerals on the axis links of a liquid node, for the VOP kernel
-  if (liq && (axis & C_MIN)) {
-#pragma unroll
-    for (int a = 1; a < 5; ++a)
-      if (nc[a] & C_MIN) atomicOr(&vmask[(node + dn[a]) >> 5], 1u << ((node + dn[a]) & 31));
-  }
-
   // ---- solutes: concentration with the Step-2 amendment, sources
   PR S = mk<R>(R(0));      // fluid sources
   PR C[NPX], Sk[NPX];
@@ -598,7 +606,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
             ++nsrc;
           } else {
             int nrec = 0;
-            const int yn = nn / nx, xn = nn - yn * nx;
+            const int yn = node_row(P, nn), xn = nn - yn * nx;
             if (xn > 0 || px) nrec += (code[nn + (xn > 0 ? -1 : nx - 1)] & C_FLIQ) ? 1 : 0;
             if (xn + 1 < nx || px) nrec += (code[nn + (xn + 1 < nx ? 1 : 1 - nx)] & C_FLIQ) ? 1 : 0;
             if (yn > 0 || py) nrec += (code[nn + (yn > 0 ? -nx : (ny - 1) * nx)] & C_FLIQ) ? 1 : 0;
