@@ -54,7 +54,7 @@ struct DevParamsR {
   R tau[2], inv_tau[2], G11, G12, G21, a0, inv_rho10, inv_rho20, w_adh[2];
   R eos_a, eos_b4, eos_RT, six_over_G11;
   R gx, gy, shift_f[2], shift_fg[2], rho_fill[2];
-  R J0[MAXS], Ja[MAXS], inv_tau_g[MAXS], shift_c[MAXS], conc_in[MAXS], cR1[MAXS], cR3[MAXS];
+  R J0[MAXS], Ja[MAXS], inv_tau_g[MAXS], keep_g[MAXS], half_tau_g[MAXS], shift_c[MAXS], conc_in[MAXS], cR1[MAXS], cR3[MAXS];
   R k1, k1_inv_Keq, k3, k2, k4, C_F_sat, gas_yield, inv_M_C, c_total_per_rho1;
   R k1_s, k1_inv_Keq_s;   // R1 constants at liquid nodes touching D(s) (surface factor applied)
   // reactive link rule (Eqs. 29-31 as a halfway wall): link flux q = out * qa - qc,
@@ -75,6 +75,9 @@ struct DevParams {
   int r1_surf;                        // R1 surface factor differs from 1
   int tau_unit;                       // both relaxation times are 1
   int has_w;                          // a fluid-solid interaction strength differs from 0
+  int has_g;                          // a body force acts
+  int phi2_cut;                       // high word of the rho_1 / rho_10 above which exp(-rho_1 / rho_10)
+                                      // is below half an ulp of a0 (FP64 potentials)
   int in_dx, in_dy, out_dx, out_dy;   // node downstream of an inlet / upstream of an outlet
   double tau[2], G11, G12, G21, a0, rho10, rho20, w_adh[2];
   double eos_a, eos_b, eos_R, eos_T;
@@ -365,12 +368,59 @@ template <class R> __device__ __forceinline__ R psi_arg(const DevParams& P, R rh
   return rmul<R>(Q.six_over_G11, rsub<R>(p, rmul<R>(rho, R(1.0 / 3.0))));
 }
 
+// FP64 reciprocal and square root.  An FP64 instruction holds its quarter of an SM
+// for 64 cycles whatever its lanes do (measured; FP32: 2), so the FP64 kernels
+// cost what they issue.  Both take the hardware's approximation (20 bits and more)
+// and one third-order correction of Newton's iteration: with e = 1 - v r the
+// reciprocal is r (1 + e + e^2 + O(e^3)), and with e = 1 - v y^2 the square root is
+// v y (1 + e/2 + 3 e^2/8 + O(e^3)).  Arguments near the ends of the exponent
+// range, zero, infinities and NaN take the CUDA operation.
+__device__ __forceinline__ bool mid_range(double v) {
+  return (((unsigned)__double2hiint(v) >> 20) & 0x7FFu) - 24u < 2000u;
+}
+__device__ __forceinline__ double rcp64(double v) {
+  if (!mid_range(v)) return 1.0 / v;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+  const double e = __fma_rn(-v, r, 1.0);
+  return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+__device__ __forceinline__ double sqrt64(double v) {
+  if (!mid_range(v)) return sqrt(v);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+  const double g = __dmul_rn(v, y);
+  const double e = __fma_rn(-g, y, 1.0);
+  return __fma_rn(g, __dmul_rn(e, __fma_rn(0.375, e, 0.5)), g);
+}
+// Comparisons of doubles on their bits (no FP64 instruction); x is not NaN.
+__device__ __forceinline__ long long order_bits(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFLL);
+}
+template <class R> __device__ __forceinline__ bool is_nan(R x) { return !(x == x); }
+template <> __device__ __forceinline__ bool is_nan<double>(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x) & 0x7FFFFFFFu;
+  return hi > 0x7FF00000u || (hi == 0x7FF00000u && __double2loint(x) != 0);
+}
+template <class R> __device__ __forceinline__ bool above(R x, R y) { return x > y; }   // x, y not NaN
+template <> __device__ __forceinline__ bool above<double>(double x, double y) { return order_bits(x) > order_bits(y); }
+template <class R> __device__ __forceinline__ bool is_zero(R x) { return x == R(0); }
+template <> __device__ __forceinline__ bool is_zero<double>(double x) {
+  return ((__double2hiint(x) << 1) | __double2loint(x)) == 0;
+}
 template <class R> __device__ __forceinline__ R rrcp(R v);
-template <> __device__ __forceinline__ double rrcp<double>(double v) { return 1.0 / v; }
+template <> __device__ __forceinline__ double rrcp<double>(double v) { return rcp64(v); }
 template <> __device__ __forceinline__ float rrcp<float>(float v) { return __frcp_rn(v); }
 template <class R> __device__ __forceinline__ R rmax(R a, R b);
 template <> __device__ __forceinline__ double rmax<double>(double a, double b) { return fmax(a, b); }
 template <> __device__ __forceinline__ float rmax<float>(float a, float b) { return fmaxf(a, b); }
+// max(0, x), 0 for NaN
+template <class R> __device__ __forceinline__ R clamp0(R x) { return rmax<R>(R(0), x); }
+template <> __device__ __forceinline__ double clamp0<double>(double x) {
+  return __double2hiint(x) < 0 || is_nan<double>(x) ? 0.0 : x;
+}
+
 template <class R> __device__ __forceinline__ R rexp(R v);
 template <> __device__ __forceinline__ double rexp<double>(double v) { return exp(v); }
 template <> __device__ __forceinline__ float rexp<float>(float v) { return expf(v); }
@@ -540,6 +590,47 @@ __device__ __forceinline__ void potentials(const DevParams& P, R rho1, R rho2, R
   }
   phi1 = -rexpm1<R>(-rmul<R>(rho2, Q.inv_rho20));
   phi2 = rsub<R>(Q.a0, rexp<R>(-rmul<R>(rho1, Q.inv_rho10)));
+}
+// FP64: the same with few FP64 instructions (rcp64, sqrt64).  phi_2's exponential
+// is left out where it is below half an ulp of a0 (P.phi2_cut, in the liquid), and
+// phi_1 = x - x^2/2 + x^3/6 - ... is summed as it stands for small x = rho_2 /
+// rho_20 (also the liquid): for |x| < 1/16 ten terms leave 2.3e-20 of x.
+template <>
+__device__ __forceinline__ void potentials<double>(const DevParams& P, double rho1, double rho2, double& psi, double& phi1,
+                                                   double& phi2, unsigned& status) {
+  const DevParamsR<double>& Q = P.rd;
+  psi = 0.0;
+  if (P.has_G11) {
+    const double eta = Q.eos_b4 * rho1;
+    const double om = 1.0 - eta;
+    const double poly = __fma_rn(eta, __fma_rn(eta, om, 1.0), 1.0);
+    const double num = (rho1 * Q.eos_RT) * poly;
+    const double p = __fma_rn(-(Q.eos_a * rho1), rho1, num * rcp64(om * om * om));
+    double arg = Q.six_over_G11 * __fma_rn(rho1, -1.0 / 3.0, p);
+    if (is_nan(arg) || (__double2hiint(arg) < 0 && !is_zero(arg))) {
+      status |= is_nan(arg) ? ST_NONFINITE : ST_EOS;
+      arg = 0.0;
+    }
+    psi = sqrt64(arg);
+  }
+  const double x = rho2 * Q.inv_rho20;
+  if ((__double2hiint(x) & 0x7FFFFFFF) < 0x3FB00000) {
+    double s = -1.0 / 3628800.0;
+    s = __fma_rn(s, x, 1.0 / 362880.0);
+    s = __fma_rn(s, x, -1.0 / 40320.0);
+    s = __fma_rn(s, x, 1.0 / 5040.0);
+    s = __fma_rn(s, x, -1.0 / 720.0);
+    s = __fma_rn(s, x, 1.0 / 120.0);
+    s = __fma_rn(s, x, -1.0 / 24.0);
+    s = __fma_rn(s, x, 1.0 / 6.0);
+    s = __fma_rn(s, x, -0.5);
+    phi1 = __fma_rn(__dmul_rn(s, x), x, x);
+  } else {
+    phi1 = -expm1(-x);
+  }
+  const double z = rho1 * Q.inv_rho10;
+  phi2 = Q.a0;
+  if (!(__double2hiint(z) > P.phi2_cut)) phi2 = Q.a0 - exp(-z);
 }
 
 // SplitMix64 output for a given state (Steele, Lea, Flood 2014).

@@ -158,17 +158,21 @@ constexpr int vop_min_blocks() {
 template <class TF, class TG, class R, int NS>
 __global__ void __launch_bounds__(NTHREADS, vop_min_blocks<R>())
     k_vop(const DevInst* __restrict__ insts, const Work* __restrict__ work, int nwork) {
+  step_begin();
   const int lane = threadIdx.x & 31;
   const int w = (blockIdx.x * (int)blockDim.x + threadIdx.x) >> 5;
   if (w >= nwork) return;
   const Work wk = work ? work[w] : Work{0, w * 32, nwork * 32, -1};
   const DevInst* Ip = insts + wk.inst;
+  const int N = (int)Ip->N;
+  int node = Ip->mlist[min(wk.first + lane, N - 1)];   // in flight beside the counters
   const unsigned long long step = Ip->scal[S_STEP];
   if (step >= Ip->scal[S_LIMIT]) return;   // frozen instance
   const int n = (int)Ip->scal[S_NFACE];
-  for (int first = wk.first; first < n; first += wk.stride)
-    if (first + lane < n)
-      vop_node<TF, TG, R, NS>(Ip, Ip->P, (int)Ip->N, int(step & 1ULL), step, Ip->mlist[first + lane]);
+  for (int i = wk.first + lane; i < n; i += wk.stride) {
+    vop_node<TF, TG, R, NS>(Ip, Ip->P, N, int(step & 1ULL), step, node);
+    if (i + wk.stride < n) node = Ip->mlist[i + wk.stride];
+  }
 }
 
 // Append a node to a list unless it is listed (bits).
@@ -197,6 +201,7 @@ __device__ __forceinline__ void finish_step(const DevInst* Ip, unsigned long lon
 
 template <class TF, class TG, class R, int NS>
 __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ insts) {
+  step_begin();
   const DevInst* Ip = insts + blockIdx.x;
   // the counters this kernel reads, loaded together (one memory round trip)
   const volatile unsigned long long* sc = Ip->scal;

@@ -9,6 +9,23 @@
 namespace pslbm {
 namespace {
 
+// The kernels of a step are launched with programmatic stream serialisation: a
+// kernel's blocks may start while the one before it drains, and wait
+// (step_begin) for its end and its writes before they read anything.
+template <class... A>
+void launch_step(cudaStream_t s, int blocks, int threads, void (*kernel)(A...), A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = blocks <= 304 ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Streaming kernels over nwork warps; Ik: the descriptor of a single simulation
 // (mode M_SINGLE), or of a batch's first member (M_SHARED: all members have its
 // hot parameters).
@@ -16,27 +33,27 @@ template <int NS>
 void pot_l(cudaStream_t s, const Work* work, int nwork, int nstream, const DevInst* insts, const DevInst& Ik, int mode) {
   if (nwork <= 0) return;
   const int blocks = (nwork + ST_WARPS - 1) / ST_WARPS;
-  if (mode == M_SINGLE) k_pot<KTF, KR, M_SINGLE><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
-  else if (mode == M_SHARED) k_pot<KTF, KR, M_SHARED><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
-  else k_pot<KTF, KR, M_MIXED><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
+  auto k = mode == M_SINGLE ? k_pot<KTF, KR, M_SINGLE> : mode == M_SHARED ? k_pot<KTF, KR, M_SHARED> : k_pot<KTF, KR, M_MIXED>;
+  launch_step<const Work*, int, int, const DevInst*, DevInst>(s, blocks, ST_THREADS, k, work, nwork, nstream, insts, Ik);
 }
 template <int NS>
 void move_l(cudaStream_t s, const Work* work, int nwork, int nstream, const DevInst* insts, const DevInst& Ik, int mode) {
   if (nwork <= 0) return;
   const int blocks = (nwork + ST_WARPS - 1) / ST_WARPS;
-  if (mode == M_SINGLE) k_move<KTF, KTG, KR, NS, M_SINGLE><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
-  else if (mode == M_SHARED) k_move<KTF, KTG, KR, NS, M_SHARED><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
-  else k_move<KTF, KTG, KR, NS, M_MIXED><<<blocks, ST_THREADS, 0, s>>>(work, nwork, nstream, insts, Ik);
+  auto k = mode == M_SINGLE ? k_move<KTF, KTG, KR, NS, M_SINGLE>
+           : mode == M_SHARED ? k_move<KTF, KTG, KR, NS, M_SHARED> : k_move<KTF, KTG, KR, NS, M_MIXED>;
+  launch_step<const Work*, int, int, const DevInst*, DevInst>(s, blocks, ST_THREADS, k, work, nwork, nstream, insts, Ik);
 }
 template <int NS>
 void vop_l(cudaStream_t s, const DevInst* insts, const Work* work, int nwork) {
   if (nwork <= 0) return;
-  k_vop<KTF, KTG, KR, NS><<<(nwork + NTHREADS / 32 - 1) / (NTHREADS / 32), NTHREADS, 0, s>>>(insts, work, nwork);
+  launch_step<const DevInst*, const Work*, int>(s, (nwork + NTHREADS / 32 - 1) / (NTHREADS / 32), NTHREADS,
+                                                k_vop<KTF, KTG, KR, NS>, insts, work, nwork);
 }
 template <int NS>
 void amend_l(cudaStream_t s, int ninst, const DevInst* insts) {
   if (ninst <= 0) return;
-  k_amend<KTF, KTG, KR, NS><<<ninst, NTHREADS, 0, s>>>(insts);
+  launch_step<const DevInst*>(s, ninst, NTHREADS, k_amend<KTF, KTG, KR, NS>, insts);
 }
 template <int NS>
 void init_l(cudaStream_t s, DevInst* I, const uint8_t* m, const double* r1, const double* r2, const double* c,

@@ -211,6 +211,8 @@ void fill_r(DevParamsR<R>& q, const DevParams& P) {
     q.J0[k] = R(P.J0[k]);
     q.Ja[k] = R(P.Ja[k]);
     q.inv_tau_g[k] = R(P.inv_tau_g[k]);
+    q.keep_g[k] = R(1.0 - P.inv_tau_g[k]);
+    q.half_tau_g[k] = R(0.5 * P.inv_tau_g[k]);
     q.shift_c[k] = R(P.shift_c[k]);
     q.conc_in[k] = R(P.conc_in[k]);
     q.cR1[k] = R(P.cR1[k]);
@@ -358,6 +360,16 @@ DevParams to_dev(const pslbm_params* p) {
   P.Vbar_F = p->Vbar_F;
   P.V_split = p->V_split;
   P.seed = p->seed;
+  P.has_g = p->body_force[0] != 0.0 || p->body_force[1] != 0.0;
+  // exp(-z) < 2^-55 |a0| for z > ln(2^55 / |a0|); one step up in the high word
+  // covers its low bits
+  P.phi2_cut = 0x7FFFFFFF;
+  if (std::isfinite(p->a0) && std::fabs(p->a0) > 1e-290) {
+    const double cut = std::max(1.0, std::log(std::ldexp(1.0, 55) / std::fabs(p->a0)));
+    int64_t bits;
+    std::memcpy(&bits, &cut, sizeof bits);
+    P.phi2_cut = (int)(bits >> 32) + 1;
+  }
   P.has_w = p->w_adh[0] != 0.0 || p->w_adh[1] != 0.0;
   P.tau_unit = p->tau[0] == 1.0 && p->tau[1] == 1.0;
   P.has_G11 = p->G11 != 0.0;

@@ -101,6 +101,9 @@ __device__ __forceinline__ Pot<double> ld_pot(const Pot<double>* p) {
   const double2 v = __ldg(reinterpret_cast<const double2*>(p));
   return Pot<double>{v.x, v.y, __ldg(&p->p2), 0.0};
 }
+// FP64: rho_1 rides along with the potentials (eight additions less in k_move).
+__device__ __forceinline__ double pot_rho1(const Pot<double>* p) { return __ldg(&p->pad); }
+__device__ __forceinline__ float pot_rho1(const Pot<float>*) { return 0.f; }
 
 // Both kernels run over the instance's list of fluid nodes (in tile order, kept
 // up to date by the amendment kernel when nodes dissolve or fill), so that solid
@@ -112,6 +115,14 @@ constexpr int ST_THREADS = 32 * ST_WARPS;
 // a kernel argument (constant bank), or a batch's work list and descriptors; in
 // a batch of equal hot parameters those come as an argument too.
 enum { M_SINGLE = 0, M_SHARED = 1, M_MIXED = 2 };
+
+// Start of a step's kernel (kernels_impl.cuh, launch_step): the next kernel may
+// launch its blocks as this one's leave room; wait until the one before has
+// ended.  Every thread of every block calls it before anything else.
+__device__ __forceinline__ void step_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // Work of warp w: 32 list entries from `first` on, and the same again every
 // `stride` entries as far as the list goes; or reservoir nodes from entry `res`.
@@ -228,6 +239,7 @@ template <class TF, class R, int MODE>
 __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : PSLBM_POT_MINB)
     k_pot(const Work* __restrict__ work, int nwork, int nstream, const DevInst* __restrict__ insts,
           const __grid_constant__ DevInst Ik) {
+  step_begin();
   const int lane = threadIdx.x & 31;
   Work wk;
   if (!step_work(MODE == M_SINGLE, work, nwork, nstream, blockIdx.x * ST_WARPS + (threadIdx.x >> 5), wk)) return;
@@ -235,6 +247,8 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : PSLBM_POT_MIN
   const DevParams& P = I.P;
   const DevParams& Q = MODE == M_MIXED ? P : Ik.P;
   unsigned long long* scal = I.scal;
+  const int* __restrict__ flist = I.flist;
+  const int head = flist[min(wk.first + lane, (int)I.N - 1)];   // in flight beside the counters
   const unsigned long long step = scal[S_STEP];
   const bool live = step < scal[S_LIMIT];   // else a frozen instance
   const int cur = int(step & 1ULL);
@@ -250,12 +264,11 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : PSLBM_POT_MIN
   uint8_t* __restrict__ tout = I.type[cur ^ 1];
   Pot<R>* __restrict__ pot = (Pot<R>*)I.pot;
   uint8_t* __restrict__ code = I.code;
-  const int* __restrict__ flist = I.flist;
   TileAcc<R> acc{R(-1.0 / 0.0), 0u};
   {
     // the next node's populations are in flight while a lane reduces one
     R q[18];
-    int next = wk.first + lane < n ? flist[wk.first + lane] : -1;
+    int next = wk.first + lane < n ? head : -1;
     uint8_t tnext = 0;
     auto fetch = [&] {
       if (next < 0) return;
@@ -278,13 +291,18 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : PSLBM_POT_MIN
       next = i + wk.stride < n ? flist[i + wk.stride] : -1;
       fetch();
       if (!is_fluid(t)) continue;     // filled since it was listed
-      const R r1 = fshift<R>(Q, 0, t) + d1, r2 = fshift<R>(Q, 1, t) + d2;
-      if (!(r1 == r1 && r2 == r2)) acc.status |= ST_NONFINITE;
-      acc.mx = rmax<R>(acc.mx, r1);
+      R r1 = d1, r2 = d2;
+      if constexpr (sizeof(R) == 4) {      // FP64 stores no shift
+        r1 = fshift<R>(Q, 0, t) + d1;
+        r2 = fshift<R>(Q, 1, t) + d2;
+      }
+      const bool nan1 = is_nan<R>(r1);
+      if (nan1 || is_nan<R>(r2)) acc.status |= ST_NONFINITE;
+      if (!nan1 && above<R>(r1, acc.mx)) acc.mx = r1;
       R ps, p1, p2;
       potentials<R>(Q, r1, r2, ps, p1, p2, acc.status);
-      const bool liq = r1 > theta;
-      pot[node] = Pot<R>{ps, p1, p2, R(0)};
+      const bool liq = !nan1 && above<R>(r1, theta);
+      pot[node] = Pot<R>{ps, p1, p2, r1};
       code[node] = (uint8_t)(type_code(t) | (liq ? (C_MARK | C_FLIQ) : C_FGAS));
       tout[node] = liq ? T_LIQUID : T_GAS;
     }
@@ -408,6 +426,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
   using PR = Pair<R>;
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NP = (NS + 1) / 2, NPX = NP > 0 ? NP : 1;
+  step_begin();
   const int lane = threadIdx.x & 31;
   Work wk;
   if (!step_work(MODE == M_SINGLE, work, nwork, nstream, blockIdx.x * ST_WARPS + (threadIdx.x >> 5), wk)) return;
@@ -416,6 +435,8 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
   const DevParams& Q = MODE == M_MIXED ? P : Ik.P;
   const DevParamsR<R>& rates = rp<R>(P);
   auto pr = [](const R& v) { return MODE == M_SINGLE ? v : __ldg(&v); };
+  const int* __restrict__ flist = I.flist;
+  const int head = flist[min(wk.first + lane, (int)I.N - 1)];   // in flight beside the counters
   const unsigned long long step = I.scal[S_STEP];
   const bool live = step < I.scal[S_LIMIT];   // else a frozen instance
   const int cur = int(step & 1ULL);
@@ -425,7 +446,6 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
   }
   if (!live) return;
   const int n = (int)I.scal[S_NFLUID];
-  const int* __restrict__ flist = I.flist;
   const TF* __restrict__ fin = (const TF*)I.f[cur];
   TF* __restrict__ fout = (TF*)I.f[cur ^ 1];
   const TG* __restrict__ gin = (const TG*)I.g[cur];
@@ -436,7 +456,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
   const bool px = P.px != 0, py = P.py != 0;
   auto spec = [&](const R* v, int k) { return mk<R>(v[2 * k], v[2 * k + 1]); };
 
-  int next = wk.first + lane < n ? flist[wk.first + lane] : -1;
+  int next = wk.first + lane < n ? head : -1;
 #pragma unroll 1
   for (int b = wk.first; b < n; b += wk.stride) {
   const int node = next < 0 ? 0 : next;
@@ -527,15 +547,26 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
   }
   // ---- moments (Eq. 9)
   PR d, jx, jy;
-  {
+  PR sh, rho;
+  if constexpr (sizeof(R) == 4) {
     d = F[0];
 #pragma unroll
     for (int a = 1; a < 9; ++a) d = d + F[a];
     jx = ((F[1] - F[3]) + (F[5] - F[6])) + (F[8] - F[7]);
     jy = ((F[2] - F[4]) + (F[5] - F[8])) + (F[6] - F[7]);
+    sh = mk<R>(fshift<R>(Q, 0, t), fshift<R>(Q, 1, t));
+    rho = sh + d;
+  } else {
+    // no shift, and as few FP64 instructions as will do
+    R d2 = F[0].b;
+#pragma unroll
+    for (int a = 1; a < 9; ++a) d2 += F[a].b;
+    rho = d = mk<R>(pot_rho1(pot + node), d2);
+    const PR q = F[5] - F[7], r = F[8] - F[6];
+    jx = (F[1] - F[3]) + (q + r);
+    jy = (F[2] - F[4]) + (q - r);
+    sh = mk<R>(R(0));
   }
-  const PR sh = mk<R>(fshift<R>(Q, 0, t), fshift<R>(Q, 1, t));
-  const PR rho = sh + d;
   const R rho1 = rho.a, rho2 = rho.b;
   // ---- forces (Eqs. 11, 14a/b, 16 and the body force; force1, force2)
   PR Fx, Fy;
@@ -558,22 +589,37 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
       Fx = pfma<R>(mw, mk<R>(rmul<R>(R(ix), R(1.0 / 36.0))), Fx);
       Fy = pfma<R>(mw, mk<R>(rmul<R>(R(iy), R(1.0 / 36.0))), Fy);
     }
-    Fx = pfma<R>(rho, mk<R>(rp<R>(Q).gx), Fx);
-    Fy = pfma<R>(rho, mk<R>(rp<R>(Q).gy), Fy);
+    if (Q.has_g) {
+      Fx = pfma<R>(rho, mk<R>(rp<R>(Q).gx), Fx);
+      Fy = pfma<R>(rho, mk<R>(rp<R>(Q).gy), Fy);
+    }
   }
   // ---- velocities (Eqs. 17-19)
   const R it1 = rp<R>(Q).inv_tau[0], it2 = rp<R>(Q).inv_tau[1];
   const R rrt = rrcp<R>(radd<R>(rho1, rho2));
   // both relaxation times 1 (the paper's choice): the same sum, the same bits
   const R rden = Q.tau_unit ? rrt : rrcp<R>(rfma<R>(rho1, it1, rmul<R>(rho2, it2)));
-  const R urx = u_phys<R>(jx.a, jx.b, Fx.a, Fx.b, rrt);
-  const R ury = u_phys<R>(jy.a, jy.b, Fy.a, Fy.b, rrt);
+  R urx, ury;
   PR ux, uy;
   {
-    const PR q = mk<R>(rho1 != R(0) ? rmul<R>(rp<R>(Q).tau[0], rrcp<R>(rho1)) : R(0),
-                       rho2 != R(0) ? rmul<R>(rp<R>(Q).tau[1], rrcp<R>(rho2)) : R(0));
-    ux = pfma<R>(Fx, q, mk<R>(u_common<R>(jx.a, jx.b, it1, it2, rden)));
-    uy = pfma<R>(Fy, q, mk<R>(u_common<R>(jy.a, jy.b, it1, it2, rden)));
+    const R q1 = is_zero<R>(rho1) ? R(0) : rmul<R>(rp<R>(Q).tau[0], rrcp<R>(rho1));
+    const R q2 = is_zero<R>(rho2) ? R(0) : rmul<R>(rp<R>(Q).tau[1], rrcp<R>(rho2));
+    const PR q = mk<R>(q1, q2);
+    R upx, upy;
+    if (sizeof(R) == 8 && Q.tau_unit) {
+      upx = (jx.a + jx.b) * rrt;
+      upy = (jy.a + jy.b) * rrt;
+      const R h = R(0.5) * rrt;
+      urx = rfma<R>(h, Fx.a + Fx.b, upx);
+      ury = rfma<R>(h, Fy.a + Fy.b, upy);
+    } else {
+      upx = u_common<R>(jx.a, jx.b, it1, it2, rden);
+      upy = u_common<R>(jy.a, jy.b, it1, it2, rden);
+      urx = u_phys<R>(jx.a, jx.b, Fx.a, Fx.b, rrt);
+      ury = u_phys<R>(jy.a, jy.b, Fy.a, Fy.b, rrt);
+    }
+    ux = pfma<R>(Fx, q, mk<R>(upx));
+    uy = pfma<R>(Fy, q, mk<R>(upy));
   }
   // ---- solutes: concentration with the Step-2 amendment, sources
   PR S = mk<R>(R(0));      // fluid sources
@@ -635,7 +681,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
         PR s = gs[k][0];
 #pragma unroll
         for (int a = 1; a < 5; ++a) s = s + gs[k][a];
-        C[k] = spec(rp<R>(Q).shift_c, k) + s;
+        C[k] = sizeof(R) == 8 ? s : spec(rp<R>(Q).shift_c, k) + s;
       }
       // homogeneous reactions (Eqs. 5a, 5c; sources Eqs. 27, 28)
       R CA = R(0), CB = R(0), CE = R(0), tot = R(0);
@@ -647,7 +693,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
         if (k == Q.iE) CE = ck;
         tot += ck;
       }
-      if (Q.iA == -2) CA = rmax<R>(R(0), rfma<R>(rp<R>(Q).c_total_per_rho1, rho1, -tot));
+      if (Q.iA == -2) CA = clamp0<R>(rfma<R>(rp<R>(Q).c_total_per_rho1, rho1, -tot));
       // Section 2: R1 is faster at the surface of D(s) (a liquid node with a
       // D(s) node on an axis link)
       const bool surf = Q.r1_surf && (axis & C_SOLD);
@@ -683,11 +729,32 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
       const R rs = c1 ? rho.a : rho.b, ds = c1 ? d.a : d.b, vx = c1 ? ux.a : ux.b, vy = c1 ? uy.a : uy.b,
               Ss = c1 ? S.a : S.b, it = c1 ? it1 : it2;
       TF* fo = fout + s * 9 * CELL;
-      const R uu = half_u2<R>(vx, vy);
       R feq[9];
-      feq_pairs<R>(ds, rs, vx, vy, uu, feq);
+      if (sizeof(R) == 8 && Q.tau_unit) {
+        // FP64 at tau = 1: the collision leaves the equilibrium and the source,
+        // w (rho (1 + 3 e.u + 4.5 (e.u)^2 - 1.5 u^2) + S), here with the parts that
+        // directions share formed once (30 FP64 instructions instead of 64)
+        const R xx = vx * vx, yy = vy * vy, u2 = xx + yy, tx = vx + vx;
+        const R A = rfma<R>(R(-1.5) * rs, u2, rs + Ss), A9 = R(1.0 / 9.0) * A, A36 = R(1.0 / 36.0) * A;
+        const R h = R(0.5) * rs, h8 = R(0.125) * rs, as = R(1.0 / 3.0) * rs, ad = R(1.0 / 12.0) * rs;
+        const R sx_ = rfma<R>(h, xx, A9), sy_ = rfma<R>(h, yy, A9);
+        const R sp = rfma<R>(h8, rfma<R>(tx, vy, u2), A36), sm = rfma<R>(h8, rfma<R>(-tx, vy, u2), A36);
+        const R ep = vx + vy, em = vy - vx;
+        feq[0] = R(4.0 / 9.0) * A;
+        feq[1] = rfma<R>(as, vx, sx_);
+        feq[3] = rfma<R>(-as, vx, sx_);
+        feq[2] = rfma<R>(as, vy, sy_);
+        feq[4] = rfma<R>(-as, vy, sy_);
+        feq[5] = rfma<R>(ad, ep, sp);
+        feq[7] = rfma<R>(-ad, ep, sp);
+        feq[6] = rfma<R>(ad, em, sm);
+        feq[8] = rfma<R>(-ad, em, sm);
+      } else {
+        const R uu = half_u2<R>(vx, vy);
+        feq_pairs<R>(ds, rs, vx, vy, uu, feq);
 #pragma unroll
-      for (int a = 0; a < 9; ++a) feq[a] = bgk<R>(c1 ? F[a].a : F[a].b, feq[a], it, w9<R>(a), Ss);
+        for (int a = 0; a < 9; ++a) feq[a] = bgk<R>(c1 ? F[a].a : F[a].b, feq[a], it, w9<R>(a), Ss);
+      }
       if (!odd) {
 #pragma unroll
         for (int a = 0; a < 9; ++a) st<TF, R>(fo + to[a], feq[a]);
@@ -697,7 +764,8 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
 #pragma unroll
         for (int a = 0; a < 9; ++a) {
           const bool to_liq = (a > 0 && (nc[a] & C_FLUID)) ? (nc[a] & C_MARK) != 0 : liq;
-          if (a == 0 || !(nc[a] & C_RES)) st<TF, R>(fo + to[a], rfma<R>(w9<R>(a), to_liq ? dl : dg, feq[a]));
+          if (a == 0 || !(nc[a] & C_RES))
+            st<TF, R>(fo + to[a], sizeof(R) == 8 ? feq[a] : rfma<R>(w9<R>(a), to_liq ? dl : dg, feq[a]));
         }
       }
     }
@@ -721,14 +789,26 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
         const PR J0 = spec(rp<R>(Q).J0, k), Ja = spec(rp<R>(Q).Ja, k), it = spec(rp<R>(Q).inv_tau_g, k);
-        const PR cs = C[k] - spec(rp<R>(Q).shift_c, k), hc = mk<R>(R(0.5)) * C[k];
-        const PR sa = Ja * cs, ax = hc * vx, ay = hc * vy;
-        const PR ge[5] = {J0 * cs, sa + ax, sa + ay, sa - ax, sa - ay};
+        PR go[5];
+        if constexpr (sizeof(R) == 8) {
+          // the same sum regrouped: (1 - 1/tau_g) g + J (C / tau_g + S) + C e.u / (2 tau_g)
+          const PR B = pfma<R>(it, C[k], Sk[k]), b0 = J0 * B, ba = Ja * B;
+          const PR t2 = spec(rp<R>(Q).half_tau_g, k) * C[k], n2 = mk<R>(-t2.a, -t2.b), om = spec(rp<R>(Q).keep_g, k);
+          go[0] = pfma<R>(gs[k][0], om, b0);
+          go[1] = pfma<R>(gs[k][1], om, pfma<R>(t2, vx, ba));
+          go[2] = pfma<R>(gs[k][2], om, pfma<R>(t2, vy, ba));
+          go[3] = pfma<R>(gs[k][3], om, pfma<R>(n2, vx, ba));
+          go[4] = pfma<R>(gs[k][4], om, pfma<R>(n2, vy, ba));
+        } else {
+          const PR cs = C[k] - spec(rp<R>(Q).shift_c, k), hc = mk<R>(R(0.5)) * C[k];
+          const PR sa = Ja * cs, ax = hc * vx, ay = hc * vy;
+          const PR ge[5] = {J0 * cs, sa + ax, sa + ay, sa - ax, sa - ay};
 #pragma unroll
-        for (int a = 0; a < 5; ++a) {
-          const PR g = pfma<R>(a == 0 ? J0 : Ja, Sk[k], pfma<R>(ge[a] - gs[k][a], it, gs[k][a]));
-          if (a == 0 || (nc[a] & (C_RES | C_MARK)) != (C_RES | C_MARK)) put(k, to[a], g);
+          for (int a = 0; a < 5; ++a) go[a] = pfma<R>(a == 0 ? J0 : Ja, Sk[k], pfma<R>(ge[a] - gs[k][a], it, gs[k][a]));
         }
+#pragma unroll
+        for (int a = 0; a < 5; ++a)
+          if (a == 0 || (nc[a] & (C_RES | C_MARK)) != (C_RES | C_MARK)) put(k, to[a], go[a]);
       }
     } else {
       // gas node: no solute
