@@ -60,6 +60,7 @@ struct Stepper {
   bool fp64 = false;
   Work* work = nullptr;                    // a batch's work entries: streaming kernels, then VOP kernel
   int nwork = 0, nstream = 0, nvop = 0;    // their numbers (nwork 0: not made yet)
+  int npot = 0;                            // warps of k_pot in the place of nstream (one simulation)
   int fix_shape = -1;                      // caller's choices, -1: none
   int fix_staged = -1;
   bool staged_ok = false;                  // the caller may ask for staging 1 or 2
@@ -382,26 +383,32 @@ DevParams to_dev(const pslbm_params* p) {
 }
 
 // Warps for a list of n entries now (of at most N), each taking 32 entries at a
-// time in `turns` turns.  Lists grow as nodes dissolve: a few warps more than
-// needed, so that growth does not give one warp a turn more than the others.
-int list_warps(long long n, long long N, int turns) {
-  const long long room = std::min(N, n + std::max(2048LL, n / 8));
-  return (int)std::max(1LL, (room + 32LL * turns - 1) / (32LL * turns));
+// time in `turns` turns.  Lists grow as nodes dissolve: with one turn a few warps
+// more than needed, so that growth does not give some a second one.
+int list_warps(long long n, long long N, double turns) {
+  const long long room = turns > 1.0 ? n : std::min(N, n + std::max(2048LL, n / 8));
+  return (int)std::max(1.0, std::ceil(double(room) / (32.0 * turns)));
 }
 
 // Turns a warp of the streaming kernels takes.  Several, because each saves a
-// start (descriptor, step count, list) and has the next turn's loads in flight,
-// as long as every SM keeps 8 warps: 1024x512 (FP32) takes 66 us a step with one
-// turn, 58 with four, 54 with eight and 64 with sixteen; 4096x2048 619, 610, 612
-// and 628; a batch of 24 members 428, 381, 386 and 404.  FP64 is bound by its
-// arithmetic units, where many short warps even out: two turns at most (1024x512
-// 334 us with one, 322 with two, 353 with four), 128x64 30 us with one, 46 with two.
-int stream_turns(const Stepper& st, bool fp64) {
+// start (descriptor, step count, list) and has the next turn's list entry in
+// flight.  One simulation up to 64 turns: one wave of 8 warps an SM (FP64: 16),
+// whose warps sweep the list together, so that what neighbours share is met in
+// L2: 1024x512 FP32 48.7 us a step, against 56.7 with 16 warps, 54.4 with 8 turns
+// in two waves and 66 with one turn; 2048x1024 161, 171, 169, 181; 1024x512 FP64
+// 209 with 16 warps, 214 with 8, 228 with 2 turns.  k_pot, with a third of the
+// loads in flight, takes 16 in either type (8: 2048x1024 177 us).  Longer lists: 8 turns
+// (4096x2048 601 us, one wave 619, one turn 619).  A batch, whose members' lists
+// do not join up: 8 turns (FP64 2), fewer where that leaves SMs idle (24 members
+// 384 us, one wave 405 to 450, one turn 428).
+double stream_turns(const Stepper& st, bool pot) {
   if (st.fix_shape >= 0) return SHAPE_TX[st.fix_shape] * SHAPE_TY[st.fix_shape] / 64;
-  long long n = 0;
-  for (int f : st.nfluid) n += f;
-  int turns = fp64 ? 2 : 8;
-  while (turns > 1 && n / 32 / turns < 152 * (fp64 ? 32 : 8)) turns /= 2;
+  double chunks = 0;
+  for (int f : st.nfluid) chunks += (f + 31) / 32;
+  const double wave = 152.0 * (st.fp64 || (pot && st.mode == M_SINGLE) ? 16 : 8);
+  if (st.mode == M_SINGLE && chunks <= 64 * 152 * (st.fp64 ? 16 : 8)) return std::max(1.0, chunks / wave);
+  double turns = st.mode != M_SINGLE && st.fp64 ? 2 : 8;
+  while (turns > 1 && chunks / turns < wave) turns /= 2;
   return turns;
 }
 
@@ -409,14 +416,15 @@ int stream_turns(const Stepper& st, bool fp64) {
 // 32 reservoir nodes) and of the VOP kernel.
 cudaError_t ensure_work(Stepper& st) {
   if (st.nwork) return cudaSuccess;
-  const int turns = stream_turns(st, st.fp64);
   auto nodes = [&](int i) { return (long long)st.dims[i].first * st.dims[i].second; };
   if (st.mode == M_SINGLE) {
-    st.nstream = list_warps(st.nfluid[0], nodes(0), turns);
+    st.npot = list_warps(st.nfluid[0], nodes(0), stream_turns(st, true));
+    st.nstream = list_warps(st.nfluid[0], nodes(0), stream_turns(st, false));
     st.nwork = st.nstream + (st.nres[0] + 31) / 32;
     st.nvop = list_warps(st.nface[0], nodes(0), 1);
     return cudaSuccess;
   }
+  const double turns = stream_turns(st, false);
   std::vector<Work> all;
   for (int i = 0; i < (int)st.dims.size(); ++i) {
     const int nw = list_warps(st.nfluid[i], nodes(i), turns);
@@ -466,7 +474,8 @@ void free_all(pslbm_t h) {
 
 // Enqueue the streaming kernels of one step.
 void enqueue_stream(cudaStream_t s, const Stepper& st) {
-  st.L->pot(s, st.work, st.nwork, st.nstream, st.d, st.host0, st.mode);
+  const int more = st.mode == M_SINGLE ? st.npot - st.nstream : 0;
+  st.L->pot(s, st.work, st.nwork + more, st.nstream + more, st.d, st.host0, st.mode);
   st.L->move(s, st.work, st.nwork, st.nstream, st.d, st.host0, st.mode);
 }
 
