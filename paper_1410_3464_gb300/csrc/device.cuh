@@ -105,8 +105,8 @@ template <> __host__ __device__ __forceinline__ const DevParamsR<double>& rp<dou
 
 struct DevInst {
   DevParams P;
-  void* f[2];                 // [2][9][N] populations, ping-pong
-  void* g[2];                 // [ns][5][N] solute populations, ping-pong
+  void* f[2];                 // populations in cells (foff), ping-pong
+  void* g[2];                 // solute populations in cells (goff), ping-pong
   uint8_t* type[2];           // [N] node types, ping-pong
   void* pot;                  // [N] potentials of this step (Pot<R>)
   uint8_t* code;              // [N] codes of this step (C_* bits)
@@ -125,6 +125,7 @@ struct DevInst {
   long long N;
   int evcap;
   int nres;
+  int read_once;              // populations may leave L2 once k_move has read them (pslbm_create)
 };
 
 // A warp's work: 32 entries of an instance's list from entry `first` on, and
@@ -150,13 +151,8 @@ __host__ __device__ constexpr int opp_(int a) {
 template <class R> __device__ __forceinline__ R w9(int a) {
   return a == 0 ? R(4.0 / 9.0) : (a < 5 ? R(1.0 / 9.0) : R(1.0 / 36.0));
 }
-// interaction weights w(|e|^2): 1/9 axis, 1/36 diagonal (sum w e_x^2 = c_s^2)
-template <class R> __device__ __forceinline__ R wf(int a) {
-  return a == 0 ? R(0) : (a < 5 ? R(1.0 / 9.0) : R(1.0 / 36.0));
-}
 
 __device__ __forceinline__ bool is_fluid(uint8_t t) { return t <= T_GAS; }
-__device__ __forceinline__ bool is_res(uint8_t t) { return t == T_INLET || t == T_OUTLET; }
 __device__ __forceinline__ bool is_live(uint8_t t) { return t <= T_GAS || t == T_INLET || t == T_OUTLET; }
 __device__ __forceinline__ bool is_mineral(uint8_t t) { return t == T_SOLID_D || t == T_SOLID_F; }
 
@@ -168,6 +164,34 @@ template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v
 template <class R, class T> __device__ __forceinline__ R ld(const T* p) { return R(to_f<T>(__ldg(p))); }
 template <> __device__ __forceinline__ double ld<double, double>(const double* p) { return __ldg(p); }
 template <> __device__ __forceinline__ float ld<float, float>(const float* p) { return __ldg(p); }
+// L2 eviction policies, and a load under one (read-only path).
+__device__ __forceinline__ unsigned long long l2_evict_first() {
+  unsigned long long p;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+__device__ __forceinline__ unsigned long long l2_evict_normal() {
+  unsigned long long p;
+  asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+template <class R, class T> __device__ __forceinline__ R ld_l2(const T* p, unsigned long long policy) {
+  if constexpr (sizeof(T) == 8) {
+    double v;
+    asm("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(policy));
+    return R(v);
+  } else if constexpr (sizeof(T) == 4) {
+    float v;
+    asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(policy));
+    return R(v);
+  } else {
+    unsigned short v;
+    asm("ld.global.nc.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(p), "l"(policy));
+    T t;
+    memcpy(&t, &v, sizeof t);
+    return R(to_f<T>(t));
+  }
+}
 template <class T, class R> __device__ __forceinline__ void st(T* p, R v);
 template <> __device__ __forceinline__ void st<double, double>(double* p, double v) { *p = v; }
 template <> __device__ __forceinline__ void st<float, float>(float* p, float v) { *p = v; }
@@ -337,9 +361,9 @@ __device__ __forceinline__ bool outlet_up_liquid(const DevParams& P, const uint8
 
 // Explicitly rounded operations.  The hot formulas are written with these
 // (fused where a product feeds a sum) so that the compiler cannot contract
-// them differently in different kernel variants: every variant -- plain
-// loads, TMA stages, parameters from global memory or from the constant bank
-// -- evaluates exactly the same operations and gives bit-identical results.
+// them differently in different instantiations: with parameters from global
+// memory or from the constant bank, alone or in a batch, the kernels evaluate
+// exactly the same operations and give bit-identical results.
 template <class R> __device__ __forceinline__ R radd(R a, R b);
 template <class R> __device__ __forceinline__ R rsub(R a, R b);
 template <class R> __device__ __forceinline__ R rmul(R a, R b);

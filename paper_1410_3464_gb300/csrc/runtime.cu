@@ -382,6 +382,15 @@ DevParams to_dev(const pslbm_params* p) {
   return P;
 }
 
+// Whether k_move reads populations of this many bytes (both buffers) with an L2
+// policy that lets them go first.  They are read for the last time, and while not
+// much more than the 129 MB L2 is in use that keeps what the step and the next one
+// still want: FP32, per step, 700x700 (129 MB) 45.9 -> 40.5 us, 1024x512 (138 MB)
+// 48.6 -> 42.3, 1200x600 (190 MB) 64.4 -> 60.4.  Above, lines go before the chunks
+// that share them have read them: 1448x724 (277 MB) 88.1 -> 93.6, 4096x2048 622 ->
+// 698.  FP64 does not care.
+bool read_once(size_t bytes) { return bytes <= 220000000; }
+
 // Warps for a list of n entries now (of at most N), each taking 32 entries at a
 // time in `turns` turns.  Lists grow as nodes dissolve: with one turn a few warps
 // more than needed, so that growth does not give some a second one.
@@ -705,6 +714,7 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     for (long long i = 0; i < N; ++i)
       if ((mask[i] & 15) >= PSLBM_INLET && (mask[i] & 15) <= PSLBM_OUTLET) reslist.push_back((int)i);
     I.nres = (int)reslist.size();
+    I.read_once = read_once(2 * (fb + gb)) ? 1 : 0;
     const size_t sizes[] = {fb, fb, gb, gb, (size_t)N, (size_t)N, (size_t)N * 2 * sizeof(double), (size_t)N,
                             (size_t)N * sizeof(double), (size_t)N * 2 * sizeof(int), (size_t)N * sizeof(int),
                             (size_t)((N + 31) / 32) * 2 * sizeof(unsigned), S_NSCAL * sizeof(unsigned long long),

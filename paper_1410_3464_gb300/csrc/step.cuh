@@ -107,7 +107,8 @@ __device__ __forceinline__ float pot_rho1(const Pot<float>*) { return 0.f; }
 
 // Both kernels run over the instance's list of fluid nodes (in tile order, kept
 // up to date by the amendment kernel when nodes dissolve or fill), so that solid
-// nodes cost neither lanes nor loads.  A warp takes a chunk of the list, 32 nodes
+// nodes cost neither lanes nor loads (1024x512 FP32: 62 us a step over all nodes,
+// 54 over the list; FP64 430 and 322).  A warp takes a chunk of the list, 32 nodes
 // at a time; a few warps take the reservoir nodes instead.
 constexpr int ST_WARPS = 4;
 constexpr int ST_THREADS = 32 * ST_WARPS;
@@ -136,7 +137,8 @@ __device__ __forceinline__ bool step_work(bool single, const Work* __restrict__ 
 // The fluid list and the list of minerals with a fluid axis neighbour, from the
 // node types (creation).  Both go through the lattice by tiles of 32 columns and
 // 8 rows, row by row within a tile, so that a warp's chunk of the list stays
-// together on the lattice: k_list<false> counts a tile's nodes (a warp a tile),
+// together on the lattice (4096x2048 FP32: 612 us a step, 717 to 766 with the tiles
+// in the order of an atomic counter): k_list<false> counts a tile's nodes (a warp a tile),
 // k_list_scan turns the counts into positions, k_list<true> writes the lists.
 template <bool FILL>
 static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constant__ DevInst I, int* __restrict__ counts, int ntiles) {
@@ -232,11 +234,13 @@ __device__ __noinline__ void reservoir_pot(const DevInst* I, int cur, unsigned l
   if (status) atomicOr(&I->scal[S_STATUS], (unsigned long long)status);
 }
 
-#ifndef PSLBM_POT_MINB
-#define PSLBM_POT_MINB 8
-#endif
+// Bound by its reads: 18 populations a node in, 16 bytes (FP64 32), a code and a type
+// out; in FP64 by the equation of state and the exponentials.  A kernel of its own
+// because one that also collides had to hold or recompute the ring of neighbours:
+// 1,522 warp instructions and a block barrier per 32 nodes, 77 us at 1024x512 FP32
+// (FP64 460), where k_pot and k_move take 41 (FP64 213) together.
 template <class TF, class R, int MODE>
-__global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : PSLBM_POT_MINB)
+__global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : 8)
     k_pot(const Work* __restrict__ work, int nwork, int nstream, const DevInst* __restrict__ insts,
           const __grid_constant__ DevInst Ik) {
   step_begin();
@@ -416,11 +420,16 @@ __device__ __noinline__ void reservoir_push(const DevInst* I, int cur, unsigned 
                                      R(r1), R(r2), nbits, (I->code[node] & C_MARK) != 0);
 }
 
-#ifndef PSLBM_MOVE_MINB
-#define PSLBM_MOVE_MINB 4
-#endif
+// Bound by memory latency in FP32 (18 + 5 NS populations and nine potentials in, the
+// populations out; 128 registers, so 16 warps an SM at most, and more warps at fewer
+// registers measured slower), by the FP64 pipe in FP64, where an instruction of a warp
+// takes 64 cycles however many lanes are in: hence the regrouped collisions, few
+// comparisons, and lists without idle lanes (1024x512 FP64: 322 us a step before the
+// regrouping, 228 after).  The FP32 arithmetic keeps its order and rounding.
+// Everything that depends on the node alone is loaded before the first use; the loop
+// stays within the instruction cache (nothing rare inline but the Step-2 amendment).
 template <class TF, class TG, class R, int NS, int MODE>
-__global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MINB)
+__global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : 4)
     k_move(const Work* __restrict__ work, int nwork, int nstream, const DevInst* __restrict__ insts,
            const __grid_constant__ DevInst Ik) {
   using PR = Pair<R>;
@@ -455,6 +464,8 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
   const int nx = P.nx, ny = P.ny;
   const bool px = P.px != 0, py = P.py != 0;
   auto spec = [&](const R* v, int k) { return mk<R>(v[2 * k], v[2 * k + 1]); };
+  // populations are read for the last time in this step
+  const unsigned long long once = MODE == M_SINGLE && Ik.read_once ? l2_evict_first() : l2_evict_normal();
 
   int next = wk.first + lane < n ? head : -1;
 #pragma unroll 1
@@ -467,7 +478,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
   {
     const TF* fi = fin + foff(node);
 #pragma unroll
-    for (int a = 0; a < 9; ++a) F[a] = mk<R>(ld<R>(fi + a * CELL), ld<R>(fi + (9 + a) * CELL));
+    for (int a = 0; a < 9; ++a) F[a] = mk<R>(ld_l2<R>(fi + a * CELL, once), ld_l2<R>(fi + (9 + a) * CELL, once));
   }
   const int c0 = __ldg(code + node);
   const int y = node_row(P, node), x = node - y * nx;
@@ -492,8 +503,8 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : PSLBM_MOVE_MI
     for (int k = 0; k < NP; ++k)
 #pragma unroll
       for (int a = 0; a < 5; ++a) {
-        const R ga = ld<R>(gi + (2 * k * 5 + a) * CELL);
-        const R gb = 2 * k + 1 < NS ? ld<R>(gi + ((2 * k + 1) * 5 + a) * CELL) : R(0);
+        const R ga = ld_l2<R>(gi + (2 * k * 5 + a) * CELL, once);
+        const R gb = 2 * k + 1 < NS ? ld_l2<R>(gi + ((2 * k + 1) * 5 + a) * CELL, once) : R(0);
         gs[k][a] = mk<R>(ga, gb);
         if constexpr (Is16<TG>::value) gs[k][a] = gs[k][a] * spec(rp<R>(Q).gs_div, k);
       }
