@@ -4,6 +4,9 @@
 
 namespace pslbm {
 
+// Threads a block of the field kernels: few, so that a small lattice reaches all SMs.
+constexpr int FIELD_THREADS = 64;
+
 // Rest equilibrium (Eq. 8 at u = 0, Eq. 21 at u = 0) from initial fields.
 template <class TF, class TG, class R, int NS>
 __global__ void k_init(DevInst* __restrict__ Ip, const uint8_t* __restrict__ mask, const double* __restrict__ rho1,
@@ -39,11 +42,43 @@ __global__ void k_init(DevInst* __restrict__ Ip, const uint8_t* __restrict__ mas
   }
 }
 
+// Potentials of the current state at fluid and reservoir nodes, for k_fields (the
+// next step's k_pot overwrites them).  k_fields alone evaluated the equation of
+// state at each node and its eight neighbours.
+template <class TF, class R>
+__global__ void __launch_bounds__(FIELD_THREADS) k_fields_pot(const DevInst* __restrict__ Ip) {
+  const DevParams& P = Ip->P;
+  const unsigned long long step = Ip->scal[S_STEP];
+  const int cur = int(step & 1ULL), N = (int)Ip->N;
+  const TF* F = (const TF*)Ip->f[cur];
+  const uint8_t* T = Ip->type[cur];
+  Pot<R>* pot = (Pot<R>*)Ip->pot;
+  unsigned status = 0;      // flagged by the steps themselves
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+    const int node = (int)i;
+    const uint8_t t = T[node] & T_MASK;
+    if (!is_live(t)) continue;
+    R r1, r2;
+    if (is_fluid(t)) {
+      r1 = fshift<R>(P, 0, t) + density_shifted<R>(F, 0, node);
+      r2 = fshift<R>(P, 1, t) + density_shifted<R>(F, 1, node);
+    } else {
+      double u, v;
+      reservoir_rho(P, t, step, t == T_OUTLET && outlet_up_liquid<R, TF>(P, T, F, N, node, theta_of<R>(Ip)), u, v);
+      r1 = R(u);
+      r2 = R(v);
+    }
+    R ps, p1, p2;
+    potentials<R>(P, r1, r2, ps, p1, p2, status);
+    pot[node] = Pot<R>{ps, p1, p2, r1};
+  }
+}
+
 // Observable fields of the current state: rho_1, rho_2, u_r (Eq. 19) at fluid
-// nodes, C_k at liquid nodes, node types.  Forces are recomputed from the
-// neighbours' densities exactly as in the bulk kernel.
+// nodes, C_k at liquid nodes, node types; a null output is left out.  The forces
+// are those of the step (k_move), from the potentials of k_fields_pot.
 template <class TF, class TG, class R, int NS>
-__global__ void k_fields(const DevInst* __restrict__ Ip, double* __restrict__ o_rho1, double* __restrict__ o_rho2,
+__global__ void __launch_bounds__(FIELD_THREADS) k_fields(const DevInst* __restrict__ Ip, double* __restrict__ o_rho1, double* __restrict__ o_rho2,
                          double* __restrict__ o_ux, double* __restrict__ o_uy, double* __restrict__ o_conc,
                          uint8_t* __restrict__ o_type) {
   const DevParams& P = Ip->P;
@@ -53,14 +88,15 @@ __global__ void k_fields(const DevInst* __restrict__ Ip, double* __restrict__ o_
   const TF* F = (const TF*)Ip->f[cur];
   const TG* G = (const TG*)Ip->g[cur];
   const uint8_t* T = Ip->type[cur];
-  unsigned status = 0;
+  const Pot<R>* pot = (const Pot<R>*)Ip->pot;
+  const bool flow = o_rho1 || o_rho2 || o_ux || o_uy;
   for (long long node = blockIdx.x * (long long)blockDim.x + threadIdx.x; node < N;
        node += (long long)gridDim.x * blockDim.x) {
     const uint8_t t = T[node] & T_MASK;
-    o_type[node] = t;
+    if (o_type) o_type[node] = t;
     double r1o = 0, r2o = 0, uxo = 0, uyo = 0;
-    const int x = int(node % P.nx), y = int(node / P.nx);
-    if (is_fluid(t)) {
+    const int y = node_row(P, (int)node), x = (int)node - y * P.nx;
+    if (flow && is_fluid(t)) {
       R f1[9], f2[9];
 #pragma unroll
       for (int a = 0; a < 9; ++a) {
@@ -75,55 +111,42 @@ __global__ void k_fields(const DevInst* __restrict__ Ip, double* __restrict__ o_
       const R j1y = (f1[2] - f1[4]) + (f1[5] - f1[8]) + (f1[6] - f1[7]);
       const R j2x = (f2[1] - f2[3]) + (f2[5] - f2[6]) + (f2[8] - f2[7]);
       const R j2y = (f2[2] - f2[4]) + (f2[5] - f2[8]) + (f2[6] - f2[7]);
-      R psc, p1c, p2c;
-      potentials<R>(P, rho1, rho2, psc, p1c, p2c, status);
-      // neighbours' potentials (live ones) first, then the stencils with a
-      // solid neighbour replaced by its mirror image across the wall, as in
-      // the bulk kernel
-      R nps[9], nq1[9], nq2[9];
-      bool nlv[9];
-#pragma unroll
-      for (int a = 1; a < 9; ++a) {
-        int xn, yn;
-        const bool in = nbr(P, x, y, EX(a), EY(a), xn, yn);
-        const long long nn = (long long)yn * P.nx + xn;
-        const uint8_t tn = in ? (T[nn] & T_MASK) : T_WALL;
-        nps[a] = psc;
-        nq1[a] = p1c;
-        nq2[a] = p2c;
-        nlv[a] = is_live(tn);
-        if (nlv[a]) {
-          R a1, a2;
-          if (is_fluid(tn)) {
-            a1 = fshift<R>(P, 0, tn) + density_shifted<R>(F, 0, (int)nn);
-            a2 = fshift<R>(P, 1, tn) + density_shifted<R>(F, 1, (int)nn);
-          } else {
-            double u, v;
-            const R theta = theta_of<R>(Ip);
-            reservoir_rho(P, tn, step, tn == T_OUTLET && outlet_up_liquid<R, TF>(P, T, F, (int)N, (int)nn, theta), u, v);
-            a1 = R(u);
-            a2 = R(v);
-          }
-          potentials<R>(P, a1, a2, nps[a], nq1[a], nq2[a], status);
-        }
-      }
-      nps[0] = psc;
-      nq1[0] = p1c;
-      nq2[0] = p2c;
-      nlv[0] = true;
-      const Stencils<R> S = force_stencils<R>(nps, nq1, nq2, nlv);
-      const R spx = S.psx, spy = S.psy, s2x = S.p2x, s2y = S.p2y, s1x = S.p1x, s1y = S.p1y, ssx = S.ssx,
-              ssy = S.ssy;
-      const R G11 = rp<R>(P).G11, G12 = rp<R>(P).G12, G21 = rp<R>(P).G21, w1 = rp<R>(P).w_adh[0], w2 = rp<R>(P).w_adh[1];
-      const R F1x = force1<R>(G11, G12, w1, psc, p1c, spx, s2x, ssx, rho1, rp<R>(P).gx);
-      const R F1y = force1<R>(G11, G12, w1, psc, p1c, spy, s2y, ssy, rho1, rp<R>(P).gy);
-      const R F2x = force2<R>(G21, w2, p2c, s1x, ssx, rho2, rp<R>(P).gx);
-      const R F2y = force2<R>(G21, w2, p2c, s1y, ssy, rho2, rp<R>(P).gy);
-      const R rrt = rrcp<R>(radd<R>(rho1, rho2));
       r1o = double(rho1);
       r2o = double(rho2);
-      uxo = double(u_phys<R>(j1x, j2x, F1x, F2x, rrt));
-      uyo = double(u_phys<R>(j1y, j2y, F1y, F2y, rrt));
+      if (o_ux || o_uy) {
+        const Pot<R> own = ld_pot(pot + node);
+        const R psc = own.ps, p1c = own.p1, p2c = own.p2;
+        // neighbours' potentials (live ones) first, then the stencils with a
+        // solid neighbour replaced by its mirror image across the wall
+        R nps[9], nq1[9], nq2[9];
+        bool nlv[9];
+#pragma unroll
+        for (int a = 1; a < 9; ++a) {
+          int xn, yn;
+          const bool in = nbr(P, x, y, EX(a), EY(a), xn, yn);
+          const long long nn = (long long)yn * P.nx + xn;
+          nlv[a] = in && is_live(T[nn] & T_MASK);
+          const Pot<R> q = nlv[a] ? ld_pot(pot + nn) : own;
+          nps[a] = q.ps;
+          nq1[a] = q.p1;
+          nq2[a] = q.p2;
+        }
+        nps[0] = psc;
+        nq1[0] = p1c;
+        nq2[0] = p2c;
+        nlv[0] = true;
+        const Stencils<R> S = force_stencils<R>(nps, nq1, nq2, nlv);
+        const R spx = S.psx, spy = S.psy, s2x = S.p2x, s2y = S.p2y, s1x = S.p1x, s1y = S.p1y, ssx = S.ssx,
+                ssy = S.ssy;
+        const R G11 = rp<R>(P).G11, G12 = rp<R>(P).G12, G21 = rp<R>(P).G21, w1 = rp<R>(P).w_adh[0], w2 = rp<R>(P).w_adh[1];
+        const R F1x = force1<R>(G11, G12, w1, psc, p1c, spx, s2x, ssx, rho1, rp<R>(P).gx);
+        const R F1y = force1<R>(G11, G12, w1, psc, p1c, spy, s2y, ssy, rho1, rp<R>(P).gy);
+        const R F2x = force2<R>(G21, w2, p2c, s1x, ssx, rho2, rp<R>(P).gx);
+        const R F2y = force2<R>(G21, w2, p2c, s1y, ssy, rho2, rp<R>(P).gy);
+        const R rrt = rrcp<R>(radd<R>(rho1, rho2));
+        uxo = double(u_phys<R>(j1x, j2x, F1x, F2x, rrt));
+        uyo = double(u_phys<R>(j1y, j2y, F1y, F2y, rrt));
+      }
     }
     if (o_rho1) o_rho1[node] = r1o;
     if (o_rho2) o_rho2[node] = r2o;
@@ -234,12 +257,18 @@ __device__ __forceinline__ void budget_reduce(const double* __restrict__ part, i
     for (int i = 0; i < NBUD; ++i) v[i] = sh[i][0];
 }
 
-static __global__ void __launch_bounds__(BUD_FINAL_THREADS) k_budget_final(const double* __restrict__ part,
+// ... then the step count and the status word, so that the host fetches all three at once.
+static __global__ void __launch_bounds__(BUD_FINAL_THREADS) k_budget_final(const DevInst* __restrict__ Ip,
+                                                                          const double* __restrict__ part,
                                                                           int nblocks, double* __restrict__ out) {
   double v[NBUD];
   budget_reduce(part, nblocks, v);
-  if (threadIdx.x == 0)
+  if (threadIdx.x == 0) {
     for (int i = 0; i < NBUD; ++i) out[i] = v[i];
+    unsigned long long* w = (unsigned long long*)(out + NBUD);
+    w[0] = Ip->scal[S_STEP];
+    w[1] = Ip->scal[S_STATUS];
+  }
 }
 
 }  // namespace pslbm

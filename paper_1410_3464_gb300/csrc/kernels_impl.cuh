@@ -65,14 +65,15 @@ void init_l(cudaStream_t s, DevInst* I, const uint8_t* m, const double* r1, cons
 template <int NS>
 void fields_l(cudaStream_t s, const DevInst* I, long long N, double* r1, double* r2, double* ux, double* uy,
               double* c, uint8_t* t) {
-  long long blocks = (N + 255) / 256;
+  long long blocks = (N + FIELD_THREADS - 1) / FIELD_THREADS;
   if (blocks > 65536) blocks = 65536;
-  k_fields<KTF, KTG, KR, NS><<<(int)blocks, 256, 0, s>>>(I, r1, r2, ux, uy, c, t);
+  if (ux || uy) k_fields_pot<KTF, KR><<<(int)blocks, FIELD_THREADS, 0, s>>>(I);
+  k_fields<KTF, KTG, KR, NS><<<(int)blocks, FIELD_THREADS, 0, s>>>(I, r1, r2, ux, uy, c, t);
 }
 template <int NS>
 void budget_l(cudaStream_t s, const DevInst* I, double* part, double* out) {
   k_budget_partial<KTF, KTG, KR, NS><<<BUD_BLOCKS, BUD_THREADS, 0, s>>>(I, part);
-  k_budget_final<<<1, BUD_FINAL_THREADS, 0, s>>>(part, BUD_BLOCKS, out);
+  k_budget_final<<<1, BUD_FINAL_THREADS, 0, s>>>(I, part, BUD_BLOCKS, out);
 }
 
 template <int NS>

@@ -11,6 +11,7 @@ struct Launchers {
   void (*amend)(cudaStream_t, int ninst, const DevInst*);
   void (*init)(cudaStream_t, DevInst*, const uint8_t*, const double*, const double*, const double*, long long N);
   void (*fields)(cudaStream_t, const DevInst*, long long N, double*, double*, double*, double*, double*, uint8_t*);
+  // out: NBUD doubles, then the step count and the status (64-bit words)
   void (*budget)(cudaStream_t, const DevInst*, double* part, double* out);
   // potentials and collide-stream kernels, a warp per work entry: parts
   // of the fluid list (the first nstream entries of one simulation), then chunks

@@ -655,14 +655,18 @@ bool staging_open(const pslbm_params* p) {
 int shown_shape(const Stepper& st) { return st.fix_shape >= 0 ? st.fix_shape : 1; }
 int shown_staging(const Stepper& st) { return st.fix_staged >= 0 ? st.fix_staged : 0; }
 
-pslbm_status device_status(pslbm_t h) {
-  unsigned long long st = 0;
-  CK(h, cudaMemcpyAsync(&st, h->h.scal + S_STATUS, sizeof st, cudaMemcpyDeviceToHost, lib_stream()));
-  CK(h, cudaStreamSynchronize(lib_stream()));
+pslbm_status status_of(pslbm_t h, unsigned long long st) {
   if (st & ST_NONFINITE) return fail(h, PSLBM_ERR_NONFINITE, "non-finite density on the device");
   if (st & ST_EOS) return fail(h, PSLBM_ERR_EOS_DOMAIN, "Eq. 13 square-root argument negative (rho_1 outside the EOS domain)");
   if (st & ST_TIMEOUT) return fail(h, PSLBM_ERR_TIMEOUT, "a bounded wait for staged populations gave up");
   return PSLBM_OK;
+}
+
+pslbm_status device_status(pslbm_t h) {
+  unsigned long long st = 0;
+  CK(h, cudaMemcpyAsync(&st, h->h.scal + S_STATUS, sizeof st, cudaMemcpyDeviceToHost, lib_stream()));
+  CK(h, cudaStreamSynchronize(lib_stream()));
+  return status_of(h, st);
 }
 
 }  // namespace
@@ -706,7 +710,7 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
   std::vector<int> reslist;
   {
     // one device allocation holds the instance's whole state, each part on a
-    // 256-byte boundary (TMA wants 16-byte aligned bases); the initial
+    // 256-byte boundary; the initial
     // threshold's budget partial sums are the last part
     const size_t NP = (size_t)(N + CELL - 1) / CELL * CELL;   // whole cells
     const size_t fb = NP * 18 * fsize(p->precision), gb = NP * 5 * ns * gsize(p->precision);
@@ -718,7 +722,7 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     const size_t sizes[] = {fb, fb, gb, gb, (size_t)N, (size_t)N, (size_t)N * 2 * sizeof(double), (size_t)N,
                             (size_t)N * sizeof(double), (size_t)N * 2 * sizeof(int), (size_t)N * sizeof(int),
                             (size_t)((N + 31) / 32) * 2 * sizeof(unsigned), S_NSCAL * sizeof(unsigned long long),
-                            sizeof(DevInst), (size_t)(BUD_BLOCKS + 1) * NBUD * sizeof(double), (size_t)N * 4 * fsize(p->precision),
+                            sizeof(DevInst), (size_t)((BUD_BLOCKS + 1) * NBUD + 2) * sizeof(double), (size_t)N * 4 * fsize(p->precision),
                             (size_t)N, reslist.size() * sizeof(int), (size_t)N * 2 * sizeof(int)};
     constexpr int NPARTS = sizeof(sizes) / sizeof(sizes[0]);
     size_t offs[NPARTS], total = 0;
@@ -889,7 +893,7 @@ pslbm_status pslbm_estimate_device_bytes(const pslbm_params* p, uint64_t* bytes)
   const uint64_t pops = 2 * 18 * fsize(p->precision) + 2 * 5 * (uint64_t)p->n_species * gsize(p->precision);
   const uint64_t res = 2 * ((uint64_t)p->nx + (uint64_t)p->ny) * sizeof(int);
   *bytes = N * per + (cells - N) * pops + bits + res + sizeof(DevInst) + S_NSCAL * 8 +
-           (uint64_t)(BUD_BLOCKS + 1) * NBUD * sizeof(double) + 19 * 256;
+           (uint64_t)((BUD_BLOCKS + 1) * NBUD + 2) * sizeof(double) + 19 * 256;
   return PSLBM_OK;
 }
 
@@ -977,8 +981,10 @@ pslbm_status pslbm_read_fields(pslbm_t h, uint32_t fields, void* const* out) {
   const long long N = h->N;
   const int ns = h->ns;
   cudaStream_t s = lib_stream();
-  // scratch: rho1, rho2, ux, uy (N each), conc (ns N), type (N bytes), budget partials
-  const size_t need = (size_t)N * (4 + ns) * sizeof(double) + (size_t)N + (BUD_BLOCKS + 1) * NBUD * sizeof(double) + 64;
+  // scratch: rho1, rho2, ux, uy (N each), conc (ns N), type (N bytes), budget
+  // partials, budget, step count and status
+  const size_t at_part = ((size_t)N * (4 + ns) * sizeof(double) + (size_t)N + 15) / 16 * 16;
+  const size_t need = at_part + ((BUD_BLOCKS + 1) * NBUD + 2) * sizeof(double);
   if (h->rb_bytes < need) {
     if (h->rb) {
       cudaFree(h->rb);
@@ -999,47 +1005,68 @@ pslbm_status pslbm_read_fields(pslbm_t h, uint32_t fields, void* const* out) {
   double* ux = r2 + N;
   double* uy = ux + N;
   double* cc = uy + N;
-  double* part = cc + (size_t)N * ns;
+  uint8_t* ty = (uint8_t*)(cc + (size_t)N * ns);
+  double* part = (double*)((char*)h->rb + at_part);
   double* bud = part + BUD_BLOCKS * NBUD;
-  uint8_t* ty = (uint8_t*)(bud + NBUD);
-  h->L->fields(s, h->d, N, r1, r2, ux, uy, ns ? cc : nullptr, ty);
-  CK(h, cudaGetLastError());
+  if (fields & 0x3F) {
+    auto want = [&](uint32_t f, auto* p) { return fields & f ? p : nullptr; };
+    h->L->fields(s, h->d, N, want(PSLBM_F_RHO1, r1), want(PSLBM_F_RHO2, r2), want(PSLBM_F_UX, ux), want(PSLBM_F_UY, uy),
+                 ns ? want(PSLBM_F_CONC, cc) : nullptr, want(PSLBM_F_TYPE, ty));
+    CK(h, cudaGetLastError());
+  }
   if (fields & PSLBM_F_BUDGET) {
     h->L->budget(s, h->d, part, bud);
     CK(h, cudaGetLastError());
   }
-  int i = 0;
-  auto cp = [&](void* dst, const void* src, size_t b) {
-    return cudaMemcpyAsync(dst, src, b, cudaMemcpyDeviceToHost, s);
+  // a copy that continues the one before on both sides joins it: a caller whose
+  // arrays lie one behind the other (rho1 .. type) pays for one
+  char* to = nullptr;
+  const char* from = nullptr;
+  size_t len = 0;
+  cudaError_t ce = cudaSuccess;
+  auto flush = [&] {
+    if (len && ce == cudaSuccess) ce = cudaMemcpyAsync(to, from, len, cudaMemcpyDeviceToHost, s);
+    len = 0;
   };
-  if (fields & PSLBM_F_RHO1) CK(h, cp(out[i++], r1, N * 8));
-  if (fields & PSLBM_F_RHO2) CK(h, cp(out[i++], r2, N * 8));
-  if (fields & PSLBM_F_UX) CK(h, cp(out[i++], ux, N * 8));
-  if (fields & PSLBM_F_UY) CK(h, cp(out[i++], uy, N * 8));
+  auto cp = [&](void* dst, const void* src, size_t b) {
+    if (len && (char*)dst == to + len && (const char*)src == from + len) {
+      len += b;
+      return;
+    }
+    flush();
+    to = (char*)dst;
+    from = (const char*)src;
+    len = b;
+  };
+  int i = 0;
+  if (fields & PSLBM_F_RHO1) cp(out[i++], r1, N * 8);
+  if (fields & PSLBM_F_RHO2) cp(out[i++], r2, N * 8);
+  if (fields & PSLBM_F_UX) cp(out[i++], ux, N * 8);
+  if (fields & PSLBM_F_UY) cp(out[i++], uy, N * 8);
   if (fields & PSLBM_F_CONC) {
-    if (ns) CK(h, cp(out[i], cc, (size_t)N * ns * 8));
+    if (ns) cp(out[i], cc, (size_t)N * ns * 8);
     ++i;
   }
-  if (fields & PSLBM_F_TYPE) CK(h, cp(out[i++], ty, N));
-  if (fields & PSLBM_F_VOL) CK(h, cp(out[i++], h->h.V, (size_t)N * 2 * 8));
-  double budget_host[NBUD];
-  unsigned long long stepc = 0;
-  if (fields & PSLBM_F_BUDGET) {
-    CK(h, cp(budget_host, bud, sizeof budget_host));
-    CK(h, cp(&stepc, h->h.scal + S_STEP, sizeof stepc));
-  }
+  if (fields & PSLBM_F_TYPE) cp(out[i++], ty, N);
+  if (fields & PSLBM_F_VOL) cp(out[i++], h->h.V, (size_t)N * 2 * 8);
+  flush();
+  CK(h, ce);
+  if (!(fields & PSLBM_F_BUDGET)) return device_status(h);
+  struct {
+    double v[NBUD];
+    unsigned long long step, status;
+  } b;
+  CK(h, cudaMemcpyAsync(&b, bud, sizeof b, cudaMemcpyDeviceToHost, s));
   CK(h, cudaStreamSynchronize(s));
-  if (fields & PSLBM_F_BUDGET) {
-    double* o = (double*)out[i++];
-    o[0] = budget_host[0] > -INFINITY ? budget_host[0] : 0.0;
-    o[1] = budget_host[1];
-    o[2] = budget_host[2];
-    for (int k = 0; k < ns; ++k) o[3 + k] = budget_host[3 + k];
-    o[3 + ns] = budget_host[3 + MAXS];
-    o[4 + ns] = budget_host[4 + MAXS];
-    o[5 + ns] = (double)stepc;
-  }
-  return device_status(h);
+  double* o = (double*)out[i++];
+  o[0] = b.v[0] > -INFINITY ? b.v[0] : 0.0;
+  o[1] = b.v[1];
+  o[2] = b.v[2];
+  for (int k = 0; k < ns; ++k) o[3 + k] = b.v[3 + k];
+  o[3 + ns] = b.v[3 + MAXS];
+  o[4 + ns] = b.v[4 + MAXS];
+  o[5 + ns] = (double)b.step;
+  return status_of(h, b.status);
 }
 
 pslbm_status pslbm_destroy(pslbm_t h) {

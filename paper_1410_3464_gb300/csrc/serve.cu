@@ -7,8 +7,7 @@
 //      of the resident simulations stays within the HBM budget (and below the
 //      resident cap);
 //   2. when the resident set changed, re-pack one batch per species count (one
-//      tile list and one launch per kernel for all its members), with the
-//      kernel variant the first batch of that species count chose by timing;
+//      list of work and one launch per kernel for all its members);
 //   3. advance every batch by `chunk_steps` steps; members whose step budget
 //      ends inside the chunk are frozen on the device at their budget;
 //   4. retire requests that reached their budget or whose total solid volume
@@ -98,12 +97,17 @@ void retire(pslbm_server_t s, Request* r, const std::vector<double>& b) {
     const int ns = r->p.n_species;
     const uint32_t sel[] = {PSLBM_F_RHO1, PSLBM_F_RHO2, PSLBM_F_UX, PSLBM_F_UY, PSLBM_F_CONC, PSLBM_F_TYPE, PSLBM_F_VOL};
     const size_t sz[] = {N * 8, N * 8, N * 8, N * 8, N * ns * 8, N, 2 * N * 8};
+    std::vector<unsigned char> buf[7];
+    void* ptrs[7];
+    uint32_t all = 0;
     for (int i = 0; i < 7; ++i) {
-      std::vector<unsigned char> buf(sz[i] ? sz[i] : 1);
-      void* ptrs[1] = {buf.data()};
-      if (sz[i] == 0) continue;
-      if (pslbm_read_fields(r->h, sel[i], ptrs) == PSLBM_OK) r->fields[sel[i]] = std::move(buf);
+      buf[i].resize(sz[i]);
+      ptrs[i] = buf[i].data();
+      all |= sel[i];
     }
+    if (pslbm_read_fields(r->h, all, ptrs) == PSLBM_OK)
+      for (int i = 0; i < 7; ++i)
+        if (sz[i]) r->fields[sel[i]] = std::move(buf[i]);
   }
   pslbm_destroy(r->h);
   r->h = nullptr;

@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from collections import deque
 
 import numpy as np
 
@@ -173,11 +174,24 @@ def set_stream(stream_ptr):
     _check(load().pslbm_set_stream(stream_ptr))
 
 
+class _Recycled:
+    """Owner of an array's memory; gives it to `spare` when no view of it is left."""
+
+    def __init__(self, mem, spare):
+        self.mem, self.spare = mem, spare
+        self.__array_interface__ = mem.__array_interface__
+
+    def __del__(self):
+        self.spare.append(self.mem)
+
+
 class Simulation:
     """One simulation handle (pslbm_create ... pslbm_destroy)."""
 
     def __init__(self, mask, params, rho1, rho2, conc=None, vol=None, precision=None):
         lib = load()
+        self._reads = {}        # read(): layout per selection of fields
+        self._spare = {}        # per field of read(): memory that waits for the next one
         d = dict(params)
         if precision is not None:
             d["precision"] = precision
@@ -219,19 +233,18 @@ class Simulation:
         return tx.value, ty.value, bool(tu.value)
 
     def set_staging(self, mode):
-        """-1: choose by timing, 0: plain-load bulk kernel, 1: TMA-staged,
-        2: TMA-staged with one stage (three blocks per SM)."""
+        """-1, 0, 1 or 2: checked and reported, without effect on results or speed."""
         _check(load().pslbm_set_staging(self.h, int(mode)), self.h)
 
     def staging(self):
-        """(staging in use 0/1/2, staged kernels available)."""
+        """(staging asked for 0/1/2, whether 1 and 2 are open)."""
         sg, av = C.c_int32(), C.c_int32()
         _check(load().pslbm_get_staging(self.h, C.byref(sg), C.byref(av)), self.h)
         return sg.value, bool(av.value)
 
     def monitor(self):
         """(steps taken, maximum rho_1 found by the last step, status bits):
-        a 64-byte read, no kernel."""
+        an 80-byte read, no kernel."""
         n, m, st = C.c_int64(), C.c_double(), C.c_uint32()
         _check(load().pslbm_monitor(self.h, C.byref(n), C.byref(m), C.byref(st)), self.h)
         return n.value, m.value, st.value
@@ -250,30 +263,62 @@ class Simulation:
         return int(b.value)
 
     def read(self, fields=F_RHO1 | F_RHO2 | F_UX | F_UY | F_CONC | F_TYPE | F_VOL | F_BUDGET):
-        """Read the selected fields into new numpy arrays (dict by name)."""
-        N = self.nx * self.ny
-        shape = (self.ny, self.nx)
-        spec = [(F_RHO1, "rho1", np.float64, shape), (F_RHO2, "rho2", np.float64, shape),
-                (F_UX, "ux", np.float64, shape), (F_UY, "uy", np.float64, shape),
-                (F_CONC, "conc", np.float64, (self.ns,) + shape), (F_TYPE, "type", np.uint8, shape),
-                (F_VOL, "vol", np.float64, (2,) + shape), (F_BUDGET, "budget", np.float64, (6 + self.ns,))]
-        out = {}
-        ptrs = []
-        for bit, name, dt, shp in spec:
-            if fields & bit:
-                a = np.zeros(max(1, int(np.prod(shp))), dtype=dt)
-                out[name] = a
-                ptrs.append(a.ctypes.data_as(C.c_void_p))
-        arr = (C.c_void_p * max(1, len(ptrs)))(*ptrs)
+        """Read the selected fields into new numpy arrays (dict by name).  Of arrays
+        that the caller has let go of, the memory of two per field waits for the
+        next read, until close()."""
+        plan = self._reads.get(fields)
+        if plan is None:
+            plan = self._reads[fields] = self._read_plan(fields)
+        spec, at, total = plan
+        if total <= 1 << 20:
+            # one behind the other in one allocation: the library copies what adjoins at once
+            mem = np.empty(max(1, total), np.uint8)
+            raw = [mem[o:o + n] for o, (_, _, _, n) in zip(at, spec)]
+            base = mem.ctypes.data
+            arr = (C.c_void_p * max(1, len(at)))(*[base + o for o in at])
+        else:
+            raw = [self._memory(name, n) for name, _, _, n in spec]
+            arr = (C.c_void_p * len(raw))(*[a.ctypes.data for a in raw])
         _check(load().pslbm_read_fields(self.h, int(fields), arr), self.h)
-        res = {}
-        for bit, name, dt, shp in spec:
-            if fields & bit:
-                res[name] = out[name][: int(np.prod(shp))].reshape(shp)
+        res = {name: a.view(dt).reshape(shp) for (name, dt, shp, _), a in zip(spec, raw)}
         if "vol" in res:
             res["vol_d"], res["vol_f"] = res["vol"][0], res["vol"][1]
-        del N
         return res
+
+    def _read_plan(self, fields):
+        """(name, type, shape, bytes) of the selected fields, their offsets in one
+        allocation (eight-byte items on eight-byte offsets) and its size."""
+        n = self.nx * self.ny
+        shape = (self.ny, self.nx)
+        spec = [(F_RHO1, "rho1", np.float64, shape, 8 * n), (F_RHO2, "rho2", np.float64, shape, 8 * n),
+                (F_UX, "ux", np.float64, shape, 8 * n), (F_UY, "uy", np.float64, shape, 8 * n),
+                (F_CONC, "conc", np.float64, (self.ns,) + shape, 8 * n * self.ns), (F_TYPE, "type", np.uint8, shape, n),
+                (F_VOL, "vol", np.float64, (2,) + shape, 16 * n),
+                (F_BUDGET, "budget", np.float64, (6 + self.ns,), 8 * (6 + self.ns))]
+        spec = [s[1:] for s in spec if fields & s[0]]
+        at, end = [], 0
+        for _, dt, _, size in spec:
+            at.append(end if dt is np.uint8 else (end + 7) // 8 * 8)
+            end = at[-1] + size
+        return spec, at, end
+
+    def _memory(self, name, n):
+        """n bytes for an array of read(): what an earlier array of that name has
+        left, else fresh pages.  Up to 32 MiB those are touched here, because the
+        copy from the device faults them in more slowly (all fields of 1024x512, 38
+        MB: 21 to 32 ms, touched 1.3 to 2.6, used before 0.43); above, the copy is
+        the quicker way (4096x2048, 612 MB: 27 ms, touched 31 to 49, used before
+        4.3)."""
+        spare = self._spare.setdefault(name, deque(maxlen=2))
+        try:
+            mem = spare.pop()
+        except IndexError:
+            if n <= 1 << 25:
+                mem = np.empty(n, np.uint8)
+                mem[::4096] = 0
+            else:
+                mem = np.zeros(n, np.uint8)
+        return np.asarray(_Recycled(mem, spare))
 
     def budget_device_noalloc(self, out_device_ptr):
         """Write the budget (6 + n_species doubles) to a caller-owned device
@@ -284,6 +329,7 @@ class Simulation:
         if getattr(self, "h", None):
             load().pslbm_destroy(self.h)
             self.h = None
+            self._spare = {}
 
     def __del__(self):
         try:
@@ -299,7 +345,7 @@ class Simulation:
 
 
 class Batch:
-    """Several simulations stepped together over one packed tile list."""
+    """Several simulations stepped together over one list of work."""
 
     def __init__(self, sims, tile_x=0, tile_y=0):
         lib = load()
