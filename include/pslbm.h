@@ -48,7 +48,7 @@ typedef enum {
     PSLBM_ERR_CUDA = -3,        /* CUDA runtime error (message in pslbm_last_error) */
     PSLBM_ERR_NONFINITE = -4,   /* a density became NaN/Inf on the device */
     PSLBM_ERR_EOS_DOMAIN = -5,  /* Eq. 13 square-root argument negative (rho_1 out of the EOS domain) */
-    PSLBM_ERR_TIMEOUT = -6,     /* a bounded device-side wait gave up */
+    PSLBM_ERR_TIMEOUT = -6,     /* a bounded device-side wait gave up (no kernel waits at present) */
     PSLBM_ERR_STATE = -7,       /* call not valid in the handle's current state */
     PSLBM_ERR_NODEVICE = -8     /* no CUDA device, or not an sm_103 device */
 } pslbm_status;
@@ -269,7 +269,7 @@ pslbm_status pslbm_budget_device_noalloc(pslbm_t h, double* out);
 
 /* ---------------------------------------------------------------- batching
  * A batch steps several simulations (same precision and species count) in
- * one launch per kernel over a packed list of tiles of all members.  The
+ * one launch per kernel over a packed list of work of all members.  The
  * members stay valid handles; they must not be stepped on their own while
  * the batch exists.  tile_x, tile_y choose the tile shape (16x16, 32x8,
  * 16x32 or 32x16, as for pslbm_set_tile_shape; 0, 0: the default). */

@@ -17,6 +17,7 @@ constexpr uint8_t T_NEW = 0x40;      // flag set by the amendment kernel: solid 
 constexpr uint8_t T_VANISH = 0x80;   // flag: liquid -> solid this step
 
 constexpr int NTHREADS = 256;          // threads per block of the VOP and amendment kernels
+constexpr int FUSE_FACE = NTHREADS;    // longest mineral list that k_vop_amend takes
 // Tile shapes a caller may ask for (nodes per tile: 256 or 512).
 constexpr int NSHAPES = 4;
 constexpr int SHAPE_TX[NSHAPES] = {16, 32, 16, 32};
@@ -36,7 +37,7 @@ enum {
   S_NFACE = 9,     // entries of the list of minerals facing fluid
   S_NSCAL = 10
 };
-enum { ST_NONFINITE = 1, ST_EOS = 2, ST_EVOVERFLOW = 4, ST_TIMEOUT = 8 };
+enum { ST_NONFINITE = 1, ST_EOS = 2, ST_EVOVERFLOW = 4 };
 
 // Budget reduction: [max rho1, sum rho1, sum rho2, sum C_k (MAXS), sum V_D, sum V_F].
 constexpr int NBUD = 5 + MAXS;

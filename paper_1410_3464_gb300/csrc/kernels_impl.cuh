@@ -56,6 +56,11 @@ void amend_l(cudaStream_t s, int ninst, const DevInst* insts) {
   launch_step<const DevInst*>(s, ninst, NTHREADS, k_amend<KTF, KTG, KR, NS>, insts);
 }
 template <int NS>
+void vop_amend_l(cudaStream_t s, int ninst, const DevInst* insts) {
+  if (ninst <= 0) return;
+  launch_step<const DevInst*>(s, ninst, NTHREADS, k_vop_amend<KTF, KTG, KR, NS>, insts);
+}
+template <int NS>
 void init_l(cudaStream_t s, DevInst* I, const uint8_t* m, const double* r1, const double* r2, const double* c,
             long long N) {
   long long blocks = (N + 255) / 256;
@@ -83,6 +88,7 @@ constexpr Launchers make() {
   l.move = &move_l<NS>;
   l.vop = &vop_l<NS>;
   l.amend = &amend_l<NS>;
+  l.vop_amend = &vop_amend_l<NS>;
   l.init = &init_l<NS>;
   l.fields = &fields_l<NS>;
   l.budget = &budget_l<NS>;

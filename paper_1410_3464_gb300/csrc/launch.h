@@ -9,6 +9,8 @@ struct Launchers {
   // work: the VOP chunks of a batch (null for one simulation); nwork: their number
   void (*vop)(cudaStream_t, const DevInst*, const Work* work, int nwork);
   void (*amend)(cudaStream_t, int ninst, const DevInst*);
+  // both in one launch, a block an instance
+  void (*vop_amend)(cudaStream_t, int ninst, const DevInst*);
   void (*init)(cudaStream_t, DevInst*, const uint8_t*, const double*, const double*, const double*, long long N);
   void (*fields)(cudaStream_t, const DevInst*, long long N, double*, double*, double*, double*, double*, uint8_t*);
   // out: NBUD doubles, then the step count and the status (64-bit words)

@@ -110,7 +110,7 @@ namespace {
 pslbm_status fail(pslbm_t h, pslbm_status s, const std::string& msg) {
   if (h) {
     h->err = msg;
-    if (s == PSLBM_ERR_CUDA || s == PSLBM_ERR_NONFINITE || s == PSLBM_ERR_EOS_DOMAIN || s == PSLBM_ERR_TIMEOUT)
+    if (s == PSLBM_ERR_CUDA || s == PSLBM_ERR_NONFINITE || s == PSLBM_ERR_EOS_DOMAIN)
       h->sticky = s;
   } else {
     std::lock_guard<std::mutex> lk(g_mu);
@@ -490,8 +490,14 @@ void enqueue_stream(cudaStream_t s, const Stepper& st) {
 
 // Enqueue the kernels of n steps.
 void enqueue_steps(cudaStream_t s, const Stepper& st, int64_t n) {
+  // every list within one block: VOP and amendment in one launch (k_vop_amend)
+  const bool fused = *std::max_element(st.nface.begin(), st.nface.end()) <= FUSE_FACE;
   for (int64_t i = 0; i < n; ++i) {
     enqueue_stream(s, st);
+    if (fused) {
+      st.L->vop_amend(s, st.ninst, st.d);
+      continue;
+    }
     st.L->vop(s, st.d, st.work ? st.work + st.nwork : nullptr, st.nvop);
     st.L->amend(s, st.ninst, st.d);
   }
@@ -658,7 +664,6 @@ int shown_staging(const Stepper& st) { return st.fix_staged >= 0 ? st.fix_staged
 pslbm_status status_of(pslbm_t h, unsigned long long st) {
   if (st & ST_NONFINITE) return fail(h, PSLBM_ERR_NONFINITE, "non-finite density on the device");
   if (st & ST_EOS) return fail(h, PSLBM_ERR_EOS_DOMAIN, "Eq. 13 square-root argument negative (rho_1 outside the EOS domain)");
-  if (st & ST_TIMEOUT) return fail(h, PSLBM_ERR_TIMEOUT, "a bounded wait for staged populations gave up");
   return PSLBM_OK;
 }
 
@@ -941,7 +946,6 @@ pslbm_status pslbm_monitor(pslbm_t h, int64_t* steps, double* max_rho1, uint32_t
   if (sc[S_STATUS] & ST_NONFINITE) return fail(h, PSLBM_ERR_NONFINITE, "non-finite density on the device");
   if (sc[S_STATUS] & ST_EOS)
     return fail(h, PSLBM_ERR_EOS_DOMAIN, "Eq. 13 square-root argument negative (rho_1 outside the EOS domain)");
-  if (sc[S_STATUS] & ST_TIMEOUT) return fail(h, PSLBM_ERR_TIMEOUT, "a bounded wait for staged populations gave up");
   return PSLBM_OK;
 }
 

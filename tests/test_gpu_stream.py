@@ -151,3 +151,27 @@ def test_reads_are_independent_arrays(pslbm, nx, ny):
     for a, b in zip(kept, want):
         np.testing.assert_array_equal(a, b)
     assert not np.array_equal(want[0], want[1])
+
+
+@pytest.mark.parametrize("precision", [0, 1, 3])
+@pytest.mark.parametrize("nx,ny", [(45, 20), (45, 60)])
+def test_one_launch_for_vop_and_amendment(pslbm, nx, ny, precision):
+    """step() takes VOP and amendment in one launch while every list of reactive
+    minerals was at most 256 long (45x20 has 101, 45x60 326);
+    profile_step() always takes two.  Dissolution, overflow and list growth on the way."""
+    sc = growing(nx, ny)
+    p = sc["params"]
+    p.update(G11=0.0, G12=0.0, G21=0.0, idx_F=2, idx_E=-1, k4=0.02, Vbar_F=0.2, V_split=2.0, seed=7)
+    full = sc["mask"] == 2
+    full[:, : nx // 2] = False
+    sc["mask"][full] = 3
+    sc["vol"][0][full] = 0.0
+    sc["vol"][1][full] = np.random.default_rng(2).uniform(1.99, 1.999, full.sum())
+    ref = state(pslbm, sc, 30, precision)
+    assert (ref["type"] == 3).sum() > full.sum(), "no overflow"
+    assert (ref["type"] == 2).sum() < (sc["mask"] == 2).sum(), "no node dissolved"
+    with pslbm.Simulation(sc["mask"], p, sc["rho1"], sc["rho2"], sc["conc"], sc["vol"], precision=precision) as sim:
+        sim.profile_step(30)
+        got = sim.read()
+    for name in ref:
+        np.testing.assert_array_equal(got[name], ref[name], err_msg=name)
