@@ -7,6 +7,7 @@ missing the binding raises instead of falling back to anything else.
 from __future__ import annotations
 
 import ctypes as C
+import mmap
 import os
 from collections import deque
 
@@ -174,6 +175,18 @@ def set_stream(stream_ptr):
     _check(load().pslbm_set_stream(stream_ptr))
 
 
+def _touched(mem):
+    """Write to every page of an array that a copy from the device is to fill.  A
+    page that is not there, or that the system has unmapped to see who uses it, is
+    quickly brought in by the host (1 to 2 us), slowly by the copy (12 to 15 us: all
+    fields of 1024x512, 38 MB, 21 to 32 ms into fresh pages, touched 1.3 to 2.6, into
+    used ones 0.43; 4096x2048, 612 MB, 27 to 35, 31 to 49 and 4.3, where untouched
+    used pages took up to 170)."""
+    mem[::mmap.PAGESIZE] = 0
+    mem[-1:] = 0
+    return mem
+
+
 class _Recycled:
     """Owner of an array's memory; gives it to `spare` when no view of it is left."""
 
@@ -272,7 +285,7 @@ class Simulation:
         spec, at, total = plan
         if total <= 1 << 20:
             # one behind the other in one allocation: the library copies what adjoins at once
-            mem = np.empty(max(1, total), np.uint8)
+            mem = _touched(np.empty(max(1, total), np.uint8))
             raw = [mem[o:o + n] for o, (_, _, _, n) in zip(at, spec)]
             base = mem.ctypes.data
             arr = (C.c_void_p * max(1, len(at)))(*[base + o for o in at])
@@ -304,21 +317,13 @@ class Simulation:
 
     def _memory(self, name, n):
         """n bytes for an array of read(): what an earlier array of that name has
-        left, else fresh pages.  Up to 32 MiB those are touched here, because the
-        copy from the device faults them in more slowly (all fields of 1024x512, 38
-        MB: 21 to 32 ms, touched 1.3 to 2.6, used before 0.43); above, the copy is
-        the quicker way (4096x2048, 612 MB: 27 ms, touched 31 to 49, used before
-        4.3)."""
+        left, else fresh pages."""
         spare = self._spare.setdefault(name, deque(maxlen=2))
         try:
             mem = spare.pop()
         except IndexError:
-            if n <= 1 << 25:
-                mem = np.empty(n, np.uint8)
-                mem[::4096] = 0
-            else:
-                mem = np.zeros(n, np.uint8)
-        return np.asarray(_Recycled(mem, spare))
+            mem = np.empty(n, np.uint8)
+        return np.asarray(_Recycled(_touched(mem), spare))
 
     def budget_device_noalloc(self, out_device_ptr):
         """Write the budget (6 + n_species doubles) to a caller-owned device
