@@ -14,7 +14,7 @@ Workloads (--workload):
                    (256 MiB write) before every timed step.
   large            one porous lattice 4096x2048 (seed 4).
 
-One step is one pass of the whole hot path: the fused bulk kernel, the VOP
+One step is one pass of the whole hot path: the two streaming kernels, the VOP
 kernel and the amendment kernel, over every node of every member.  Each timed
 step is bracketed per kernel by CUDA events on the library stream.  Prints one
 JSON line (rank 0).  Metric: MLUPS (all lattice nodes x steps / s, whole job).
@@ -55,9 +55,8 @@ WORKLOAD_NAMES = {
 }
 # oracle sample: members of the same trace with both sides at most this long
 SAMPLE_SIDE = 256
-STAGING_NAMES = {0: "plain loads", 1: "tma 2-stage", 2: "tma d2q9-box"}
 PROFILE_TAGS = {"batch": "batch256", "porous": "porous1024x512", "large": "porous4096x2048"}
-KERNEL_NAMES = {0: "k_bulk", 1: "k_bulk_tma<D2Q9+D2Q5 boxes>", 2: "k_bulk_tma<D2Q9 box, 3 blocks>"}
+KERNEL_NAME = "k_pot + k_move"
 
 
 def parse():
@@ -243,44 +242,35 @@ def algorithmic_bytes(types, ns, fs, gs):
     return n_fluid * 36 * fs + n_liq * 10 * ns * gs + 2 * types.size, n_fluid, n_liq
 
 
-def profile_traffic(workload, variant):
-    """DRAM bytes per bulk launch from the committed ncu summary of the same
-    kernel variant built from the same device sources (None otherwise)."""
+def profile_summary(workload, precision):
+    """The committed ncu summary of the streaming kernels on a workload, if it was
+    made from these device sources (None otherwise)."""
     from paper_1410_3464_gb300 import profile_case
-    path = os.path.join(ROOT, "profiles", f"k_bulk_{PROFILE_TAGS[workload]}_fp32.json")
+    path = os.path.join(ROOT, "profiles", f"step_{PROFILE_TAGS[workload]}_{precision}.json")
     if not os.path.exists(path):
         return None
     pj = json.load(open(path))
-    if pj.get("source_hash") != profile_case.kernel_source_hash():
-        return None
-    return pj.get("traffic_per_launch", {}).get(variant)
+    return pj if pj.get("source_hash") == profile_case.kernel_source_hash(precision) else None
 
 
 # GB300's nominal FP64 rate: 152 SMs x 2.07 GHz x 2 FP64 FMA per clock x 2 flops
 FP64_PEAK_TFLOPS = 152 * 2.07e9 * 2 * 2 / 1e12
 
 
-def fp64_roofline(workload, variant, kernel_ms):
-    """FP64-ALU roofline of the FP64 bulk kernel: the FP64 operations one launch
-    executes (ncu count from the committed summary of the same kernel variant
-    built from the same sources) per launch time, against the nominal FP64
-    rate.  None without a matching summary."""
-    from paper_1410_3464_gb300 import profile_case
-    path = os.path.join(ROOT, "profiles", f"k_bulk_{PROFILE_TAGS[workload]}_fp64.json")
-    if not os.path.exists(path):
+def fp64_roofline(workload, kernel_ms):
+    """FP64-ALU roofline of the streaming kernels: the FP64 operations a step
+    executes (ncu count of the committed summary) per step time, against the
+    nominal FP64 rate.  None without a matching summary."""
+    pj = profile_summary(workload, "fp64")
+    if pj is None:
         return None
-    pj = json.load(open(path))
-    if pj.get("source_hash") != profile_case.kernel_source_hash("fp64"):
-        return None
-    flops = pj.get("fp64_flops_per_launch", {}).get(variant)
-    if not flops:
-        return None
+    flops = pj["fp64_flops_per_step"]
     achieved = flops / (kernel_ms * 1e-3) / 1e12
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None, "kernel": "k_bulk<double>", "variant": variant,
+            "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None, "kernel": KERNEL_NAME,
             "flops_per_launch": flops, "kernel_ms": kernel_ms,
             "peak_source": "nominal GB300 FP64 rate (152 SMs x 2.07 GHz x 2 FMA/clock x 2 flops)",
-            "fp64_pipe_active_pct_ncu": pj.get("fp64_pipe_active_pct", {}).get(variant)}
+            "fp64_pipe_active_pct_ncu": pj.get("fp64_pipe_active_pct")}
 
 
 def ours_arm(args):
@@ -322,39 +312,9 @@ def ours_arm(args):
         return v, t
 
     sims = make_sims()
-    trials = None
-    if batch:
-        runner = pslbm.Batch(sims)
-        runner.step(90)              # variant autotuning (10 variants x 4 steps, twice) and a first warm-up
-    else:
-        # one lattice: each variant timed for 5 steps under the timed loop's own
-        # conditions (L2 flushed before every step for the 1024x512 lattice)
-        runner = sims[0]
-        trials = {}
-        stagings = [0, 1, 2] if runner.staging()[1] else [0]
-        with torch.cuda.stream(stream):
-            for shape in ((16, 16), (32, 8), (16, 32), (32, 16)):
-                for sg in stagings:
-                    if sg == 1 and shape[0] * shape[1] > 256:
-                        continue     # two nodes per thread: no staging 1
-                    runner.set_staging(-1)
-                    runner.set_tile_shape(*shape)
-                    runner.set_staging(sg)
-                    ts = []
-                    for _ in range(5):
-                        if flush is not None:
-                            flush.zero_()
-                        ts.append(runner.profile_step(1)[1])
-                    trials[(shape, sg)] = statistics.median(ts[1:])
-        torch.cuda.synchronize()
-        best = min(trials, key=trials.get)
-        runner.set_staging(-1)
-        runner.set_tile_shape(*best[0])
-        runner.set_staging(best[1])
-    runner.step(args.warmup)         # warm-up with the chosen variant
+    runner = pslbm.Batch(sims) if batch else sims[0]
+    runner.step(args.warmup)
     torch.cuda.synchronize()
-    tshape = runner.tile_shape()
-    staged = runner.staging()[0]
 
     replicas.barrier(ws)
     torch.cuda.synchronize()
@@ -373,10 +333,7 @@ def ours_arm(args):
             tot.append(total)
     torch.cuda.synchronize()
     clk = clocks.stop()
-    if batch:
-        runner.sync()
-    else:
-        runner.sync()
+    runner.sync()
     replicas.barrier(ws)
     my_ms = replicas.max_over_ranks(float(sum(tot)), ws)
     value = replicas.whole_job_rate(N * args.steps, ws, my_ms * 1e-3) / 1e6
@@ -396,17 +353,16 @@ def ours_arm(args):
         peaks = json.load(open(pk_path))
     peak = peaks.get("hbm_gbs", 6800.0)
     achieved = nbytes / (bulk_ms * 1e-3) / 1e9
-    variant = f"{tshape[0]}x{tshape[1]} {STAGING_NAMES[staged]}"
-    traffic = profile_traffic(args.workload, variant) if prec == pslbm.FP32 else None
+    prof = profile_summary(args.workload, "fp32") if prec == pslbm.FP32 else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": traffic, "kernel": KERNEL_NAMES[staged], "variant": variant,
+                "traffic": prof and prof["traffic_per_step"], "kernel": KERNEL_NAME,
                 "bytes_per_launch": nbytes, "kernel_ms": bulk_ms,
                 "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs, burst copy)" if "hbm_gbs" in peaks
                 else "fallback 6.8 TB/s",
                 "kernel_share": bulk_ms / statistics.mean(tot)}
     if prec == pslbm.FP64:
         # the FP64 path is bound by FP64 arithmetic, not by HBM
-        alu = fp64_roofline(args.workload, variant, bulk_ms)
+        alu = fp64_roofline(args.workload, bulk_ms)
         if alu is not None:
             alu["kernel_share"] = roofline["kernel_share"]
             alu["hbm"] = {k: roofline[k] for k in ("achieved", "peak", "unit", "frac", "bytes_per_launch")}
@@ -416,12 +372,7 @@ def ours_arm(args):
            "fluid_nodes": n_fluid, "liquid_nodes": n_liq, "precision": args.precision,
            "l2": ("flushed (256 MiB write) before every timed step" if flush is not None else
                   "not flushed: the state is far larger than the 129 MB L2"),
-           "parallelism": f"{'instances sharded over' if batch else 'replicas on'} {ws} GPU(s), no data-path exchange",
-           "tile": f"{tshape[0]}x{tshape[1]}", "staging": STAGING_NAMES[staged],
-           "variant_choice": ("the library's autotuner (each open variant timed for 3 steps, in two passes, best pass kept)" if trials is None else
-                              "each variant timed for 5 steps under the timed loop's conditions: " +
-                              ", ".join(f"{k[0][0]}x{k[0][1]} {STAGING_NAMES[k[1]]} {v:.4f} ms"
-                                        for k, v in sorted(trials.items())))}
+           "parallelism": f"{'instances sharded over' if batch else 'replicas on'} {ws} GPU(s), no data-path exchange"}
     line = {"metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": my_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None,
@@ -451,17 +402,14 @@ def ours_arm(args):
         t0 = time.perf_counter()
         sims2 = make_sims(pscenes)
         if batch:
-            r2 = pslbm.Batch(sims2, tile_x=tshape[0], tile_y=tshape[1])
-            r2.set_staging(staged)
+            r2 = pslbm.Batch(sims2)
         else:
             r2 = sims2[0]
-            r2.set_tile_shape(*tshape[:2])
-            r2.set_staging(staged)
         mon_bytes = 0
         for _ in range(args.steps):
             r2.step(1)
             r2.monitor()
-            mon_bytes += 16 * len(sims2) if batch else 64
+            mon_bytes += 16 * len(sims2) if batch else 80
         if batch:
             r2.close()
         # every member's budget into one device buffer (no allocation per

@@ -14,21 +14,21 @@
         independent porous geometries (seed 4), sides log-uniform 128-1024
         (multiples of 16), porosity U[0.4, 0.8], rates log-uniform 1e-6-1e-1,
         stepped together as one batch (one launch per kernel per step over the
-        packed tile list, CUDA graphs of up to 32 steps)
+        packed node lists, CUDA graphs of up to 32 steps)
     python -m paper_1410_3464_gb300.throughput --workload batch --variants [--trials 5]
-        every bulk-kernel variant (tile shape, nodes per thread, staging)
+        every tile shape (turns of a warp) and staging the library accepts
         fixed in turn on the workload (large, batch, or porous: 1024x512 seed
         1 with L2 flushed before every step): median over --trials profiled
-        steps of the bulk kernel's and the whole step's CUDA-event time
+        steps of the streaming kernels' and the whole step's CUDA-event time
 
 The large-lattice and batch working sets exceed the 129 MB L2 by an order of
 magnitude, so no flush is needed between steps; the plain scene (3.7 MB in
 FP64) lives in L2 and is launch-bound, and its figure is MLUPS only.  The step count is timed with CUDA events on the
-library stream after the variant autotuning and a warm-up; the JSON line
-gives MLUPS over all nodes, the algorithmic bytes of the bulk kernel (fluid
+library stream after a warm-up; the JSON line
+gives MLUPS over all nodes, the algorithmic bytes of the streaming kernels (fluid
 nodes x 144 B + liquid nodes x 120 B + 2 B per node for FP32 with three
 species) per step, the achieved GB/s of the whole step against the measured
-HBM bandwidth, and the chosen kernel variant.
+HBM bandwidth, and the tile shape and staging as reported.
 """
 from __future__ import annotations
 
@@ -42,7 +42,6 @@ import numpy as np
 from . import inputs, pslbm
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-STAGING_NAMES = {0: "plain loads", 1: "tma 2-stage", 2: "tma d2q9-box"}
 
 
 def peak_gbs():
@@ -79,7 +78,7 @@ def large(args, precision=pslbm.FP32, scene=None, name=None):
     fs = 8 if precision == pslbm.FP64 else 4
     with pslbm.Simulation(sc["mask"], sc["params"], sc["rho1"], sc["rho2"], sc["conc"], sc["vol"],
                           precision=precision) as s:
-        s.step(90)                       # autotuning (up to 10 variants x 4 steps, twice) and warm-up
+        s.step(90)                       # warm-up
         s.sync()
         el = timed(s.step, args.steps, stream)
         s.sync()
@@ -94,7 +93,7 @@ def large(args, precision=pslbm.FP32, scene=None, name=None):
                 nodes=N, fluid_nodes=nf, liquid_nodes=nl, steps=args.steps, seconds=el,
                 mlups=N * args.steps / el / 1e6, ms_per_step=1e3 * el / args.steps,
                 bulk_bytes_per_step=nbytes, step_gbs=gbs, peak_gbs=pk, peak_source=src, frac_of_peak=gbs / pk,
-                tile=f"{tx}x{ty}", staging=STAGING_NAMES[staged], scene_generation_s=gen_s)
+                tile=f"{tx}x{ty}", staging=staged, scene_generation_s=gen_s)
 
 
 def batch(args):
@@ -109,7 +108,7 @@ def batch(args):
     sims = [pslbm.Simulation(sc["mask"], sc["params"], sc["rho1"], sc["rho2"], sc["conc"], sc["vol"],
                              precision=pslbm.FP32) for sc in scenes]
     b = pslbm.Batch(sims)
-    b.step(90)                           # autotuning (up to 10 variants x 4 steps, twice) and warm-up
+    b.step(90)                           # warm-up
     b.sync()
     el = timed(b.step, args.steps, stream)
     b.sync()
@@ -134,11 +133,11 @@ def batch(args):
                 mean_nodes_per_instance=N / args.instances, min_side=int(sides.min()), max_side=int(sides.max()),
                 steps=args.steps, seconds=el, mlups=N * args.steps / el / 1e6, ms_per_step=1e3 * el / args.steps,
                 bulk_bytes_per_step=nbytes, step_gbs=gbs, peak_gbs=pk, peak_source=src, frac_of_peak=gbs / pk,
-                tile=f"{tx}x{ty}", staging=STAGING_NAMES[staged], scene_generation_s=gen_s)
+                tile=f"{tx}x{ty}", staging=staged, scene_generation_s=gen_s)
 
 
-# Bulk-kernel variants: (tile shape, staging); the two-node shapes (16x32,
-# 32x16) have no staging 1.
+# (tile shape, staging) as the library accepts them: 16x32 and 32x16 not with
+# staging 1.
 VARIANTS = [((16, 16), 0), ((16, 16), 1), ((16, 16), 2), ((32, 8), 0), ((32, 8), 1), ((32, 8), 2),
             ((16, 32), 0), ((16, 32), 2), ((32, 16), 0), ((32, 16), 2)]
 
@@ -160,8 +159,7 @@ def variants(args):
                     step_ms=statistics.median(t[1] for t in ts))
 
     def name(shape, sg):
-        npt = shape[0] * shape[1] // 256
-        return f"{shape[0]}x{shape[1]} ({npt} node{'s' if npt > 1 else ''}/thread), {STAGING_NAMES[sg]}"
+        return f"{shape[0]}x{shape[1]} ({shape[0] * shape[1] // 64} turns), staging {sg}"
 
     res = {}
     if args.workload == "batch":
@@ -203,7 +201,7 @@ def variants(args):
 def main(argv=None):
     ap = argparse.ArgumentParser(description=__doc__, formatter_class=argparse.RawDescriptionHelpFormatter)
     ap.add_argument("--workload", choices=["large", "batch", "plain", "porous-fp64", "porous"], default="large")
-    ap.add_argument("--variants", action="store_true", help="time every bulk-kernel variant (large, batch, porous)")
+    ap.add_argument("--variants", action="store_true", help="time every tile shape and staging (large, batch, porous)")
     ap.add_argument("--trials", type=int, default=5)
     ap.add_argument("--nx", type=int, default=4096)
     ap.add_argument("--ny", type=int, default=2048)
