@@ -100,8 +100,8 @@ __global__ void __launch_bounds__(FIELD_THREADS) k_fields(const DevInst* __restr
       R f1[9], f2[9];
 #pragma unroll
       for (int a = 0; a < 9; ++a) {
-        f1[a] = ldc<R>(F + foff((int)node) + a * CELL);
-        f2[a] = ldc<R>(F + foff((int)node) + (9 + a) * CELL);
+        f1[a] = ld<R>(F + foff((int)node) + a * CELL);
+        f2[a] = ld<R>(F + foff((int)node) + (9 + a) * CELL);
       }
       R d1 = f1[0], d2 = f2[0];
 #pragma unroll
@@ -158,9 +158,9 @@ __global__ void __launch_bounds__(FIELD_THREADS) k_fields(const DevInst* __restr
         double c = 0.0;
         if (t == T_LIQUID) {
           const TG* gk = G + goff<NS>((int)node) + k * 5 * CELL;
-          R s = gldc<R>(P, k, gk);
+          R s = gld<R>(P, k, gk);
 #pragma unroll
-          for (int a = 1; a < 5; ++a) s += gldc<R>(P, k, gk + a * CELL);
+          for (int a = 1; a < 5; ++a) s += gld<R>(P, k, gk + a * CELL);
           c = double(rp<R>(P).shift_c[k] + s);
         }
         o_conc[k * N + node] = c;
@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(BUD_THREADS) k_budget_partial(const DevInst* _
   for (long long node = lo + threadIdx.x; node < hi; node += blockDim.x) {
     const uint8_t t = T[node] & T_MASK;
     if (is_fluid(t)) {
-      const double r1 = double(fshift<R>(P, 0, t) + density_c<R>(F, 0, (int)node));
-      const double r2 = double(fshift<R>(P, 1, t) + density_c<R>(F, 1, (int)node));
+      const double r1 = double(fshift<R>(P, 0, t) + density_shifted<R>(F, 0, (int)node));
+      const double r2 = double(fshift<R>(P, 1, t) + density_shifted<R>(F, 1, (int)node));
       acc[0] = fmax(acc[0], r1);
       acc[1] += r1;
       acc[2] += r2;
@@ -201,9 +201,9 @@ __global__ void __launch_bounds__(BUD_THREADS) k_budget_partial(const DevInst* _
 #pragma unroll
       for (int k = 0; k < NS; ++k) {
         const TG* gk = G + goff<NS>((int)node) + k * 5 * CELL;
-        R s = gldc<R>(P, k, gk);
+        R s = gld<R>(P, k, gk);
 #pragma unroll
-        for (int a = 1; a < 5; ++a) s += gldc<R>(P, k, gk + a * CELL);
+        for (int a = 1; a < 5; ++a) s += gld<R>(P, k, gk + a * CELL);
         acc[3 + k] += double(rp<R>(P).shift_c[k] + s);
       }
     }

@@ -162,10 +162,14 @@ template <class T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f<__half>(__half v) { return __half2float(v); }
 template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <class R, class T> __device__ __forceinline__ R ld(const T* p) { return R(to_f<T>(__ldg(p))); }
-template <> __device__ __forceinline__ double ld<double, double>(const double* p) { return __ldg(p); }
-template <> __device__ __forceinline__ float ld<float, float>(const float* p) { return __ldg(p); }
-// L2 eviction policies, and a load under one (read-only path).
+// All loads of simulation state are coherent ones (ld.global).  A step's kernels may
+// be resident while the kernel before them still writes that state (launch_step), and
+// the read-only path wants memory that does not change during a kernel's whole life:
+// its loads are free to move above the wait (step_begin).
+template <class R, class T> __device__ __forceinline__ R ld(const T* p) { return R(to_f<T>(*p)); }
+template <> __device__ __forceinline__ double ld<double, double>(const double* p) { return *p; }
+template <> __device__ __forceinline__ float ld<float, float>(const float* p) { return *p; }
+// L2 eviction policies, and a load under one (volatile: it stays behind the wait).
 __device__ __forceinline__ unsigned long long l2_evict_first() {
   unsigned long long p;
   asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
@@ -179,15 +183,15 @@ __device__ __forceinline__ unsigned long long l2_evict_normal() {
 template <class R, class T> __device__ __forceinline__ R ld_l2(const T* p, unsigned long long policy) {
   if constexpr (sizeof(T) == 8) {
     double v;
-    asm("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(policy));
+    asm volatile("ld.global.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(policy));
     return R(v);
   } else if constexpr (sizeof(T) == 4) {
     float v;
-    asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(policy));
+    asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(policy));
     return R(v);
   } else {
     unsigned short v;
-    asm("ld.global.nc.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(p), "l"(policy));
+    asm volatile("ld.global.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(p), "l"(policy));
     T t;
     memcpy(&t, &v, sizeof t);
     return R(to_f<T>(t));
@@ -206,23 +210,13 @@ template <class T> struct Is16 { static constexpr bool value = false; };
 template <> struct Is16<__half> { static constexpr bool value = true; };
 template <> struct Is16<__nv_bfloat16> { static constexpr bool value = true; };
 
-// plain (coherent) loads for data written earlier in the same kernel sequence
-template <class R, class T> __device__ __forceinline__ R ldc(const T* p) { return R(to_f<T>(*p)); }
-template <> __device__ __forceinline__ double ldc<double, double>(const double* p) { return *p; }
-template <> __device__ __forceinline__ float ldc<float, float>(const float* p) { return *p; }
-
 // Solute population of species k as the compute precision sees it: the
 // stored value times the species' storage scale (16-bit storage only).
-// gld: read-only path (__ldg); gldc: coherent load; gst: store.
+// gld: load; gst: store.
 template <class R, class TG>
 __device__ __forceinline__ R gld(const DevParams& P, int k, const TG* p) {
   if constexpr (Is16<TG>::value) return ld<R>(p) * rp<R>(P).gs_div[k];
   else return ld<R>(p);
-}
-template <class R, class TG>
-__device__ __forceinline__ R gldc(const DevParams& P, int k, const TG* p) {
-  if constexpr (Is16<TG>::value) return ldc<R>(p) * rp<R>(P).gs_div[k];
-  else return ldc<R>(p);
 }
 template <class TG, class R>
 __device__ __forceinline__ void gst(const DevParams& P, int k, TG* p, R v) {
@@ -291,17 +285,6 @@ __device__ __forceinline__ R density_shifted(const TF* f, int comp, int node) {
   R s = ld<R>(p);
 #pragma unroll
   for (int a = 1; a < 9; ++a) s += ld<R>(p + a * CELL);
-  return s;
-}
-
-// Same sum through plain (coherent) loads, for data written by an earlier kernel
-// of the same step.
-template <class R, class TF>
-__device__ __forceinline__ R density_c(const TF* f, int comp, int node) {
-  const TF* p = f + foff(node) + comp * 9 * CELL;
-  R s = ldc<R>(p);
-#pragma unroll
-  for (int a = 1; a < 9; ++a) s += ldc<R>(p + a * CELL);
   return s;
 }
 

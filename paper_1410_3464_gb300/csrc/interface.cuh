@@ -80,10 +80,10 @@ __device__ __forceinline__ void vop_node(const DevInst* Ip, const DevParams& P, 
       oB[b - 1] = oE[b - 1] = oF[b - 1] = R(0);
       if (nn < 0) continue;
       if (useB) {
-        oB[b - 1] = gldc<R>(P, P.iB, gout + goff<NS>(nn) + (P.iB * 5 + b) * CELL);
-        if (P.iE >= 0) oE[b - 1] = gldc<R>(P, P.iE, gout + goff<NS>(nn) + (P.iE * 5 + b) * CELL);
+        oB[b - 1] = gld<R>(P, P.iB, gout + goff<NS>(nn) + (P.iB * 5 + b) * CELL);
+        if (P.iE >= 0) oE[b - 1] = gld<R>(P, P.iE, gout + goff<NS>(nn) + (P.iE * 5 + b) * CELL);
       }
-      if (useF) oF[b - 1] = gldc<R>(P, P.iF, gout + goff<NS>(nn) + (P.iF * 5 + b) * CELL);
+      if (useF) oF[b - 1] = gld<R>(P, P.iF, gout + goff<NS>(nn) + (P.iF * 5 + b) * CELL);
     }
 #pragma unroll
     for (int b = 1; b < 5; ++b) {
@@ -281,17 +281,17 @@ __device__ __forceinline__ void amend(const DevInst* Ip) {
       const long long nn = (long long)yn * P.nx + xn;
       const uint8_t tf = T[nn];
       if (surv_fluid(tf)) {
-        s1 += fshift<R>(P, 0, tf) + density_c<R>(F, 0, (int)nn);
-        s2 += fshift<R>(P, 1, tf) + density_c<R>(F, 1, (int)nn);
+        s1 += fshift<R>(P, 0, tf) + density_shifted<R>(F, 0, (int)nn);
+        s2 += fshift<R>(P, 1, tf) + density_shifted<R>(F, 1, (int)nn);
         ++nf;
       }
       if (surv_liquid(tf)) {
 #pragma unroll
         for (int k = 0; k < NS; ++k) {
           const TG* gk = G + goff<NS>((int)nn) + k * 5 * CELL;
-          R c = gldc<R>(P, k, gk);
+          R c = gld<R>(P, k, gk);
 #pragma unroll
-          for (int a = 1; a < 5; ++a) c += gldc<R>(P, k, gk + a * CELL);
+          for (int a = 1; a < 5; ++a) c += gld<R>(P, k, gk + a * CELL);
           sc[k] += rp<R>(P).shift_c[k] + c;
         }
         ++nl;
@@ -347,15 +347,15 @@ __device__ __forceinline__ void amend(const DevInst* Ip) {
         nf += surv_fluid(tz) ? 1 : 0;
         nl += surv_liquid(tz) ? 1 : 0;
       }
-      add1 += (fshift<R>(P, 0, T[w]) + density_c<R>(F, 0, (int)w)) / R(nf);
-      add2 += (fshift<R>(P, 1, T[w]) + density_c<R>(F, 1, (int)w)) / R(nf);
+      add1 += (fshift<R>(P, 0, T[w]) + density_shifted<R>(F, 0, (int)w)) / R(nf);
+      add2 += (fshift<R>(P, 1, T[w]) + density_shifted<R>(F, 1, (int)w)) / R(nf);
       if (nliq && nl) {
 #pragma unroll
         for (int k = 0; k < NS; ++k) {
           const TG* gk = G + goff<NS>((int)w) + k * 5 * CELL;
-          R c = gldc<R>(P, k, gk);
+          R c = gld<R>(P, k, gk);
 #pragma unroll
-          for (int a = 1; a < 5; ++a) c += gldc<R>(P, k, gk + a * CELL);
+          for (int a = 1; a < 5; ++a) c += gld<R>(P, k, gk + a * CELL);
           addc[k] += (rp<R>(P).shift_c[k] + c) / R(nl);
         }
       }
@@ -365,8 +365,8 @@ __device__ __forceinline__ void amend(const DevInst* Ip) {
       const R w = w9<R>(a);
       TF* p1 = F + foff(n) + a * CELL;
       TF* p2 = F + foff(n) + (9 + a) * CELL;
-      st<TF, R>(p1, ldc<R>(p1) + w * add1);
-      st<TF, R>(p2, ldc<R>(p2) + w * add2);
+      st<TF, R>(p1, ld<R>(p1) + w * add1);
+      st<TF, R>(p2, ld<R>(p2) + w * add2);
     }
     if (nliq) {
 #pragma unroll
@@ -375,7 +375,7 @@ __device__ __forceinline__ void amend(const DevInst* Ip) {
 #pragma unroll
         for (int a = 0; a < 5; ++a) {
           TG* p = G + goff<NS>(n) + (k * 5 + a) * CELL;
-          gst<TG, R>(P, k, p, gldc<R>(P, k, p) + (a == 0 ? J0 : Ja) * addc[k]);
+          gst<TG, R>(P, k, p, gld<R>(P, k, p) + (a == 0 ? J0 : Ja) * addc[k]);
         }
       }
     }

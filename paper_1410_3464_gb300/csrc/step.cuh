@@ -94,15 +94,15 @@ struct alignas(16) Pot {
   R ps, p1, p2, pad;
 };
 __device__ __forceinline__ Pot<float> ld_pot(const Pot<float>* p) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+  const float4 v = *reinterpret_cast<const float4*>(p);
   return Pot<float>{v.x, v.y, v.z, v.w};
 }
 __device__ __forceinline__ Pot<double> ld_pot(const Pot<double>* p) {
-  const double2 v = __ldg(reinterpret_cast<const double2*>(p));
-  return Pot<double>{v.x, v.y, __ldg(&p->p2), 0.0};
+  const double2 v = *reinterpret_cast<const double2*>(p);
+  return Pot<double>{v.x, v.y, p->p2, 0.0};
 }
 // FP64: rho_1 rides along with the potentials (eight additions less in k_move).
-__device__ __forceinline__ double pot_rho1(const Pot<double>* p) { return __ldg(&p->pad); }
+__device__ __forceinline__ double pot_rho1(const Pot<double>* p) { return p->pad; }
 __device__ __forceinline__ float pot_rho1(const Pot<float>*) { return 0.f; }
 
 // Both kernels run over the instance's list of fluid nodes (in tile order, kept
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : 8)
   const DevParams& P = I.P;
   const DevParams& Q = MODE == M_MIXED ? P : Ik.P;
   unsigned long long* scal = I.scal;
-  const int* __restrict__ flist = I.flist;
+  const int* flist = I.flist;
   const int head = flist[min(wk.first + lane, (int)I.N - 1)];   // in flight beside the counters
   const unsigned long long step = scal[S_STEP];
   const bool live = step < scal[S_LIMIT];   // else a frozen instance
@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : 8)
   if (!live) return;
   const int n = (int)scal[S_NFLUID];
   const R theta = theta_of<R>(&I);
-  const TF* __restrict__ fin = (const TF*)I.f[cur];
-  const uint8_t* __restrict__ tin = I.type[cur];
+  const TF* fin = (const TF*)I.f[cur];
+  const uint8_t* tin = I.type[cur];
   uint8_t* __restrict__ tout = I.type[cur ^ 1];
   Pot<R>* __restrict__ pot = (Pot<R>*)I.pot;
   uint8_t* __restrict__ code = I.code;
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : 4)
   const DevParams& Q = MODE == M_MIXED ? P : Ik.P;
   const DevParamsR<R>& rates = rp<R>(P);
   auto pr = [](const R& v) { return MODE == M_SINGLE ? v : __ldg(&v); };
-  const int* __restrict__ flist = I.flist;
+  const int* flist = I.flist;
   const int head = flist[min(wk.first + lane, (int)I.N - 1)];   // in flight beside the counters
   const unsigned long long step = I.scal[S_STEP];
   const bool live = step < I.scal[S_LIMIT];   // else a frozen instance
@@ -455,12 +455,12 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : 4)
   }
   if (!live) return;
   const int n = (int)I.scal[S_NFLUID];
-  const TF* __restrict__ fin = (const TF*)I.f[cur];
+  const TF* fin = (const TF*)I.f[cur];
   TF* __restrict__ fout = (TF*)I.f[cur ^ 1];
-  const TG* __restrict__ gin = (const TG*)I.g[cur];
+  const TG* gin = (const TG*)I.g[cur];
   TG* __restrict__ gout = (TG*)I.g[cur ^ 1];
-  const Pot<R>* __restrict__ pot = (const Pot<R>*)I.pot;
-  const uint8_t* __restrict__ code = I.code;
+  const Pot<R>* pot = (const Pot<R>*)I.pot;
+  const uint8_t* code = I.code;
   const int nx = P.nx, ny = P.ny;
   const bool px = P.px != 0, py = P.py != 0;
   auto spec = [&](const R* v, int k) { return mk<R>(v[2 * k], v[2 * k + 1]); };
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : 4)
 #pragma unroll
     for (int a = 0; a < 9; ++a) F[a] = mk<R>(ld_l2<R>(fi + a * CELL, once), ld_l2<R>(fi + (9 + a) * CELL, once));
   }
-  const int c0 = __ldg(code + node);
+  const int c0 = code[node];
   const int y = node_row(P, node), x = node - y * nx;
   // ---- neighbours: index offsets (with periodic wrap) and codes (outside a
   // non-periodic edge a wall)
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : 4)
   for (int a = 1; a < 9; ++a) {
     dn[a] = (EX(a) > 0 ? orr : EX(a) < 0 ? ol : 0) + (EY(a) > 0 ? ou : EY(a) < 0 ? od : 0);
     const bool in = (EX(a) > 0 ? vr : EX(a) < 0 ? vl : true) && (EY(a) > 0 ? vu : EY(a) < 0 ? vd : true);
-    nc[a] = in ? (int)__ldg(code + node + dn[a]) : 0;
+    nc[a] = in ? (int)code[node + dn[a]] : 0;
   }
   PR gs[NPX][5];   // solute populations, two species a pair (unused at a node that was gas)
   if constexpr (NS > 0) {
