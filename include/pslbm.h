@@ -61,7 +61,8 @@ typedef enum {
 } pslbm_precision;
 
 /* Node types (Fig. 2: liquid, gas, solid D(s), solid F(s); plus inert walls and
- * reservoir nodes that push a fixed equilibrium state into their neighbours). */
+ * reservoir nodes that push a fixed equilibrium state into their neighbours).
+ * Only the low nibble of a mask byte counts; a type above PSLBM_OUTLET acts as a wall. */
 enum {
     PSLBM_LIQUID = 0, PSLBM_GAS = 1, PSLBM_SOLID_D = 2, PSLBM_SOLID_F = 3,
     PSLBM_WALL = 4, PSLBM_INLET = 5, PSLBM_OUTLET = 6

@@ -61,8 +61,9 @@ __device__ __forceinline__ void flush_acc(TileAcc<R>& acc, unsigned long long* s
 // type D(s), fluid and marked).
 constexpr int C_FLUID = 1, C_MARK = 2, C_RES = 4, C_MIN = 8, C_FGAS = 16, C_OLDLIQ = 32, C_SOLD = 64, C_FLIQ = 128;
 constexpr int C_LIVE = C_FLUID | C_RES;     // test with != 0
-// ... by type, before marking.
+// ... by type, before marking; a type outside the enumeration is a wall.
 __device__ __forceinline__ int type_code(int t) {
+  if (t > T_OUTLET) return 0;
   constexpr unsigned lo = unsigned(C_FLUID | C_OLDLIQ) | unsigned(C_FLUID) << 8 | unsigned(C_MIN | C_SOLD) << 16 |
                           unsigned(C_MIN) << 24;
   constexpr unsigned hi = unsigned(C_RES) << 8 | unsigned(C_RES) << 16;
