@@ -376,31 +376,8 @@ template <class R> __device__ __forceinline__ R psi_arg(const DevParams& P, R rh
   return rmul<R>(Q.six_over_G11, rsub<R>(p, rmul<R>(rho, R(1.0 / 3.0))));
 }
 
-// FP64 reciprocal and square root.  An FP64 instruction holds its quarter of an SM
-// for 64 cycles whatever its lanes do (measured; FP32: 2), so the FP64 kernels
-// cost what they issue.  Both take the hardware's approximation (20 bits and more)
-// and one third-order correction of Newton's iteration: with e = 1 - v r the
-// reciprocal is r (1 + e + e^2 + O(e^3)), and with e = 1 - v y^2 the square root is
-// v y (1 + e/2 + 3 e^2/8 + O(e^3)).  Arguments near the ends of the exponent
-// range, zero, infinities and NaN take the CUDA operation.
-__device__ __forceinline__ bool mid_range(double v) {
-  return (((unsigned)__double2hiint(v) >> 20) & 0x7FFu) - 24u < 2000u;
-}
-__device__ __forceinline__ double rcp64(double v) {
-  if (!mid_range(v)) return 1.0 / v;
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
-  const double e = __fma_rn(-v, r, 1.0);
-  return __fma_rn(r, __fma_rn(e, e, e), r);
-}
-__device__ __forceinline__ double sqrt64(double v) {
-  if (!mid_range(v)) return sqrt(v);
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
-  const double g = __dmul_rn(v, y);
-  const double e = __fma_rn(-g, y, 1.0);
-  return __fma_rn(g, __dmul_rn(e, __fma_rn(0.375, e, 0.5)), g);
-}
+// An FP64 instruction holds its quarter of an SM for 64 cycles whatever its lanes do
+// (measured; FP32: 2), so the FP64 kernels cost what they issue: hence what follows.
 // Comparisons of doubles on their bits (no FP64 instruction); x is not NaN.
 __device__ __forceinline__ long long order_bits(double x) {
   const long long b = __double_as_longlong(x);
@@ -418,7 +395,7 @@ template <> __device__ __forceinline__ bool is_zero<double>(double x) {
   return ((__double2hiint(x) << 1) | __double2loint(x)) == 0;
 }
 template <class R> __device__ __forceinline__ R rrcp(R v);
-template <> __device__ __forceinline__ double rrcp<double>(double v) { return rcp64(v); }
+template <> __device__ __forceinline__ double rrcp<double>(double v) { return __drcp_rn(v); }
 template <> __device__ __forceinline__ float rrcp<float>(float v) { return __frcp_rn(v); }
 template <class R> __device__ __forceinline__ R rmax(R a, R b);
 template <> __device__ __forceinline__ double rmax<double>(double a, double b) { return fmax(a, b); }
@@ -599,27 +576,22 @@ __device__ __forceinline__ void potentials(const DevParams& P, R rho1, R rho2, R
   phi1 = -rexpm1<R>(-rmul<R>(rho2, Q.inv_rho20));
   phi2 = rsub<R>(Q.a0, rexp<R>(-rmul<R>(rho1, Q.inv_rho10)));
 }
-// FP64: the same with few FP64 instructions (rcp64, sqrt64).  phi_2's exponential
-// is left out where it is below half an ulp of a0 (P.phi2_cut, in the liquid), and
-// phi_1 = x - x^2/2 + x^3/6 - ... is summed as it stands for small x = rho_2 /
-// rho_20 (also the liquid): for |x| < 1/16 ten terms leave 2.3e-20 of x.
+// FP64: the same with few FP64 instructions.  phi_2's exponential is left out where
+// it is below half an ulp of a0 (P.phi2_cut, in the liquid), and phi_1 = x - x^2/2 +
+// x^3/6 - ... is summed as it stands for small x = rho_2 / rho_20 (also the liquid):
+// for |x| < 1/16 ten terms leave 2.3e-20 of x.
 template <>
 __device__ __forceinline__ void potentials<double>(const DevParams& P, double rho1, double rho2, double& psi, double& phi1,
                                                    double& phi2, unsigned& status) {
   const DevParamsR<double>& Q = P.rd;
   psi = 0.0;
   if (P.has_G11) {
-    const double eta = Q.eos_b4 * rho1;
-    const double om = 1.0 - eta;
-    const double poly = __fma_rn(eta, __fma_rn(eta, om, 1.0), 1.0);
-    const double num = (rho1 * Q.eos_RT) * poly;
-    const double p = __fma_rn(-(Q.eos_a * rho1), rho1, num * rcp64(om * om * om));
-    double arg = Q.six_over_G11 * __fma_rn(rho1, -1.0 / 3.0, p);
+    double arg = psi_arg<double>(P, rho1);
     if (is_nan(arg) || (__double2hiint(arg) < 0 && !is_zero(arg))) {
       status |= is_nan(arg) ? ST_NONFINITE : ST_EOS;
       arg = 0.0;
     }
-    psi = sqrt64(arg);
+    psi = sqrt(arg);
   }
   const double x = rho2 * Q.inv_rho20;
   if ((__double2hiint(x) & 0x7FFFFFFF) < 0x3FB00000) {

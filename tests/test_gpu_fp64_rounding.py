@@ -1,0 +1,72 @@
+"""FP64 arithmetic of the potentials and velocities, operation by operation.
+
+A state at rest gives velocities that follow from the densities by a few dozen
+operations (Eqs. 11-13, 19 and the body force).  Here they are done on the host with
+correctly rounded operations (addition, product, quotient, square root, fused
+multiply-add) in the order of the device code; the device has to give the same bits:
+its quotient, reciprocal and square root are the correctly rounded ones.
+"""
+import ctypes
+import math
+
+import numpy as np
+import pytest
+
+from paper_1410_3464_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+_libm = ctypes.CDLL("libm.so.6")
+_libm.fma.restype = ctypes.c_double
+_libm.fma.argtypes = [ctypes.c_double] * 3
+fma = np.vectorize(lambda a, b, c: _libm.fma(a, b, c), otypes=[np.float64])
+
+
+@pytest.fixture(scope="module")
+def pslbm():
+    from paper_1410_3464_gb300 import build, pslbm as m
+    build.build()
+    return m
+
+
+def psi(rho, p):
+    eta = (p["eos_b"] / 4.0) * rho
+    om = 1.0 - eta
+    poly = fma(eta, fma(eta, om, 1.0), 1.0)
+    num = (rho * (p["eos_R"] * p["eos_T"])) * poly
+    pr = fma(-(p["eos_a"] * rho), rho, num / ((om * om) * om))
+    arg = (6.0 / p["G11"]) * (pr - rho * (1.0 / 3.0))
+    assert (arg >= 0).all()
+    return np.sqrt(arg)
+
+
+@pytest.mark.parametrize("top", [1.0, 1e-3])
+@pytest.mark.parametrize("G11", [True, False])
+def test_velocities_at_rest_are_correctly_rounded(pslbm, G11, top):
+    """Densities over the liquid (top 1) and the gas (top 1e-3) range; with the EOS
+    forces, and with the body force alone (the reciprocal of the density)."""
+    nx, ny = 48, 40
+    rng = np.random.default_rng(5)
+    p = inputs.base_params(nx, ny)
+    p.update(periodic_x=1, periodic_y=1, n_species=0, idx_A=-1, idx_B=-1, idx_E=-1, idx_F=-1, G12=0.0, G21=0.0,
+             w_adh=(0.0, 0.0), body_force=(1.3e-5, -7.1e-6))
+    if not G11:
+        p["G11"] = 0.0
+    rho1 = top * inputs.COEX_ORIGINAL_07[0] * rng.uniform(0.9, 1.1, (ny, nx))
+    rho2 = rng.uniform(1e-5, 2e-3, (ny, nx))
+    with pslbm.Simulation(np.zeros((ny, nx), np.uint8), p, rho1, rho2, None, None, precision=pslbm.FP64) as sim:
+        got = sim.read()
+    r1, r2 = got["rho1"], got["rho2"]
+    F1 = [np.zeros_like(r1), np.zeros_like(r1)]
+    if G11:
+        s0 = psi(r1, p)
+        v = [s0] + [np.roll(s0, (-ey, -ex), (0, 1)) for ex, ey in ((1, 0), (0, 1), (-1, 0), (0, -1), (1, 1), (-1, 1), (-1, -1), (1, -1))]
+        d57, d86 = v[5] - v[7], v[8] - v[6]
+        S = (fma(1.0 / 9.0, v[1] - v[3], (1.0 / 36.0) * (d57 + d86)), fma(1.0 / 9.0, v[2] - v[4], (1.0 / 36.0) * (d57 - d86)))
+        F1 = [-((p["G11"] * s0) * s) for s in S]
+    for i, name in ((0, "ux"), (1, "uy")):
+        g = p["body_force"][i]
+        f1, f2 = fma(r1, g, F1[i]), r2 * g
+        u = (0.5 * (f1 + f2)) * (1.0 / (r1 + r2))
+        np.testing.assert_array_equal(got[name], u, err_msg=name)
+    assert math.isfinite(float(got["ux"].sum()))
