@@ -742,28 +742,20 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : 4)
               Ss = c1 ? S.a : S.b, it = c1 ? it1 : it2;
       TF* fo = fout + s * 9 * CELL;
       R feq[9];
+      feq_pairs<R>(ds, rs, vx, vy, half_u2<R>(vx, vy), feq);
       if (sizeof(R) == 8 && Q.tau_unit) {
-        // FP64 at tau = 1: the collision leaves the equilibrium and the source,
-        // w (rho (1 + 3 e.u + 4.5 (e.u)^2 - 1.5 u^2) + S), here with the parts that
-        // directions share formed once (30 FP64 instructions instead of 64)
-        const R xx = vx * vx, yy = vy * vy, u2 = xx + yy, tx = vx + vx;
-        const R A = rfma<R>(R(-1.5) * rs, u2, rs + Ss), A9 = R(1.0 / 9.0) * A, A36 = R(1.0 / 36.0) * A;
-        const R h = R(0.5) * rs, h8 = R(0.125) * rs, as = R(1.0 / 3.0) * rs, ad = R(1.0 / 12.0) * rs;
-        const R sx_ = rfma<R>(h, xx, A9), sy_ = rfma<R>(h, yy, A9);
-        const R sp = rfma<R>(h8, rfma<R>(tx, vy, u2), A36), sm = rfma<R>(h8, rfma<R>(-tx, vy, u2), A36);
-        const R ep = vx + vy, em = vy - vx;
-        feq[0] = R(4.0 / 9.0) * A;
-        feq[1] = rfma<R>(as, vx, sx_);
-        feq[3] = rfma<R>(-as, vx, sx_);
-        feq[2] = rfma<R>(as, vy, sy_);
-        feq[4] = rfma<R>(-as, vy, sy_);
-        feq[5] = rfma<R>(ad, ep, sp);
-        feq[7] = rfma<R>(-ad, ep, sp);
-        feq[6] = rfma<R>(ad, em, sm);
-        feq[8] = rfma<R>(-ad, em, sm);
+        // FP64 at tau = 1: the collision leaves the equilibrium, and a liquid node's
+        // source.  Each direction is rounded by itself: with rho (1 - 1.5 u^2) + S
+        // formed once for all nine (30 instructions instead of 44, 64 with the BGK
+        // difference) the nine errors had one sign, and the beaker's densities were
+        // 2.2e-15 off after 200 steps instead of 5.2e-16
+        if constexpr (NS > 0) {
+          if (liq) {
+#pragma unroll
+            for (int a = 0; a < 9; ++a) feq[a] = rfma<R>(w9<R>(a), Ss, feq[a]);
+          }
+        }
       } else {
-        const R uu = half_u2<R>(vx, vy);
-        feq_pairs<R>(ds, rs, vx, vy, uu, feq);
 #pragma unroll
         for (int a = 0; a < 9; ++a) feq[a] = bgk<R>(c1 ? F[a].a : F[a].b, feq[a], it, w9<R>(a), Ss);
       }

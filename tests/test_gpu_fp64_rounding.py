@@ -70,3 +70,53 @@ def test_velocities_at_rest_are_correctly_rounded(pslbm, G11, top):
         u = (0.5 * (f1 + f2)) * (1.0 / (r1 + r2))
         np.testing.assert_array_equal(got[name], u, err_msg=name)
     assert math.isfinite(float(got["ux"].sum()))
+
+
+W9 = (4.0 / 9.0,) + (1.0 / 9.0,) * 4 + (1.0 / 36.0,) * 4
+E9 = ((0, 0), (1, 0), (0, 1), (-1, 0), (0, -1), (1, 1), (-1, 1), (-1, -1), (1, -1))
+
+
+def feq9(rho, ux, uy):
+    """Eq. 8, opposite directions together (the even part, then plus and minus the odd one)."""
+    uu = 1.5 * fma(ux, ux, uy * uy)
+    f = [None] * 9
+    f[0] = W9[0] * fma(rho, -uu, rho)
+    for p, m, e in ((1, 3, ux), (2, 4, uy), (5, 7, ux + uy), (6, 8, uy - ux)):
+        sym = W9[p] * fma(rho, fma(4.5, e * e, -uu), rho)
+        asym = ((1.0 / 3.0 if p < 5 else 1.0 / 12.0) * rho) * e
+        f[p], f[m] = sym + asym, sym - asym
+    return f
+
+
+def streamed_sum(f, e):
+    f = [np.roll(v, (e[a][1], e[a][0]), (0, 1)) for a, v in enumerate(f)]
+    s = f[0]
+    for v in f[1:]:
+        s = s + v
+    return s
+
+
+def reacting(nx, ny, tau_g, seed=8):
+    """Liquid at rest with a body force and one species that turns into gas."""
+    rng = np.random.default_rng(seed)
+    p = inputs.base_params(nx, ny)
+    p.update(periodic_x=1, periodic_y=1, n_species=1, idx_A=0, idx_B=-1, idx_E=-1, idx_F=-1, G11=0.0, G12=0.0, G21=0.0,
+             w_adh=(0.0, 0.0), body_force=(3e-4, -2e-4), J0=(0.3, 0, 0, 0), tau_g=(tau_g, 1, 1, 1), k1=2e-3, gas_yield=0.4)
+    rho1 = rng.uniform(7.0, 8.5, (ny, nx))
+    rho2 = rng.uniform(1e-5, 2e-3, (ny, nx))
+    return p, rho1, rho2, rng.uniform(0.2, 1.5, (1, ny, nx))
+
+
+@pytest.mark.parametrize("tau_g", [0.8])
+def test_one_fluid_step_is_correctly_rounded(pslbm, tau_g):
+    p, rho1, rho2, conc = reacting(44, 36, tau_g)
+    with pslbm.Simulation(np.zeros(rho1.shape, np.uint8), p, rho1, rho2, conc, None, precision=pslbm.FP64) as sim:
+        r0 = sim.read()
+        sim.step(1)
+        got = sim.read()
+    y1 = p["gas_yield"] * (p["k1"] * r0["conc"][0])
+    for name, S in (("rho1", -y1), ("rho2", y1)):
+        rho = r0[name]
+        ux, uy = ((rho * g) * (1.0 / rho) for g in p["body_force"])
+        f = [fma(w, S, v) for w, v in zip(W9, feq9(rho, ux, uy))]
+        np.testing.assert_array_equal(got[name], streamed_sum(f, E9), err_msg=name)
