@@ -55,7 +55,7 @@ struct DevParamsR {
   R tau[2], inv_tau[2], G11, G12, G21, a0, inv_rho10, inv_rho20, w_adh[2];
   R eos_a, eos_b4, eos_RT, six_over_G11;
   R gx, gy, shift_f[2], shift_fg[2], rho_fill[2];
-  R J0[MAXS], Ja[MAXS], inv_tau_g[MAXS], keep_g[MAXS], half_tau_g[MAXS], shift_c[MAXS], conc_in[MAXS], cR1[MAXS], cR3[MAXS];
+  R J0[MAXS], Ja[MAXS], inv_tau_g[MAXS], shift_c[MAXS], conc_in[MAXS], cR1[MAXS], cR3[MAXS];
   R k1, k1_inv_Keq, k3, k2, k4, C_F_sat, gas_yield, inv_M_C, c_total_per_rho1;
   R k1_s, k1_inv_Keq_s;   // R1 constants at liquid nodes touching D(s) (surface factor applied)
   // reactive link rule (Eqs. 29-31 as a halfway wall): link flux q = out * qa - qc,

@@ -212,8 +212,6 @@ void fill_r(DevParamsR<R>& q, const DevParams& P) {
     q.J0[k] = R(P.J0[k]);
     q.Ja[k] = R(P.Ja[k]);
     q.inv_tau_g[k] = R(P.inv_tau_g[k]);
-    q.keep_g[k] = R(1.0 - P.inv_tau_g[k]);
-    q.half_tau_g[k] = R(0.5 * P.inv_tau_g[k]);
     q.shift_c[k] = R(P.shift_c[k]);
     q.conc_in[k] = R(P.conc_in[k]);
     q.cR1[k] = R(P.cR1[k]);

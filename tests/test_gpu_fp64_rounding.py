@@ -120,3 +120,22 @@ def test_one_fluid_step_is_correctly_rounded(pslbm, tau_g):
         ux, uy = ((rho * g) * (1.0 / rho) for g in p["body_force"])
         f = [fma(w, S, v) for w, v in zip(W9, feq9(rho, ux, uy))]
         np.testing.assert_array_equal(got[name], streamed_sum(f, E9), err_msg=name)
+
+
+@pytest.mark.parametrize("tau_g", [0.8, 1.0, 3.3])
+def test_one_solute_step_is_correctly_rounded(pslbm, tau_g):
+    p, rho1, rho2, conc = reacting(44, 36, tau_g, seed=9)
+    with pslbm.Simulation(np.zeros(rho1.shape, np.uint8), p, rho1, rho2, conc, None, precision=pslbm.FP64) as sim:
+        r0 = sim.read()
+        sim.step(1)
+        got = sim.read()
+    r1, r2, C = r0["rho1"], r0["rho2"], r0["conc"][0]
+    J0 = p["J0"][0]
+    J = [J0] + [(1.0 - J0) / 4.0] * 4
+    h = 0.5 * (1.0 / (r1 + r2))
+    ux, uy = (h * (r1 * g + r2 * g) for g in p["body_force"])      # no momentum yet
+    sa, ax, ay = J[1] * C, (0.5 * C) * ux, (0.5 * C) * uy
+    ge = [J0 * C, sa + ax, sa + ay, sa - ax, sa - ay]
+    S = -(p["k1"] * C)
+    go = [fma(J[a], S, fma(ge[a] - J[a] * conc[0], 1.0 / tau_g, J[a] * conc[0])) for a in range(5)]
+    np.testing.assert_array_equal(got["conc"][0], streamed_sum(go, E9))
