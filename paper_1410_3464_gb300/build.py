@@ -14,6 +14,12 @@ OUT_DIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(OUT_DIR, "libpslbm.so")
 SOURCES = ["kernels_f64.cu", "kernels_f32.cu", "kernels_f32h.cu", "kernels_f32b.cu", "runtime.cu", "noalloc.cu", "serve.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+# No product is fused into a sum but where the source says so: otherwise the compiler
+# may do it in one instantiation of the FP64 kernels (one simulation, batch of like or
+# unlike members, VOP and amendment in one launch or two) and not in another, and
+# their bits would differ.  The FP32 units keep the default, on which the bits of
+# their expf and expm1f rest.
+FLAGS = {"kernels_f64.cu": ["-fmad=false"]}
 
 
 def nvcc():
@@ -26,6 +32,12 @@ def nvcc():
     raise RuntimeError("nvcc not found")
 
 
+def compile_command(src, cc="nvcc"):
+    obj = os.path.join(OUT_DIR, "obj", src.replace(".cu", ".o"))
+    return ([cc] + ARCH + ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC"] + FLAGS.get(src, []) +
+            ["-c", os.path.join(CSRC, src), "-o", obj])
+
+
 def _stale(obj, src_files):
     if not os.path.exists(obj):
         return True
@@ -36,15 +48,14 @@ def _stale(obj, src_files):
 def build(verbose=False, force=False):
     os.makedirs(os.path.join(OUT_DIR, "obj"), exist_ok=True)
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
-    headers.append(os.path.join(os.path.dirname(HERE), "include", "pslbm.h"))
+    headers += [os.path.join(os.path.dirname(HERE), "include", "pslbm.h"), os.path.abspath(__file__)]
     cc = nvcc()
     jobs = []
     for src in SOURCES:
         s = os.path.join(CSRC, src)
         o = os.path.join(OUT_DIR, "obj", src.replace(".cu", ".o"))
         if force or _stale(o, [s] + headers):
-            cmd = [cc] + ARCH + ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-c", s, "-o", o]
-            jobs.append((src, cmd))
+            jobs.append((src, compile_command(src, cc)))
     if jobs:
         with cf.ThreadPoolExecutor(max_workers=len(jobs)) as ex:
             futs = {ex.submit(subprocess.run, cmd, capture_output=True, text=True): src for src, cmd in jobs}

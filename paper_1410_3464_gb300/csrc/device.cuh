@@ -307,8 +307,8 @@ __device__ __forceinline__ void reservoir_rho(const DevParams& P, uint8_t t, uns
         wg = (R > 0 && ph >= per - R) ? 1.0 - double(ph - (per - R) + 1) / double(R + 1) : 1.0;
       }
     }
-    r1 = (1.0 - wg) * P.rho_in_liq[0] + wg * P.rho_in_gas[0];
-    r2 = (1.0 - wg) * P.rho_in_liq[1] + wg * P.rho_in_gas[1];
+    r1 = __fma_rn(1.0 - wg, P.rho_in_liq[0], __dmul_rn(wg, P.rho_in_gas[0]));
+    r2 = __fma_rn(1.0 - wg, P.rho_in_liq[1], __dmul_rn(wg, P.rho_in_gas[1]));
   } else {
     // outlet: the coexistence state of the phase arriving from upstream
     r1 = up_liquid ? P.rho_out[0] : P.rho_out_gas[0];
@@ -343,11 +343,13 @@ __device__ __forceinline__ bool outlet_up_liquid(const DevParams& P, const uint8
   return liquid_at<R, TF>(P, tin, fin, N, yn * P.nx + xn, theta);
 }
 
-// Explicitly rounded operations.  The hot formulas are written with these
-// (fused where a product feeds a sum) so that the compiler cannot contract
+// Explicitly rounded operations.  The formulas are written with these (fused
+// where a product feeds a sum) so that the compiler cannot contract
 // them differently in different instantiations: with parameters from global
-// memory or from the constant bank, alone or in a batch, the kernels evaluate
-// exactly the same operations and give bit-identical results.
+// memory or from the constant bank, alone or in a batch, VOP and amendment in one
+// launch or in two, the kernels evaluate
+// exactly the same operations and give bit-identical results.  The FP64 unit is
+// compiled without contraction besides (build.py).
 template <class R> __device__ __forceinline__ R radd(R a, R b);
 template <class R> __device__ __forceinline__ R rsub(R a, R b);
 template <class R> __device__ __forceinline__ R rmul(R a, R b);
@@ -593,7 +595,7 @@ __device__ __forceinline__ void potentials<double>(const DevParams& P, double rh
     }
     psi = sqrt(arg);
   }
-  const double x = rho2 * Q.inv_rho20;
+  const double x = __dmul_rn(rho2, Q.inv_rho20);
   if ((__double2hiint(x) & 0x7FFFFFFF) < 0x3FB00000) {
     double s = -1.0 / 3628800.0;
     s = __fma_rn(s, x, 1.0 / 362880.0);
@@ -608,9 +610,9 @@ __device__ __forceinline__ void potentials<double>(const DevParams& P, double rh
   } else {
     phi1 = -expm1(-x);
   }
-  const double z = rho1 * Q.inv_rho10;
+  const double z = __dmul_rn(rho1, Q.inv_rho10);
   phi2 = Q.a0;
-  if (!(__double2hiint(z) > P.phi2_cut)) phi2 = Q.a0 - exp(-z);
+  if (!(__double2hiint(z) > P.phi2_cut)) phi2 = __dsub_rn(Q.a0, exp(-z));
 }
 
 // SplitMix64 output for a given state (Steele, Lea, Flood 2014).

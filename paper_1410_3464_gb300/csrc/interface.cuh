@@ -92,26 +92,26 @@ __device__ __forceinline__ void vop_node(const DevInst* Ip, const DevParams& P, 
       if (useB) {
         const int iB = P.iB;
         const R sh = rp<R>(P).vB_sh;
-        const R out = oB[b - 1] + sh;
-        const R q = out * rp<R>(P).vB_qa;
-        const R bk = out - q;
-        gst<TG, R>(P, iB, gout + goff<NS>(nn) + (iB * 5 + b) * CELL, bk - sh);
-        sB += q;
-        if (P.iE >= 0) gst<TG, R>(P, P.iE, gout + goff<NS>(nn) + (P.iE * 5 + b) * CELL, oE[b - 1] + q);
+        const R out = radd<R>(oB[b - 1], sh);
+        const R q = rmul<R>(out, rp<R>(P).vB_qa);
+        const R bk = rsub<R>(out, q);
+        gst<TG, R>(P, iB, gout + goff<NS>(nn) + (iB * 5 + b) * CELL, rsub<R>(bk, sh));
+        sB = radd<R>(sB, q);
+        if (P.iE >= 0) gst<TG, R>(P, P.iE, gout + goff<NS>(nn) + (P.iE * 5 + b) * CELL, radd<R>(oE[b - 1], q));
       }
       if (useF) {
         const int iF = P.iF;
         const R sh = rp<R>(P).vF_sh;
-        const R out = oF[b - 1] + sh;
-        const R q = out * rp<R>(P).vF_qa - rp<R>(P).vF_qc;
-        gst<TG, R>(P, iF, gout + goff<NS>(nn) + (iF * 5 + b) * CELL, (out - q) - sh);
-        sF += q;
+        const R out = radd<R>(oF[b - 1], sh);
+        const R q = rfma<R>(out, rp<R>(P).vF_qa, -rp<R>(P).vF_qc);
+        gst<TG, R>(P, iF, gout + goff<NS>(nn) + (iF * 5 + b) * CELL, rsub<R>(rsub<R>(out, q), sh));
+        sF = radd<R>(sF, q);
       }
     }
   }
   // volumes accumulate in FP64: per-step increments are far below FP32 resolution of V
-  if (t == T_SOLID_D) VD = VD - P.Vbar_D * double(sB);   // Eq. 33
-  VF = VF + P.Vbar_F * double(sF);                        // Eq. 35 (precipitation adds volume)
+  if (t == T_SOLID_D) VD = __fma_rn(-P.Vbar_D, double(sB), VD);   // Eq. 33
+  VF = __fma_rn(P.Vbar_F, double(sF), VF);                        // Eq. 35 (precipitation adds volume)
   if (VD < 0.0) VD = 0.0;
   const double total = VD + VF;
   int ev = EV_NONE;
@@ -302,8 +302,8 @@ __device__ __forceinline__ void amend(const DevInst* Ip) {
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
       const R w = w9<R>(a);
-      st<TF, R>(F + foff(node) + a * CELL, w * r1 - w * rp<R>(P).shift_f[0]);
-      st<TF, R>(F + foff(node) + (9 + a) * CELL, w * r2 - w * rp<R>(P).shift_f[1]);
+      st<TF, R>(F + foff(node) + a * CELL, rfma<R>(w, r1, -rmul<R>(w, rp<R>(P).shift_f[0])));
+      st<TF, R>(F + foff(node) + (9 + a) * CELL, rfma<R>(w, r2, -rmul<R>(w, rp<R>(P).shift_f[1])));
     }
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
@@ -312,7 +312,7 @@ __device__ __forceinline__ void amend(const DevInst* Ip) {
 #pragma unroll
       for (int a = 0; a < 5; ++a) {
         const R ja = a == 0 ? J0 : Ja;
-        gst<TG, R>(P, k, G + goff<NS>(node) + (k * 5 + a) * CELL, ja * c - ja * rp<R>(P).shift_c[k]);
+        gst<TG, R>(P, k, G + goff<NS>(node) + (k * 5 + a) * CELL, rfma<R>(ja, c, -rmul<R>(ja, rp<R>(P).shift_c[k])));
       }
     }
   }
@@ -365,8 +365,8 @@ __device__ __forceinline__ void amend(const DevInst* Ip) {
       const R w = w9<R>(a);
       TF* p1 = F + foff(n) + a * CELL;
       TF* p2 = F + foff(n) + (9 + a) * CELL;
-      st<TF, R>(p1, ld<R>(p1) + w * add1);
-      st<TF, R>(p2, ld<R>(p2) + w * add2);
+      st<TF, R>(p1, rfma<R>(w, add1, ld<R>(p1)));
+      st<TF, R>(p2, rfma<R>(w, add2, ld<R>(p2)));
     }
     if (nliq) {
 #pragma unroll
@@ -375,7 +375,7 @@ __device__ __forceinline__ void amend(const DevInst* Ip) {
 #pragma unroll
         for (int a = 0; a < 5; ++a) {
           TG* p = G + goff<NS>(n) + (k * 5 + a) * CELL;
-          gst<TG, R>(P, k, p, gld<R>(P, k, p) + (a == 0 ? J0 : Ja) * addc[k]);
+          gst<TG, R>(P, k, p, rfma<R>(a == 0 ? J0 : Ja, addc[k], gld<R>(P, k, p)));
         }
       }
     }

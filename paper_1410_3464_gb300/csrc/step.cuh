@@ -619,11 +619,11 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 2 : 4)
     const PR q = mk<R>(q1, q2);
     R upx, upy;
     if (sizeof(R) == 8 && Q.tau_unit) {
-      upx = (jx.a + jx.b) * rrt;
-      upy = (jy.a + jy.b) * rrt;
-      const R h = R(0.5) * rrt;
-      urx = rfma<R>(h, Fx.a + Fx.b, upx);
-      ury = rfma<R>(h, Fy.a + Fy.b, upy);
+      upx = rmul<R>(radd<R>(jx.a, jx.b), rrt);
+      upy = rmul<R>(radd<R>(jy.a, jy.b), rrt);
+      const R h = rmul<R>(R(0.5), rrt);
+      urx = rfma<R>(h, radd<R>(Fx.a, Fx.b), upx);
+      ury = rfma<R>(h, radd<R>(Fy.a, Fy.b), upy);
     } else {
       upx = u_common<R>(jx.a, jx.b, it1, it2, rden);
       upy = u_common<R>(jy.a, jy.b, it1, it2, rden);
