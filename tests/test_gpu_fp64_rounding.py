@@ -139,3 +139,38 @@ def test_one_solute_step_is_correctly_rounded(pslbm, tau_g):
     S = -(p["k1"] * C)
     go = [fma(J[a], S, fma(ge[a] - J[a] * conc[0], 1.0 / tau_g, J[a] * conc[0])) for a in range(5)]
     np.testing.assert_array_equal(got["conc"][0], streamed_sum(go, E9))
+
+
+def test_potentials_of_eq_15(pslbm):
+    """phi_1 = 1 - exp(-x), x = rho_2 / rho_20, is a series below 1/16; phi_2 = a0 -
+    exp(-z), z = rho_1 / rho_10, is a0 where the exponential is below half an ulp of it.
+    Sources (rho_2 > 0) stand alone in fours, so that the velocity of the node east of
+    one is G21 phi_2 (own) phi_1 (source) / 9 / (2 rho_1).  Bounds: phi_1 to an ulp, phi_2
+    to an ulp of a0 + exp(-z) and the rounding of z, and six roundings more."""
+    n = 64
+    p = inputs.base_params(n, n)
+    p.update(periodic_x=1, periodic_y=1, n_species=0, idx_A=-1, idx_B=-1, idx_E=-1, idx_F=-1, G11=0.0, G12=0.0, G21=1.0,
+             w_adh=(0.0, 0.0), body_force=(0.0, 0.0))
+    m = n // 4
+    k = m * m
+    cut = math.log(2.0 ** 55 / p["a0"])
+    x = np.concatenate([np.geomspace(1e-12, 0.06, k // 2), 0.0625 * (1 + np.linspace(-1e-3, 1e-3, k // 4)),
+                        np.nextafter(0.0625, [0, 1]), np.geomspace(0.063, 30.0, k - k // 2 - k // 4 - 2)])
+    z = np.concatenate([np.geomspace(1e-3, 30.0, k // 2), cut * (1 + np.linspace(-0.02, 0.02, k // 4)),
+                        np.linspace(cut + 1, 300.0, k - k // 2 - k // 4)])
+    z = np.random.default_rng(3).permutation(z)
+    rho1, rho2 = np.full((n, n), 0.1), np.zeros((n, n))
+    rho2[::4, 1::4] = (x * p["rho20"]).reshape(m, m)
+    rho1[::4, 2::4] = (z * p["rho10"]).reshape(m, m)
+    with pslbm.Simulation(np.zeros((n, n), np.uint8), p, rho1, rho2, None, None, precision=pslbm.FP64) as sim:
+        got = sim.read()
+    L = np.longdouble
+    r1, r2 = got["rho1"][::4, 2::4].astype(L), got["rho2"][::4, 1::4].astype(L)
+    ex = np.exp(-r1 / L(p["rho10"]))
+    phi1, phi2 = -np.expm1(-r2 / L(p["rho20"])), L(p["a0"]) - ex
+    want = phi2 * phi1 / 9 / (2 * r1)
+    eps = 2.0 ** -53
+    bound = eps * phi1 / 9 / (2 * r1) * (12 * np.abs(phi2) + 2 * p["a0"] + 2 * ex * (1 + 2 * r1 / L(p["rho10"])))
+    err = np.abs(got["ux"][::4, 2::4].astype(L) - want)
+    worst = np.unravel_index((err / bound).argmax(), err.shape)
+    assert (err <= bound).all(), (float((err / bound).max()), float(r2[worst] / p["rho20"]), float(r1[worst] / p["rho10"]))
