@@ -276,22 +276,18 @@ class Simulation:
         return int(b.value)
 
     def read(self, fields=F_RHO1 | F_RHO2 | F_UX | F_UY | F_CONC | F_TYPE | F_VOL | F_BUDGET):
-        """Read the selected fields into new numpy arrays (dict by name).  Of arrays
-        that the caller has let go of, the memory of two per field waits for the
-        next read, until close()."""
+        """Read the selected fields into new numpy arrays (dict by name), each with
+        memory of its own.  Of arrays over 1 MiB together that the caller has let go
+        of, the memory of two per field waits for the next read, until close()."""
         plan = self._reads.get(fields)
         if plan is None:
             plan = self._reads[fields] = self._read_plan(fields)
-        spec, at, total = plan
+        spec, total = plan
         if total <= 1 << 20:
-            # one behind the other in one allocation: the library copies what adjoins at once
-            mem = _touched(np.empty(max(1, total), np.uint8))
-            raw = [mem[o:o + n] for o, (_, _, _, n) in zip(at, spec)]
-            base = mem.ctypes.data
-            arr = (C.c_void_p * max(1, len(at)))(*[base + o for o in at])
+            raw = [np.empty(n, np.uint8) for _, _, _, n in spec]     # filled by the host
         else:
             raw = [self._memory(name, n) for name, _, _, n in spec]
-            arr = (C.c_void_p * len(raw))(*[a.ctypes.data for a in raw])
+        arr = (C.c_void_p * max(1, len(raw)))(*[a.ctypes.data for a in raw])
         _check(load().pslbm_read_fields(self.h, int(fields), arr), self.h)
         res = {name: a.view(dt).reshape(shp) for (name, dt, shp, _), a in zip(spec, raw)}
         if "vol" in res:
@@ -299,8 +295,7 @@ class Simulation:
         return res
 
     def _read_plan(self, fields):
-        """(name, type, shape, bytes) of the selected fields, their offsets in one
-        allocation (eight-byte items on eight-byte offsets) and its size."""
+        """(name, type, shape, bytes) of the selected fields, and their bytes together."""
         n = self.nx * self.ny
         shape = (self.ny, self.nx)
         spec = [(F_RHO1, "rho1", np.float64, shape, 8 * n), (F_RHO2, "rho2", np.float64, shape, 8 * n),
@@ -309,11 +304,7 @@ class Simulation:
                 (F_VOL, "vol", np.float64, (2,) + shape, 16 * n),
                 (F_BUDGET, "budget", np.float64, (6 + self.ns,), 8 * (6 + self.ns))]
         spec = [s[1:] for s in spec if fields & s[0]]
-        at, end = [], 0
-        for _, dt, _, size in spec:
-            at.append(end if dt is np.uint8 else (end + 7) // 8 * 8)
-            end = at[-1] + size
-        return spec, at, end
+        return spec, sum(s[3] for s in spec)
 
     def _memory(self, name, n):
         """n bytes for an array of read(): what an earlier array of that name has
