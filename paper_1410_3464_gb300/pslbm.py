@@ -9,7 +9,7 @@ from __future__ import annotations
 import ctypes as C
 import mmap
 import os
-from collections import deque
+import threading
 
 import numpy as np
 
@@ -187,6 +187,36 @@ def _touched(mem):
     return mem
 
 
+class _Spare:
+    """Memory of one array of one simulation that waits for the next read: the last
+    one given back, while all simulations together hold at most `most` bytes.  After
+    close() nothing is kept."""
+
+    most = 1 << 30
+    held = 0
+    lock = threading.RLock()      # give() may run as a collection starts inside take() or give()
+
+    def __init__(self):
+        self.mem, self.open = None, True
+
+    def take(self):
+        with _Spare.lock:
+            mem, self.mem = self.mem, None
+            if mem is not None:
+                _Spare.held -= mem.nbytes
+        return mem
+
+    def give(self, mem):
+        with _Spare.lock:
+            if self.open and self.mem is None and _Spare.held + mem.nbytes <= _Spare.most:
+                self.mem = mem
+                _Spare.held += mem.nbytes
+
+    def close(self):
+        self.open = False
+        self.take()
+
+
 class _Recycled:
     """Owner of an array's memory; gives it to `spare` when no view of it is left."""
 
@@ -195,7 +225,7 @@ class _Recycled:
         self.__array_interface__ = mem.__array_interface__
 
     def __del__(self):
-        self.spare.append(self.mem)
+        self.spare.give(self.mem)
 
 
 class Simulation:
@@ -278,7 +308,8 @@ class Simulation:
     def read(self, fields=F_RHO1 | F_RHO2 | F_UX | F_UY | F_CONC | F_TYPE | F_VOL | F_BUDGET):
         """Read the selected fields into new numpy arrays (dict by name), each with
         memory of its own.  Of arrays over 1 MiB together that the caller has let go
-        of, the memory of two per field waits for the next read, until close()."""
+        of, the memory of one per field waits for the next read, until close() (1 GiB
+        over all simulations)."""
         plan = self._reads.get(fields)
         if plan is None:
             plan = self._reads[fields] = self._read_plan(fields)
@@ -309,12 +340,9 @@ class Simulation:
     def _memory(self, name, n):
         """n bytes for an array of read(): what an earlier array of that name has
         left, else fresh pages."""
-        spare = self._spare.setdefault(name, deque(maxlen=2))
-        try:
-            mem = spare.pop()
-        except IndexError:
-            mem = np.empty(n, np.uint8)
-        return np.asarray(_Recycled(_touched(mem), spare))
+        spare = self._spare.setdefault(name, _Spare())
+        mem = spare.take()
+        return np.asarray(_Recycled(_touched(np.empty(n, np.uint8) if mem is None else mem), spare))
 
     def budget_device_noalloc(self, out_device_ptr):
         """Write the budget (6 + n_species doubles) to a caller-owned device
@@ -325,7 +353,8 @@ class Simulation:
         if getattr(self, "h", None):
             load().pslbm_destroy(self.h)
             self.h = None
-            self._spare = {}
+            for spare in self._spare.values():
+                spare.close()
 
     def __del__(self):
         try:
