@@ -116,13 +116,13 @@ struct DevInst {
   double* xs;                 // [N] overflow excess of an event node
   int* evlist;                // [evcap] event node indices
   int* claim;                 // [N] zero except while the amendment kernel runs
-  int* flist;                 // [N] fluid nodes (S_NFLUID entries; an entry may have filled since)
+  int* flist;                 // [N - nres] fluid nodes (S_NFLUID entries; an entry may have filled since)
   int* mlist;                 // [N] minerals with a fluid axis neighbour (S_NFACE entries; an entry may
                               // have lost its fluid neighbours, or dissolved, since)
   unsigned* fbits;            // [(N + 31) / 32] bit per node: listed in flist
   unsigned* mbits;            // [(N + 31) / 32] bit per node: listed in mlist
   unsigned long long* scal;   // [S_NSCAL]
-  int* reslist;               // [nres] reservoir nodes
+  int* reslist;               // [nres] reservoir nodes (behind flist)
   long long N;
   int evcap;
   int nres;

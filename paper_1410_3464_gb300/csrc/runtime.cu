@@ -732,7 +732,7 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
                             (size_t)N * sizeof(double), (size_t)N * 2 * sizeof(int), (size_t)N * sizeof(int),
                             (size_t)((N + 31) / 32) * 2 * sizeof(unsigned), S_NSCAL * sizeof(unsigned long long),
                             sizeof(DevInst), (size_t)((BUD_BLOCKS + 1) * NBUD + 2) * sizeof(double), (size_t)N * 4 * fsize(p->precision),
-                            (size_t)N, reslist.size() * sizeof(int), (size_t)N * 2 * sizeof(int)};
+                            (size_t)N, (size_t)N * 2 * sizeof(int)};
     constexpr int NPARTS = sizeof(sizes) / sizeof(sizes[0]);
     size_t offs[NPARTS], total = 0;
     for (int i = 0; i < NPARTS; ++i) {
@@ -756,13 +756,14 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     I.claim = (int*)(base + offs[10]);
     I.fbits = (unsigned*)(base + offs[11]);
     I.mbits = I.fbits + (N + 31) / 32;
-    I.flist = (int*)(base + offs[18]);
+    I.flist = (int*)(base + offs[17]);
     I.mlist = I.flist + N;
+    // a reservoir node never is fluid: its entry lies behind those of all nodes that may be
+    I.reslist = I.flist + (N - I.nres);
     I.scal = (unsigned long long*)(base + offs[12]);
     h->d = (DevInst*)(base + offs[13]);
     I.pot = base + offs[15];
     I.code = (uint8_t*)(base + offs[16]);
-    I.reslist = (int*)(base + offs[17]);
     double* part = (double*)(base + offs[14]);
     double* res = part + (size_t)BUD_BLOCKS * NBUD;
 
@@ -897,12 +898,11 @@ pslbm_status pslbm_estimate_device_bytes(const pslbm_params* p, uint64_t* bytes)
   const uint64_t per = 2 * 18 * fsize(p->precision) + 2 * 5 * (uint64_t)p->n_species * gsize(p->precision) +
                        2 /*types*/ + 4 * fsize(p->precision) + 1 /*potentials, codes*/ + 16 /*V*/ + 1 /*events*/ + 8 /*excess*/ + 8 /*event lists*/ + 4 /*claims*/ + 8 /*node lists*/;
   const uint64_t bits = ((N + 31) / 32) * 8;
-  // whole cells; reservoir nodes: the edges of the lattice
+  // whole cells
   const uint64_t cells = (N + CELL - 1) / CELL * CELL;
   const uint64_t pops = 2 * 18 * fsize(p->precision) + 2 * 5 * (uint64_t)p->n_species * gsize(p->precision);
-  const uint64_t res = 2 * ((uint64_t)p->nx + (uint64_t)p->ny) * sizeof(int);
-  *bytes = N * per + (cells - N) * pops + bits + res + sizeof(DevInst) + S_NSCAL * 8 +
-           (uint64_t)((BUD_BLOCKS + 1) * NBUD + 2) * sizeof(double) + 19 * 256;
+  *bytes = N * per + (cells - N) * pops + bits + sizeof(DevInst) + S_NSCAL * 8 +
+           (uint64_t)((BUD_BLOCKS + 1) * NBUD + 2) * sizeof(double) + 18 * 256;
   return PSLBM_OK;
 }
 
