@@ -109,12 +109,12 @@ struct DevInst {
   void* f[2];                 // populations in cells (foff), ping-pong
   void* g[2];                 // solute populations in cells (goff), ping-pong
   uint8_t* type[2];           // [N] node types, ping-pong
-  void* pot;                  // [N] potentials of this step (Pot<R>)
+  void* pot;                  // [N] potentials of this step (Pot<R>), until the VOP kernel
   uint8_t* code;              // [N] codes of this step (C_* bits)
   double* V;                  // [2][N] V_D, V_F
   uint8_t* evt;               // [N] VOP events (zero except during a step)
-  double* xs;                 // [N] overflow excess of an event node
-  int* evlist;                // [evcap] event node indices
+  double* xs;                 // [N] overflow excess of an event node (in the bytes of pot)
+  int* evlist;                // [2 evcap] event node indices, vanishing nodes (in the bytes of pot)
   int* claim;                 // [N] zero except while the amendment kernel runs
   int* flist;                 // [N - nres] fluid nodes (S_NFLUID entries; an entry may have filled since)
   int* mlist;                 // [N] minerals with a fluid axis neighbour (S_NFACE entries; an entry may

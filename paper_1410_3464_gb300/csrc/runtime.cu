@@ -729,7 +729,7 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     I.nres = (int)reslist.size();
     I.read_once = read_once(2 * (fb + gb)) ? 1 : 0;
     const size_t sizes[] = {fb, fb, gb, gb, (size_t)N, (size_t)N, (size_t)N * 2 * sizeof(double), (size_t)N,
-                            (size_t)N * sizeof(double), (size_t)N * 2 * sizeof(int), (size_t)N * sizeof(int),
+                            (size_t)N * sizeof(int),
                             (size_t)((N + 31) / 32) * 2 * sizeof(unsigned), S_NSCAL * sizeof(unsigned long long),
                             sizeof(DevInst), (size_t)((BUD_BLOCKS + 1) * NBUD + 2) * sizeof(double), (size_t)N * 4 * fsize(p->precision),
                             (size_t)N, (size_t)N * 2 * sizeof(int)};
@@ -751,20 +751,23 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     I.type[1] = (uint8_t*)(base + offs[5]);
     I.V = (double*)(base + offs[6]);
     I.evt = (uint8_t*)(base + offs[7]);
-    I.xs = (double*)(base + offs[8]);
-    I.evlist = (int*)(base + offs[9]);
-    I.claim = (int*)(base + offs[10]);
-    I.fbits = (unsigned*)(base + offs[11]);
+    I.claim = (int*)(base + offs[8]);
+    I.fbits = (unsigned*)(base + offs[9]);
     I.mbits = I.fbits + (N + 31) / 32;
-    I.flist = (int*)(base + offs[17]);
+    I.scal = (unsigned long long*)(base + offs[10]);
+    h->d = (DevInst*)(base + offs[11]);
+    I.pot = base + offs[13];
+    // the potentials are done with before the VOP kernel runs, and its events with the
+    // amendment before the next potentials: both in the same bytes
+    I.xs = (double*)I.pot;
+    I.evlist = (int*)(I.xs + N);
+    static_assert(4 * sizeof(float) >= sizeof(double) + 2 * sizeof(int), "room for xs and evlist");
+    I.code = (uint8_t*)(base + offs[14]);
+    I.flist = (int*)(base + offs[15]);
     I.mlist = I.flist + N;
     // a reservoir node never is fluid: its entry lies behind those of all nodes that may be
     I.reslist = I.flist + (N - I.nres);
-    I.scal = (unsigned long long*)(base + offs[12]);
-    h->d = (DevInst*)(base + offs[13]);
-    I.pot = base + offs[15];
-    I.code = (uint8_t*)(base + offs[16]);
-    double* part = (double*)(base + offs[14]);
+    double* part = (double*)(base + offs[12]);
     double* res = part + (size_t)BUD_BLOCKS * NBUD;
 
     // the inputs are staged in the second population buffer (at least 72
@@ -896,13 +899,13 @@ pslbm_status pslbm_estimate_device_bytes(const pslbm_params* p, uint64_t* bytes)
   if (!v.empty()) return fail(nullptr, PSLBM_ERR_PARAM, v);
   const uint64_t N = (uint64_t)p->nx * (uint64_t)p->ny;
   const uint64_t per = 2 * 18 * fsize(p->precision) + 2 * 5 * (uint64_t)p->n_species * gsize(p->precision) +
-                       2 /*types*/ + 4 * fsize(p->precision) + 1 /*potentials, codes*/ + 16 /*V*/ + 1 /*events*/ + 8 /*excess*/ + 8 /*event lists*/ + 4 /*claims*/ + 8 /*node lists*/;
+                       2 /*types*/ + 4 * fsize(p->precision) + 1 /*potentials, codes*/ + 16 /*V*/ + 1 /*events*/ + 4 /*claims*/ + 8 /*node lists*/;
   const uint64_t bits = ((N + 31) / 32) * 8;
   // whole cells
   const uint64_t cells = (N + CELL - 1) / CELL * CELL;
   const uint64_t pops = 2 * 18 * fsize(p->precision) + 2 * 5 * (uint64_t)p->n_species * gsize(p->precision);
   *bytes = N * per + (cells - N) * pops + bits + sizeof(DevInst) + S_NSCAL * 8 +
-           (uint64_t)((BUD_BLOCKS + 1) * NBUD + 2) * sizeof(double) + 18 * 256;
+           (uint64_t)((BUD_BLOCKS + 1) * NBUD + 2) * sizeof(double) + 16 * 256;
   return PSLBM_OK;
 }
 

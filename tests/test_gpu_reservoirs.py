@@ -1,5 +1,5 @@
-"""Reservoir nodes anywhere in the lattice: the device bytes stay within the estimate by
-which a server admits, and the steps agree with the oracle."""
+"""Device bytes of a simulation, by which a server admits, and reservoir nodes anywhere
+in the lattice: the bytes stay within the estimate, and the steps agree with the oracle."""
 import numpy as np
 import pytest
 
@@ -26,6 +26,20 @@ def test_device_bytes_within_the_estimate(pslbm, nx, ny, share):
     for precision in (pslbm.FP64, pslbm.FP32):
         with pslbm.Simulation(mask, p, rho1, rho2, None, None, precision=precision) as sim:
             assert sim.device_bytes() <= pslbm.estimate_device_bytes(p, precision)
+
+
+@pytest.mark.parametrize("precision,beside", [(0, 65), (1, 49), (2, 49), (3, 49)])
+def test_bytes_a_node(pslbm, precision, beside):
+    """What a node takes beside its populations: two types, two volumes, potentials
+    (their bytes hold the events too), a code, an event code, two lists, a claim and
+    two bits: 64.25 bytes in FP64, 48.25 in FP32."""
+    sc = inputs.porous_discs(nx=512, ny=256, seed=1)
+    n = 512 * 256
+    per = 2 * 18 * (4 if precision else 8) + 2 * 5 * 3 * (8, 4, 2, 2)[precision] + beside
+    fixed = 64 * 1024
+    assert pslbm.estimate_device_bytes(sc["params"], precision) <= n * per + fixed
+    with pslbm.Simulation(sc["mask"], sc["params"], sc["rho1"], sc["rho2"], sc["conc"], None, precision=precision) as sim:
+        assert sim.device_bytes() <= n * per + fixed
 
 
 @pytest.mark.parametrize("axis", ["x", "y"])
