@@ -35,7 +35,8 @@ enum {
   S_THETAF = 7,    // the same rounded to FP32 (bits in the low word)
   S_NFLUID = 8,    // entries of the fluid list
   S_NFACE = 9,     // entries of the list of minerals facing fluid
-  S_NSCAL = 10
+  S_NRES = 10,     // reservoir nodes (set at creation)
+  S_NSCAL = 11
 };
 enum { ST_NONFINITE = 1, ST_EOS = 2, ST_EVOVERFLOW = 4 };
 
@@ -116,16 +117,15 @@ struct DevInst {
   double* xs;                 // [N] overflow excess of an event node (in the bytes of pot)
   int* evlist;                // [2 evcap] event node indices, vanishing nodes (in the bytes of pot)
   int* claim;                 // [N] zero except while the amendment kernel runs
-  int* flist;                 // [N - nres] fluid nodes (S_NFLUID entries; an entry may have filled since)
+  int* flist;                 // [N] fluid nodes (S_NFLUID entries from the front; an entry may have filled
+                              // since); reservoir nodes (S_NRES entries) from the back (reservoir_node)
   int* mlist;                 // [N] minerals with a fluid axis neighbour (S_NFACE entries; an entry may
                               // have lost its fluid neighbours, or dissolved, since)
   unsigned* fbits;            // [(N + 31) / 32] bit per node: listed in flist
   unsigned* mbits;            // [(N + 31) / 32] bit per node: listed in mlist
   unsigned long long* scal;   // [S_NSCAL]
-  int* reslist;               // [nres] reservoir nodes (behind flist)
   long long N;
   int evcap;
-  int nres;
   int read_once;              // populations may leave L2 once k_move has read them (pslbm_create)
 };
 

@@ -716,17 +716,12 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
   I.N = N;
   I.evcap = (int)N;
   pslbm_status st = PSLBM_OK;
-  std::vector<int> reslist;
   {
     // one device allocation holds the instance's whole state, each part on a
     // 256-byte boundary; the initial
     // threshold's budget partial sums are the last part
     const size_t NP = (size_t)(N + CELL - 1) / CELL * CELL;   // whole cells
     const size_t fb = NP * 18 * fsize(p->precision), gb = NP * 5 * ns * gsize(p->precision);
-    // the reservoir nodes (their types never change)
-    for (long long i = 0; i < N; ++i)
-      if ((mask[i] & 15) >= PSLBM_INLET && (mask[i] & 15) <= PSLBM_OUTLET) reslist.push_back((int)i);
-    I.nres = (int)reslist.size();
     I.read_once = read_once(2 * (fb + gb)) ? 1 : 0;
     const size_t sizes[] = {fb, fb, gb, gb, (size_t)N, (size_t)N, (size_t)N * 2 * sizeof(double), (size_t)N,
                             (size_t)N * sizeof(int),
@@ -765,8 +760,6 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     I.code = (uint8_t*)(base + offs[14]);
     I.flist = (int*)(base + offs[15]);
     I.mlist = I.flist + N;
-    // a reservoir node never is fluid: its entry lies behind those of all nodes that may be
-    I.reslist = I.flist + (N - I.nres);
     double* part = (double*)(base + offs[12]);
     double* res = part + (size_t)BUD_BLOCKS * NBUD;
 
@@ -795,8 +788,6 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
         e = cudaGetLastError();
       }
     }
-    if (e == cudaSuccess && I.nres)
-      e = cudaMemcpyAsync(I.reslist, reslist.data(), reslist.size() * sizeof(int), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d, &I, sizeof(DevInst), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
       L->init(s, h->d, dmask, dr1, dr2, dc, N);
@@ -819,13 +810,13 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     // the host copy of the descriptor is read by the copy above before the
     // call returns only for pageable memory; synchronise once for it and for
     // the errors of everything above
-    unsigned long long counts[2] = {0, 0};
-    static_assert(S_NFACE == S_NFLUID + 1, "read together");
+    unsigned long long counts[3] = {0, 0, 0};
+    static_assert(S_NFACE == S_NFLUID + 1 && S_NRES == S_NFACE + 1, "read together");
     if (e == cudaSuccess) e = cudaMemcpyAsync(counts, I.scal + S_NFLUID, sizeof counts, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     h->run.nfluid.assign(1, (int)counts[0]);
     h->run.nface.assign(1, (int)counts[1]);
-    h->run.nres.assign(1, I.nres);
+    h->run.nres.assign(1, (int)counts[2]);
     if (e != cudaSuccess) {
       st = fail(nullptr, e == cudaErrorMemoryAllocation ? PSLBM_ERR_OOM : PSLBM_ERR_CUDA,
                 std::string("create: ") + cudaGetErrorString(e));
@@ -942,7 +933,7 @@ pslbm_status pslbm_get_staging(pslbm_t h, int32_t* staged, int32_t* available) {
 pslbm_status pslbm_monitor(pslbm_t h, int64_t* steps, double* max_rho1, uint32_t* status) {
   if (!h) return fail(nullptr, PSLBM_ERR_PARAM, "handle is NULL");
   if (h->sticky) return h->sticky;
-  unsigned long long sc[S_NSCAL];
+  unsigned long long sc[S_STATUS + 1];
   CK(h, cudaMemcpyAsync(sc, h->h.scal, sizeof sc, cudaMemcpyDeviceToHost, lib_stream()));
   CK(h, cudaStreamSynchronize(lib_stream()));
   const unsigned long long n = sc[S_STEP];

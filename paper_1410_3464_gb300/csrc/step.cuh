@@ -135,8 +135,8 @@ __device__ __forceinline__ bool step_work(bool single, const Work* __restrict__ 
   return true;
 }
 
-// The fluid list and the list of minerals with a fluid axis neighbour, from the
-// node types (creation).  Both go through the lattice by tiles of 32 columns and
+// The fluid list, the list of minerals with a fluid axis neighbour and the reservoir
+// nodes (in any order), from the node types (creation).  The first two go through the lattice by tiles of 32 columns and
 // 8 rows, row by row within a tile, so that a warp's chunk of the list stays
 // together on the lattice (4096x2048 FP32: 612 us a step, 717 to 766 with the tiles
 // in the order of an atomic counter): k_list<false> counts a tile's nodes (a warp a tile),
@@ -177,6 +177,14 @@ static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constan
         I.mlist[bm + __popc(mm & below)] = node;
         atomicOr(&I.mbits[node >> 5], 1u << (node & 31));
       }
+      const bool res = t == T_INLET || t == T_OUTLET;
+      const unsigned mr = __ballot_sync(FULL, res);
+      if (mr) {
+        int at = 0;
+        if (lane == 0) at = (int)atomicAdd(&I.scal[S_NRES], (unsigned long long)__popc(mr));
+        at = __shfl_sync(FULL, at, 0);
+        if (res) I.flist[I.N - 1 - (at + __popc(mr & below))] = node;
+      }
     }
     bf += __popc(mf);
     bm += __popc(mm);
@@ -214,14 +222,18 @@ static __global__ void __launch_bounds__(1024) k_list_scan(int* __restrict__ cou
   }
 }
 
+// Reservoir node i of an instance.  A reservoir node never is fluid, so the array of
+// the fluid list has room for it.
+__device__ __forceinline__ int reservoir_node(const DevInst* I, int i) { return I->flist[I->N - 1 - i]; }
+
 // Reservoir nodes i .. i + 31 of an instance: densities of the step, potentials
 // and codes.
 template <class TF, class R>
 __device__ __noinline__ void reservoir_pot(const DevInst* I, int cur, unsigned long long step, int i) {
   i += threadIdx.x & 31;
-  if (i >= I->nres) return;
+  if (i >= (int)I->scal[S_NRES]) return;
   const DevParams& P = I->P;
-  const int node = I->reslist[i];
+  const int node = reservoir_node(I, i);
   const uint8_t* tin = I->type[cur];
   const uint8_t t = tin[node] & T_MASK;
   const R theta = theta_of<R>(I);
@@ -401,9 +413,9 @@ __device__ __forceinline__ void reservoir_push_node(const DevParams& P, const ui
 template <class TF, class TG, class R, int NS>
 __device__ __noinline__ void reservoir_push(const DevInst* I, int cur, unsigned long long step, int i) {
   i += threadIdx.x & 31;
-  if (i >= I->nres) return;
+  if (i >= (int)I->scal[S_NRES]) return;
   const DevParams& P = I->P;
-  const int node = I->reslist[i], N = (int)I->N;
+  const int node = reservoir_node(I, i), N = (int)I->N;
   const uint8_t* tin = I->type[cur];
   const TF* fin = (const TF*)I->f[cur];
   const uint8_t t = tin[node] & T_MASK;

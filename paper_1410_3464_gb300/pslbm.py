@@ -287,7 +287,7 @@ class Simulation:
 
     def monitor(self):
         """(steps taken, maximum rho_1 found by the last step, status bits):
-        an 80-byte read, no kernel."""
+        a 32-byte read, no kernel."""
         n, m, st = C.c_int64(), C.c_double(), C.c_uint32()
         _check(load().pslbm_monitor(self.h, C.byref(n), C.byref(m), C.byref(st)), self.h)
         return n.value, m.value, st.value
