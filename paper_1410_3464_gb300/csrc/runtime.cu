@@ -59,7 +59,11 @@ struct Stepper {
   DevInst* d = nullptr;
   int ninst = 0;
   std::vector<std::pair<int, int>> dims;   // (nx, ny) per instance
-  std::vector<int> nfluid, nface, nres;    // listed nodes and reservoirs per instance, as created
+  std::vector<const DevInst*> inst;        // host descriptors
+  std::vector<int> nfluid, nface, nres;    // listed nodes and reservoirs per instance, as last seen
+  long long plan_fluid = 0, plan_face = 0; // their sums when the work was laid out
+  bool plan_fused = false;                 // VOP and amendment in one launch
+  int64_t since = 0;                       // steps since the lists were made
   DevInst host0{};                         // host descriptor of the first instance
   int mode = M_SINGLE;
   bool fp64 = false;
@@ -425,12 +429,37 @@ double stream_turns(const Stepper& st, bool pot) {
   return turns;
 }
 
+// Whether every list of minerals is short enough for one launch of VOP and amendment
+// with a block an instance (k_vop_amend); a plan that has it keeps it for half as much
+// more, or a list around the line would have its plan changed over and over.
+bool fused(const Stepper& st) {
+  return *std::max_element(st.nface.begin(), st.nface.end()) <= (st.plan_fused ? FUSE_FACE + FUSE_FACE / 2 : FUSE_FACE);
+}
+
+// Whether the lists, as last seen, ask for another plan than the one there is: an eighth
+// longer (list_warps leaves that much room), half as long, or across the line of `fused`.
+bool outgrown(const Stepper& st) {
+  auto sum = [](const std::vector<int>& v) {
+    long long n = 0;
+    for (int k : v) n += k;
+    return n;
+  };
+  auto off = [](long long n, long long plan) { return n > plan + std::max(2048LL, plan / 8) || n < plan / 2; };
+  return off(sum(st.nfluid), st.plan_fluid) || off(sum(st.nface), st.plan_face) || fused(st) != st.plan_fused;
+}
+
 // Work entries of the streaming kernels (parts of the fluid lists, then chunks of
-// 32 reservoir nodes) and of the VOP kernel.
+// 32 reservoir nodes) and of the VOP kernel.  A plan that the lists have outgrown is
+// made again; without memory for it the one there is goes on.
 cudaError_t ensure_work(Stepper& st) {
-  if (st.nwork) return cudaSuccess;
+  if (st.nwork && !outgrown(st)) return cudaSuccess;
+  st.plan_fluid = st.plan_face = 0;
+  for (int k : st.nfluid) st.plan_fluid += k;
+  for (int k : st.nface) st.plan_face += k;
+  st.plan_fused = fused(st);
   auto nodes = [&](int i) { return (long long)st.dims[i].first * st.dims[i].second; };
   if (st.mode == M_SINGLE) {
+    st.graphs.clear();
     st.npot = list_warps(st.nfluid[0], nodes(0), stream_turns(st, true));
     st.nstream = list_warps(st.nfluid[0], nodes(0), stream_turns(st, false));
     st.nwork = st.nstream + (st.nres[0] + 31) / 32;
@@ -451,6 +480,10 @@ cudaError_t ensure_work(Stepper& st) {
   }
   Work* d = nullptr;
   cudaError_t e = cudaMalloc(&d, all.size() * sizeof(Work));
+  if (e == cudaErrorMemoryAllocation && st.nwork) {
+    cudaGetLastError();
+    return cudaSuccess;
+  }
   if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(d, all.data(), all.size() * sizeof(Work), cudaMemcpyHostToDevice, lib_stream());
   if (e == cudaSuccess) e = cudaStreamSynchronize(lib_stream());
@@ -458,6 +491,7 @@ cudaError_t ensure_work(Stepper& st) {
     cudaFree(d);
     return e;
   }
+  st.drop_work();
   st.work = d;
   st.nwork = nwork;
   st.nvop = (int)all.size() - nwork;
@@ -494,11 +528,9 @@ void enqueue_stream(cudaStream_t s, const Stepper& st) {
 
 // Enqueue the kernels of n steps.
 void enqueue_steps(cudaStream_t s, const Stepper& st, int64_t n) {
-  // every list within one block: VOP and amendment in one launch (k_vop_amend)
-  const bool fused = *std::max_element(st.nface.begin(), st.nface.end()) <= FUSE_FACE;
   for (int64_t i = 0; i < n; ++i) {
     enqueue_stream(s, st);
-    if (fused) {
+    if (st.plan_fused) {
       st.L->vop_amend(s, st.ninst, st.d);
       continue;
     }
@@ -587,6 +619,25 @@ __global__ void k_batch_monitor(const DevInst* __restrict__ insts, int n, unsign
   }
 }
 
+// Enqueue the kernels that make an instance's lists from its node types; the counts of
+// the tiles go where the events go, of which there are none between steps.
+cudaError_t make_lists(cudaStream_t s, const DevInst& I, bool reservoirs) {
+  cudaError_t e = cudaMemsetAsync(I.fbits, 0, (size_t)((I.N + 31) / 32) * 2 * sizeof(unsigned), s);
+  if (e != cudaSuccess) return e;
+  const int tiles = ((I.P.nx + 31) / 32) * ((I.P.ny + 7) / 8);
+  const int blocks = (tiles + ST_WARPS - 1) / ST_WARPS;
+  k_list<false><<<blocks, ST_THREADS, 0, s>>>(I, I.evlist, tiles, reservoirs);
+  k_list_scan<<<1, 1024, 0, s>>>(I.evlist, tiles, I.scal);
+  k_list<true><<<blocks, ST_THREADS, 0, s>>>(I, I.evlist, tiles, reservoirs);
+  return cudaGetLastError();
+}
+
+// Steps after which the lists are made again.  They only grow: nodes that dissolve join
+// the fluid list out of order and stay on the list of minerals, so that a step takes
+// ever longer (100x160 FP32, 1,500 of 13,000 minerals dissolved in 17,000 steps: 19.4 us, with
+// new lists 15.8).  Making them takes an instance's share of some 10 us, four launches.
+int64_t list_life(const Stepper& st) { return 1024LL * std::max(1, st.ninst / 16); }
+
 // Run n steps, replaying captured graphs of up to 32 steps.
 pslbm_status run_steps(Stepper& st, int64_t n, std::string& err) {
   cudaStream_t s = lib_stream();
@@ -628,6 +679,17 @@ pslbm_status run_steps(Stepper& st, int64_t n, std::string& err) {
       return PSLBM_ERR_CUDA;
     }
     n -= k;
+    st.since += k;
+    if (st.since < list_life(st)) continue;
+    st.since = 0;
+    for (size_t i = 0; i < st.inst.size(); ++i) {
+      if (!st.nface[i]) continue;       // no mineral that faces fluid: nothing changes
+      e = make_lists(s, *st.inst[i], false);
+      if (e != cudaSuccess) {
+        err = std::string("node lists: ") + cudaGetErrorString(e);
+        return PSLBM_ERR_CUDA;
+      }
+    }
   }
   return PSLBM_OK;
 }
@@ -671,11 +733,14 @@ pslbm_status status_of(pslbm_t h, unsigned long long st) {
   return PSLBM_OK;
 }
 
+// Status bits; the lengths of the lists, which a step's plan depends on, come along.
 pslbm_status device_status(pslbm_t h) {
-  unsigned long long st = 0;
-  CK(h, cudaMemcpyAsync(&st, h->h.scal + S_STATUS, sizeof st, cudaMemcpyDeviceToHost, lib_stream()));
+  unsigned long long sc[S_NFACE + 1];
+  CK(h, cudaMemcpyAsync(sc, h->h.scal, sizeof sc, cudaMemcpyDeviceToHost, lib_stream()));
   CK(h, cudaStreamSynchronize(lib_stream()));
-  return status_of(h, st);
+  h->run.nfluid[0] = (int)sc[S_NFLUID];
+  h->run.nface[0] = (int)sc[S_NFACE];
+  return status_of(h, sc[S_STATUS]);
 }
 
 }  // namespace
@@ -776,7 +841,6 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     if (e == cudaSuccess && dc) e = cudaMemcpyAsync(dc, conc, N * ns * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(I.evt, 0, (size_t)N, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(I.claim, 0, (size_t)N * sizeof(int), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(I.fbits, 0, (size_t)((N + 31) / 32) * 2 * sizeof(unsigned), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(I.scal, 0, S_NSCAL * sizeof(unsigned long long), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(I.scal + S_LIMIT, 0xff, sizeof(unsigned long long), s);
     if (e == cudaSuccess && ns) e = cudaMemsetAsync(I.g[1], 0, gb, s);
@@ -791,13 +855,7 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d, &I, sizeof(DevInst), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
       L->init(s, h->d, dmask, dr1, dr2, dc, N);
-      // node lists (the tile counts use the event list, empty between steps)
-      const int tiles = ((p->nx + 31) / 32) * ((p->ny + 7) / 8);
-      const int blocks = (tiles + ST_WARPS - 1) / ST_WARPS;
-      k_list<false><<<blocks, ST_THREADS, 0, s>>>(I, I.evlist, tiles);
-      k_list_scan<<<1, 1024, 0, s>>>(I.evlist, tiles, I.scal);
-      k_list<true><<<blocks, ST_THREADS, 0, s>>>(I, I.evlist, tiles);
-      e = cudaGetLastError();
+      e = make_lists(s, I, true);
     }
     // initial liquid threshold: half the maximum initial rho_1 over fluid
     // nodes (the first budget entry), decoded on the device
@@ -828,6 +886,7 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
   h->run.ninst = 1;
   h->run.dims.assign(1, {p->nx, p->ny});
   h->run.host0 = h->h;
+  h->run.inst.assign(1, &h->h);
   h->run.fp64 = p->precision == PSLBM_FP64;
   h->run.staged_ok = staging_open(p);
   {
@@ -1148,6 +1207,8 @@ pslbm_status pslbm_batch_create(int32_t n, const pslbm_t* members, int32_t tile_
     b->run.nfluid.push_back(members[i]->run.nfluid[0]);
     b->run.nface.push_back(members[i]->run.nface[0]);
     b->run.nres.push_back(members[i]->run.nres[0]);
+    b->run.inst.push_back(&members[i]->h);
+    b->run.since = std::max(b->run.since, members[i]->run.since);
     if (!same_hot_params(members[i]->h.P, members[0]->h.P)) b->run.mode = M_MIXED;
   }
   if (e == cudaSuccess) e = ensure_work(b->run);
@@ -1168,6 +1229,10 @@ pslbm_status pslbm_batch_step(pslbm_batch_t b, int64_t n) {
   if (b->sticky) return b->sticky;
   if (n < 0) return fail(nullptr, PSLBM_ERR_PARAM, "n < 0");
   if (n == 0) return PSLBM_OK;
+  for (size_t i = 0; i < b->members.size(); ++i) {
+    b->run.nfluid[i] = b->members[i]->run.nfluid[0];
+    b->run.nface[i] = b->members[i]->run.nface[0];
+  }
   std::string err;
   pslbm_status st = run_steps(b->run, n, err);
   if (st != PSLBM_OK) {
@@ -1263,7 +1328,10 @@ pslbm_status pslbm_batch_destroy(pslbm_batch_t b) {
   b->run.release();
   if (b->d) cudaFree(b->d);
   if (b->mon) cudaFree(b->mon);
-  for (pslbm_t m : b->members) m->in_batch = 0;
+  for (pslbm_t m : b->members) {
+    m->in_batch = 0;
+    m->run.since = b->run.since;
+  }
   delete b;
   return PSLBM_OK;
 }

@@ -135,21 +135,21 @@ __device__ __forceinline__ bool step_work(bool single, const Work* __restrict__ 
   return true;
 }
 
-// The fluid list, the list of minerals with a fluid axis neighbour and the reservoir
-// nodes (in any order), from the node types (creation).  The first two go through the lattice by tiles of 32 columns and
+// The fluid list, the list of minerals with a fluid axis neighbour and, at creation, the
+// reservoir nodes (in any order), from the node types.  The first two go through the lattice by tiles of 32 columns and
 // 8 rows, row by row within a tile, so that a warp's chunk of the list stays
 // together on the lattice (4096x2048 FP32: 612 us a step, 717 to 766 with the tiles
 // in the order of an atomic counter): k_list<false> counts a tile's nodes (a warp a tile),
 // k_list_scan turns the counts into positions, k_list<true> writes the lists.
 template <bool FILL>
-static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constant__ DevInst I, int* __restrict__ counts, int ntiles) {
+static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constant__ DevInst I, int* __restrict__ counts, int ntiles, bool reservoirs) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int nx = I.P.nx, ny = I.P.ny, ncx = (nx + 31) >> 5;
   const int ti = blockIdx.x * ST_WARPS + (threadIdx.x >> 5);
   if (ti >= ntiles) return;
   const int y0 = ti / ncx * 8, x = (ti % ncx) * 32 + lane;
-  const uint8_t* type = I.type[0];
+  const uint8_t* type = I.type[int(I.scal[S_STEP] & 1ULL)];
   int bf = FILL ? counts[ti] : 0, bm = FILL ? counts[ntiles + ti] : 0;
   const unsigned below = (1u << lane) - 1u;
 #pragma unroll 4
@@ -177,7 +177,7 @@ static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constan
         I.mlist[bm + __popc(mm & below)] = node;
         atomicOr(&I.mbits[node >> 5], 1u << (node & 31));
       }
-      const bool res = t == T_INLET || t == T_OUTLET;
+      const bool res = reservoirs && (t == T_INLET || t == T_OUTLET);
       const unsigned mr = __ballot_sync(FULL, res);
       if (mr) {
         int at = 0;
