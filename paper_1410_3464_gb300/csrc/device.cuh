@@ -118,7 +118,7 @@ struct DevInst {
   int* evlist;                // [2 evcap] event node indices, vanishing nodes (in the bytes of pot)
   int* claim;                 // [N] zero except while the amendment kernel runs
   int* flist;                 // [N] fluid nodes (S_NFLUID entries from the front; an entry may have filled
-                              // since); reservoir nodes (S_NRES entries) from the back (reservoir_node)
+                              // since); reservoir nodes (S_NRES entries) at its end (reservoir_node)
   int* mlist;                 // [N] minerals with a fluid axis neighbour (S_NFACE entries; an entry may
                               // have lost its fluid neighbours, or dissolved, since)
   unsigned* fbits;            // [(N + 31) / 32] bit per node: listed in flist

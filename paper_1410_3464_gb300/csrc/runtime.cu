@@ -619,16 +619,18 @@ __global__ void k_batch_monitor(const DevInst* __restrict__ insts, int n, unsign
   }
 }
 
-// Enqueue the kernels that make an instance's lists from its node types; the counts of
-// the tiles go where the events go, of which there are none between steps.
-cudaError_t make_lists(cudaStream_t s, const DevInst& I, bool reservoirs) {
+// Enqueue the kernels that make an instance's lists from its node types (kinds 2: of
+// fluid and of minerals, 3: of reservoirs too).  The counts of the tiles, at most 12
+// bytes a node, go where the potentials go, which are not needed between steps.
+cudaError_t make_lists(cudaStream_t s, const DevInst& I, int kinds) {
   cudaError_t e = cudaMemsetAsync(I.fbits, 0, (size_t)((I.N + 31) / 32) * 2 * sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
   const int tiles = ((I.P.nx + 31) / 32) * ((I.P.ny + 7) / 8);
   const int blocks = (tiles + ST_WARPS - 1) / ST_WARPS;
-  k_list<false><<<blocks, ST_THREADS, 0, s>>>(I, I.evlist, tiles, reservoirs);
-  k_list_scan<<<1, 1024, 0, s>>>(I.evlist, tiles, I.scal);
-  k_list<true><<<blocks, ST_THREADS, 0, s>>>(I, I.evlist, tiles, reservoirs);
+  int* counts = (int*)I.pot;
+  k_list<false><<<blocks, ST_THREADS, 0, s>>>(I, counts, tiles, kinds);
+  k_list_scan<<<1, 1024, 0, s>>>(counts, tiles, I.scal, kinds);
+  k_list<true><<<blocks, ST_THREADS, 0, s>>>(I, counts, tiles, kinds);
   return cudaGetLastError();
 }
 
@@ -684,7 +686,7 @@ pslbm_status run_steps(Stepper& st, int64_t n, std::string& err) {
     st.since = 0;
     for (size_t i = 0; i < st.inst.size(); ++i) {
       if (!st.nface[i]) continue;       // no mineral that faces fluid: nothing changes
-      e = make_lists(s, *st.inst[i], false);
+      e = make_lists(s, *st.inst[i], 2);
       if (e != cudaSuccess) {
         err = std::string("node lists: ") + cudaGetErrorString(e);
         return PSLBM_ERR_CUDA;
@@ -855,7 +857,7 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d, &I, sizeof(DevInst), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
       L->init(s, h->d, dmask, dr1, dr2, dc, N);
-      e = make_lists(s, I, true);
+      e = make_lists(s, I, 3);
     }
     // initial liquid threshold: half the maximum initial rho_1 over fluid
     // nodes (the first budget entry), decoded on the device

@@ -135,14 +135,14 @@ __device__ __forceinline__ bool step_work(bool single, const Work* __restrict__ 
   return true;
 }
 
-// The fluid list, the list of minerals with a fluid axis neighbour and, at creation, the
-// reservoir nodes (in any order), from the node types.  The first two go through the lattice by tiles of 32 columns and
+// The fluid list, the list of minerals with a fluid axis neighbour and, at creation
+// (kinds 3), the reservoir nodes, from the node types.  All go through the lattice by tiles of 32 columns and
 // 8 rows, row by row within a tile, so that a warp's chunk of the list stays
 // together on the lattice (4096x2048 FP32: 612 us a step, 717 to 766 with the tiles
 // in the order of an atomic counter): k_list<false> counts a tile's nodes (a warp a tile),
 // k_list_scan turns the counts into positions, k_list<true> writes the lists.
 template <bool FILL>
-static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constant__ DevInst I, int* __restrict__ counts, int ntiles, bool reservoirs) {
+static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constant__ DevInst I, int* __restrict__ counts, int ntiles, int kinds) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int nx = I.P.nx, ny = I.P.ny, ncx = (nx + 31) >> 5;
@@ -151,6 +151,7 @@ static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constan
   const int y0 = ti / ncx * 8, x = (ti % ncx) * 32 + lane;
   const uint8_t* type = I.type[int(I.scal[S_STEP] & 1ULL)];
   int bf = FILL ? counts[ti] : 0, bm = FILL ? counts[ntiles + ti] : 0;
+  int br = FILL && kinds > 2 ? int(I.N) - int(I.scal[S_NRES]) + counts[2 * ntiles + ti] : 0;
   const unsigned below = (1u << lane) - 1u;
 #pragma unroll 4
   for (int r = 0; r < 8; ++r) {
@@ -167,7 +168,8 @@ static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constan
       }
     }
     const bool fl = in && is_fluid(t);
-    const unsigned mf = __ballot_sync(FULL, fl), mm = __ballot_sync(FULL, face);
+    const bool res = kinds > 2 && (t == T_INLET || t == T_OUTLET);
+    const unsigned mf = __ballot_sync(FULL, fl), mm = __ballot_sync(FULL, face), mr = __ballot_sync(FULL, res);
     if constexpr (FILL) {
       if (fl) {
         I.flist[bf + __popc(mf & below)] = node;
@@ -177,28 +179,23 @@ static __global__ void __launch_bounds__(ST_THREADS) k_list(const __grid_constan
         I.mlist[bm + __popc(mm & below)] = node;
         atomicOr(&I.mbits[node >> 5], 1u << (node & 31));
       }
-      const bool res = reservoirs && (t == T_INLET || t == T_OUTLET);
-      const unsigned mr = __ballot_sync(FULL, res);
-      if (mr) {
-        int at = 0;
-        if (lane == 0) at = (int)atomicAdd(&I.scal[S_NRES], (unsigned long long)__popc(mr));
-        at = __shfl_sync(FULL, at, 0);
-        if (res) I.flist[I.N - 1 - (at + __popc(mr & below))] = node;
-      }
+      if (res) I.flist[br + __popc(mr & below)] = node;
     }
     bf += __popc(mf);
     bm += __popc(mm);
+    br += __popc(mr);
   }
   if (!FILL && lane == 0) {
     counts[ti] = bf;
     counts[ntiles + ti] = bm;
+    if (kinds > 2) counts[2 * ntiles + ti] = br;
   }
 }
-// One block: exclusive sums of both count arrays in place, totals into scal.
-static __global__ void __launch_bounds__(1024) k_list_scan(int* __restrict__ counts, int ntiles, unsigned long long* scal) {
+// One block: exclusive sums of the count arrays in place, totals into scal.
+static __global__ void __launch_bounds__(1024) k_list_scan(int* __restrict__ counts, int ntiles, unsigned long long* scal, int kinds) {
   __shared__ int sums[1024];
   const int per = (ntiles + 1023) / 1024;
-  for (int k = 0; k < 2; ++k) {
+  for (int k = 0; k < kinds; ++k) {
     int* c = counts + k * ntiles;
     const int lo = min(threadIdx.x * per, ntiles), hi = min(lo + per, ntiles);
     int s = 0;
@@ -222,18 +219,19 @@ static __global__ void __launch_bounds__(1024) k_list_scan(int* __restrict__ cou
   }
 }
 
-// Reservoir node i of an instance.  A reservoir node never is fluid, so the array of
-// the fluid list has room for it.
-__device__ __forceinline__ int reservoir_node(const DevInst* I, int i) { return I->flist[I->N - 1 - i]; }
+// Reservoir node i of the nres of an instance.  A reservoir node never is fluid, so
+// the array of the fluid list has room for it at its end.
+__device__ __forceinline__ int reservoir_node(const DevInst* I, int nres, int i) { return I->flist[I->N - nres + i]; }
 
 // Reservoir nodes i .. i + 31 of an instance: densities of the step, potentials
 // and codes.
 template <class TF, class R>
 __device__ __noinline__ void reservoir_pot(const DevInst* I, int cur, unsigned long long step, int i) {
   i += threadIdx.x & 31;
-  if (i >= (int)I->scal[S_NRES]) return;
+  const int nres = (int)I->scal[S_NRES];
+  if (i >= nres) return;
   const DevParams& P = I->P;
-  const int node = reservoir_node(I, i);
+  const int node = reservoir_node(I, nres, i);
   const uint8_t* tin = I->type[cur];
   const uint8_t t = tin[node] & T_MASK;
   const R theta = theta_of<R>(I);
@@ -413,9 +411,10 @@ __device__ __forceinline__ void reservoir_push_node(const DevParams& P, const ui
 template <class TF, class TG, class R, int NS>
 __device__ __noinline__ void reservoir_push(const DevInst* I, int cur, unsigned long long step, int i) {
   i += threadIdx.x & 31;
-  if (i >= (int)I->scal[S_NRES]) return;
+  const int nres = (int)I->scal[S_NRES];
+  if (i >= nres) return;
   const DevParams& P = I->P;
-  const int node = reservoir_node(I, i), N = (int)I->N;
+  const int node = reservoir_node(I, nres, i), N = (int)I->N;
   const uint8_t* tin = I->type[cur];
   const TF* fin = (const TF*)I->f[cur];
   const uint8_t t = tin[node] & T_MASK;
