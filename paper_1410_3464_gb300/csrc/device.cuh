@@ -118,12 +118,14 @@ struct DevInst {
   int* evlist;                // [2 evcap] event node indices, vanishing nodes (in the bytes of pot)
   int* claim;                 // [N] zero except while the amendment kernel runs
   int* flist;                 // [N] fluid nodes (S_NFLUID entries from the front; an entry may have filled
-                              // since); reservoir nodes (S_NRES entries) at its end (reservoir_node)
+                              // since); reservoir nodes, which never are fluid, at its end
   int* mlist;                 // [N] minerals with a fluid axis neighbour (S_NFACE entries; an entry may
                               // have lost its fluid neighbours, or dissolved, since)
   unsigned* fbits;            // [(N + 31) / 32] bit per node: listed in flist
   unsigned* mbits;            // [(N + 31) / 32] bit per node: listed in mlist
   unsigned long long* scal;   // [S_NSCAL]
+  int* reslist;               // [nres] reservoir nodes (set once k_list has counted them)
+  int nres;
   long long N;
   int evcap;
   int read_once;              // populations may leave L2 once k_move has read them (pslbm_create)

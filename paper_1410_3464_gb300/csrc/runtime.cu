@@ -877,6 +877,9 @@ pslbm_status pslbm_create(const uint8_t* mask, const double* rho1, const double*
     h->run.nfluid.assign(1, (int)counts[0]);
     h->run.nface.assign(1, (int)counts[1]);
     h->run.nres.assign(1, (int)counts[2]);
+    I.nres = (int)counts[2];
+    I.reslist = I.flist + (N - I.nres);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->d, &I, sizeof(DevInst), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) {
       st = fail(nullptr, e == cudaErrorMemoryAllocation ? PSLBM_ERR_OOM : PSLBM_ERR_CUDA,
                 std::string("create: ") + cudaGetErrorString(e));

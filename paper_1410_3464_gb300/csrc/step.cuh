@@ -219,19 +219,14 @@ static __global__ void __launch_bounds__(1024) k_list_scan(int* __restrict__ cou
   }
 }
 
-// Reservoir node i of the nres of an instance.  A reservoir node never is fluid, so
-// the array of the fluid list has room for it at its end.
-__device__ __forceinline__ int reservoir_node(const DevInst* I, int nres, int i) { return I->flist[I->N - nres + i]; }
-
 // Reservoir nodes i .. i + 31 of an instance: densities of the step, potentials
 // and codes.
 template <class TF, class R>
 __device__ __noinline__ void reservoir_pot(const DevInst* I, int cur, unsigned long long step, int i) {
   i += threadIdx.x & 31;
-  const int nres = (int)I->scal[S_NRES];
-  if (i >= nres) return;
+  if (i >= I->nres) return;
   const DevParams& P = I->P;
-  const int node = reservoir_node(I, nres, i);
+  const int node = I->reslist[i];
   const uint8_t* tin = I->type[cur];
   const uint8_t t = tin[node] & T_MASK;
   const R theta = theta_of<R>(I);
@@ -411,10 +406,9 @@ __device__ __forceinline__ void reservoir_push_node(const DevParams& P, const ui
 template <class TF, class TG, class R, int NS>
 __device__ __noinline__ void reservoir_push(const DevInst* I, int cur, unsigned long long step, int i) {
   i += threadIdx.x & 31;
-  const int nres = (int)I->scal[S_NRES];
-  if (i >= nres) return;
+  if (i >= I->nres) return;
   const DevParams& P = I->P;
-  const int node = reservoir_node(I, nres, i), N = (int)I->N;
+  const int node = I->reslist[i], N = (int)I->N;
   const uint8_t* tin = I->type[cur];
   const TF* fin = (const TF*)I->f[cur];
   const uint8_t t = tin[node] & T_MASK;
