@@ -190,7 +190,9 @@ pslbm_status pslbm_read_fields(pslbm_t h, uint32_t fields, void* const* out);
  * mean duration per step (ms) of the streaming kernels (Eqs. 6-31), the VOP
  * kernel (Eqs. 32-35) and the amendment kernel (Section 4.5); total_ms the
  * mean time per step from the first to the last event.  Same results as
- * pslbm_step. */
+ * pslbm_step, which takes the VOP and the amendment kernel in one launch where
+ * the list of minerals that face fluid is short: here they are two launches
+ * always, and total_ms is the time of that form. */
 pslbm_status pslbm_profile_step(pslbm_t h, int64_t n, double* kernel_ms, double* total_ms);
 
 /* Freeze the simulation once it has taken `limit` steps (limit < 0: no limit).
@@ -285,7 +287,7 @@ pslbm_status pslbm_batch_set_staging(pslbm_batch_t b, int32_t mode);
 pslbm_status pslbm_batch_get_staging(pslbm_batch_t b, int32_t* staged, int32_t* available);
 /* As pslbm_profile_step for a batch: n >= 1 steps without graph capture, each
  * kernel timed with CUDA events on the library stream; kernel_ms[3] receives
- * the mean ms per step of the bulk, VOP and amendment kernels over all
+ * the mean ms per step of the streaming, VOP and amendment kernels over all
  * members, total_ms (nullable) the mean ms per step.  Synchronises. */
 pslbm_status pslbm_batch_profile_step(pslbm_batch_t b, int64_t n, double* kernel_ms, double* total_ms);
 /* Per-step monitor of a batch: the smallest step count over the members and

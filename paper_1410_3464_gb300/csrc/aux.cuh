@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(FIELD_THREADS) k_fields_pot(const DevInst* __r
       r2 = fshift<R>(P, 1, t) + density_shifted<R>(F, 1, node);
     } else {
       double u, v;
-      reservoir_rho(P, t, step, t == T_OUTLET && outlet_up_liquid<R, TF>(P, T, F, N, node, theta_of<R>(Ip)), u, v);
+      reservoir_rho(P, t, step, t == T_OUTLET && outlet_up_liquid<R, TF>(P, T, F, node, theta_of<R>(Ip)), u, v);
       r1 = R(u);
       r2 = R(v);
     }

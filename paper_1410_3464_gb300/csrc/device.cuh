@@ -261,7 +261,7 @@ __host__ __device__ inline double ord_dec(unsigned long long e) {
 }
 
 // The liquid threshold of the current step in the compute precision, decoded
-// once per step by the amendment kernel (no FP64 arithmetic in the FP32 bulk).
+// once per step by the amendment kernel (no FP64 arithmetic in the FP32 kernels).
 template <class R> __device__ __forceinline__ R theta_of(const DevInst* Ip);
 template <> __device__ __forceinline__ double theta_of<double>(const DevInst* Ip) {
   return __longlong_as_double((long long)Ip->scal[S_THETA]);
@@ -325,11 +325,9 @@ __device__ __forceinline__ R fshift(const DevParams& P, int comp, uint8_t t) {
   return (t & T_MASK) == T_GAS ? rp<R>(P).shift_fg[comp] : rp<R>(P).shift_f[comp];
 }
 
-// Marking of an arbitrary node from global memory (same arithmetic as the
-// shared-memory path, so both give the same answer bit for bit).
+// Marking of an arbitrary node, by k_pot's arithmetic: the same answer, bit for bit.
 template <class R, class TF>
-__device__ __forceinline__ bool liquid_at(const DevParams& P, const uint8_t* tin, const TF* fin, int N, int node,
-                                          R theta) {
+__device__ __forceinline__ bool liquid_at(const DevParams& P, const uint8_t* tin, const TF* fin, int node, R theta) {
   uint8_t t = tin[node] & T_MASK;
   if (!is_fluid(t)) return false;
   R rho1 = fshift<R>(P, 0, t) + density_shifted<R>(fin, 0, node);
@@ -338,11 +336,11 @@ __device__ __forceinline__ bool liquid_at(const DevParams& P, const uint8_t* tin
 
 // Marking of the node upstream of an outlet node at index idx.
 template <class R, class TF>
-__device__ __forceinline__ bool outlet_up_liquid(const DevParams& P, const uint8_t* tin, const TF* fin, int N, int idx,
+__device__ __forceinline__ bool outlet_up_liquid(const DevParams& P, const uint8_t* tin, const TF* fin, int idx,
                                                  R theta) {
   int xn, yn;
   if (!nbr(P, idx % P.nx, idx / P.nx, P.out_dx, P.out_dy, xn, yn)) return false;
-  return liquid_at<R, TF>(P, tin, fin, N, yn * P.nx + xn, theta);
+  return liquid_at<R, TF>(P, tin, fin, yn * P.nx + xn, theta);
 }
 
 // Explicitly rounded operations.  The formulas are written with these (fused
@@ -537,19 +535,6 @@ __device__ __forceinline__ void feq_pairs(R dr, R rho, R ux, R uy, R uu, R* feq)
     feq[pa[q]] = radd<R>(sym, asym);
     feq[pb[q]] = rsub<R>(sym, asym);
   }
-}
-
-// The five D2Q5 equilibria of Eq. 21 relative to the species' shift sh:
-// J_a (C - sh) + C e.u / 2, opposite directions together.
-template <class R>
-__device__ __forceinline__ void geq_pairs(R J0, R Ja, R C, R sh, R ux, R uy, R* geq) {
-  const R cs = rsub<R>(C, sh), hc = rmul<R>(R(0.5), C);
-  const R sa = rmul<R>(Ja, cs), ax = rmul<R>(hc, ux), ay = rmul<R>(hc, uy);
-  geq[0] = rmul<R>(J0, cs);
-  geq[1] = radd<R>(sa, ax);
-  geq[3] = rsub<R>(sa, ax);
-  geq[2] = radd<R>(sa, ay);
-  geq[4] = rsub<R>(sa, ay);
 }
 
 // exp(v) - 1 without the cancellation of evaluating exp(v) first (phi_1 of

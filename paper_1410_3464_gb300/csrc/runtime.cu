@@ -1,5 +1,5 @@
 // Host runtime behind the C ABI of include/pslbm.h: parameter validation,
-// device allocation of the structure-of-arrays state, tile lists, CUDA-graph
+// device allocation of the state, node lists and the layout of the work, CUDA-graph
 // capture of whole steps, field read-out and batches.
 #include <cuda_runtime.h>
 
@@ -968,7 +968,7 @@ pslbm_status pslbm_set_tile_shape(pslbm_t h, int32_t tile_x, int32_t tile_y) {
   if (!h) return fail(nullptr, PSLBM_ERR_PARAM, "handle is NULL");
   if (set_shape(h->run, tile_x, tile_y) != PSLBM_OK)
     return fail(h, PSLBM_ERR_PARAM,
-                "unsupported tile shape (0x0, 16x16, 32x8, 16x32 or 32x16; the last two have no staged kernel)");
+                "unsupported tile shape (0x0, 16x16, 32x8, 16x32 or 32x16; not the last two while staging 1 is asked for)");
   return PSLBM_OK;
 }
 
@@ -983,7 +983,7 @@ pslbm_status pslbm_get_tile_shape(pslbm_t h, int32_t* tile_x, int32_t* tile_y, i
 pslbm_status pslbm_set_staging(pslbm_t h, int32_t mode) {
   if (!h) return fail(nullptr, PSLBM_ERR_PARAM, "handle is NULL");
   if (set_staging(h->run, mode) != PSLBM_OK)
-    return fail(h, PSLBM_ERR_PARAM, "staging must be -1, 0, 1 or 2 (1, 2 only where the handle has TMA descriptors)");
+    return fail(h, PSLBM_ERR_PARAM, "staging must be -1, 0, 1 or 2 (1, 2 only with FP32 populations and rows of a multiple of 16 bytes)");
   return PSLBM_OK;
 }
 
@@ -1259,7 +1259,7 @@ pslbm_status pslbm_batch_get_tile_shape(pslbm_batch_t b, int32_t* tile_x, int32_
 pslbm_status pslbm_batch_set_staging(pslbm_batch_t b, int32_t mode) {
   if (!b) return fail(nullptr, PSLBM_ERR_PARAM, "batch is NULL");
   if (set_staging(b->run, mode) != PSLBM_OK)
-    return fail(nullptr, PSLBM_ERR_PARAM, "staging must be -1, 0, 1 or 2 (1, 2 only where every member has TMA descriptors)");
+    return fail(nullptr, PSLBM_ERR_PARAM, "staging must be -1, 0, 1 or 2 (1, 2 only where every member has them)");
   return PSLBM_OK;
 }
 

@@ -231,7 +231,7 @@ __device__ __noinline__ void reservoir_pot(const DevInst* I, int cur, unsigned l
   const uint8_t t = tin[node] & T_MASK;
   const R theta = theta_of<R>(I);
   double a, b;
-  reservoir_rho(P, t, step, t == T_OUTLET && outlet_up_liquid<R, TF>(P, tin, (const TF*)I->f[cur], (int)I->N, node, theta), a, b);
+  reservoir_rho(P, t, step, t == T_OUTLET && outlet_up_liquid<R, TF>(P, tin, (const TF*)I->f[cur], node, theta), a, b);
   unsigned status = 0;
   R ps, p1, p2;
   potentials<R>(P, R(a), R(b), ps, p1, p2, status);
@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : 8)
 // equilibrium into its liquid ones.
 template <class R, class TF, class TG, int NS>
 __device__ __forceinline__ void reservoir_push_node(const DevParams& P, const uint8_t* tin, const TF* fin, const TG* gin,
-                                                 TF* fout, TG* gout, int N, int x, int y, uint8_t t, R r1, R r2,
+                                                 TF* fout, TG* gout, int x, int y, uint8_t t, R r1, R r2,
                                                  unsigned nbits, bool marked) {
   R ux = R(0), uy = R(0);
   int xn, yn;
@@ -408,7 +408,7 @@ __device__ __noinline__ void reservoir_push(const DevInst* I, int cur, unsigned 
   i += threadIdx.x & 31;
   if (i >= I->nres) return;
   const DevParams& P = I->P;
-  const int node = I->reslist[i], N = (int)I->N;
+  const int node = I->reslist[i];
   const uint8_t* tin = I->type[cur];
   const TF* fin = (const TF*)I->f[cur];
   const uint8_t t = tin[node] & T_MASK;
@@ -421,8 +421,8 @@ __device__ __noinline__ void reservoir_push(const DevInst* I, int cur, unsigned 
     if (nbr(P, x, y, EX(a), EY(a), xn, yn)) nbits |= unsigned(I->code[yn * P.nx + xn] & 0xF) << (4 * (a - 1));
   }
   double r1, r2;
-  reservoir_rho(P, t, step, t == T_OUTLET && outlet_up_liquid<R, TF>(P, tin, fin, N, node, theta), r1, r2);
-  reservoir_push_node<R, TF, TG, NS>(P, tin, fin, (const TG*)I->g[cur], (TF*)I->f[cur ^ 1], (TG*)I->g[cur ^ 1], N, x, y, t,
+  reservoir_rho(P, t, step, t == T_OUTLET && outlet_up_liquid<R, TF>(P, tin, fin, node, theta), r1, r2);
+  reservoir_push_node<R, TF, TG, NS>(P, tin, fin, (const TG*)I->g[cur], (TF*)I->f[cur ^ 1], (TG*)I->g[cur ^ 1], x, y, t,
                                      R(r1), R(r2), nbits, (I->code[node] & C_MARK) != 0);
 }
 

@@ -260,7 +260,8 @@ class Simulation:
         _check(load().pslbm_sync(self.h), self.h)
 
     def profile_step(self, n=1):
-        """Run n steps with per-kernel CUDA-event timing; returns
+        """Run n steps with per-kernel CUDA-event timing (VOP and amendment as two
+        launches, which step() joins where few minerals face fluid); returns
         ({'bulk', 'vop', 'amend'} mean ms per step, mean total ms per step)."""
         k = (C.c_double * 3)()
         t = C.c_double()
@@ -400,7 +401,8 @@ class Batch:
         return sg.value, bool(av.value)
 
     def profile_step(self, n=1):
-        """Run n steps with per-kernel CUDA-event timing; returns
+        """Run n steps with per-kernel CUDA-event timing (VOP and amendment as two
+        launches, which step() joins where few minerals face fluid); returns
         ({'bulk', 'vop', 'amend'} mean ms per step, mean total ms per step)."""
         k = (C.c_double * 3)()
         t = C.c_double()
