@@ -275,7 +275,10 @@ pslbm_status pslbm_budget_device_noalloc(pslbm_t h, double* out);
  * one launch per kernel over a packed list of work of all members.  The
  * members stay valid handles; they must not be stepped on their own while
  * the batch exists.  tile_x, tile_y choose the tile shape (16x16, 32x8,
- * 16x32 or 32x16, as for pslbm_set_tile_shape; 0, 0: the default). */
+ * 16x32 or 32x16, as for pslbm_set_tile_shape; 0, 0: the default).  Steps are
+ * queued as by pslbm_step; where members' lists have outgrown the packed one,
+ * the first step call after a sync or read that saw it makes it again, which
+ * synchronises. */
 pslbm_status pslbm_batch_create(int32_t n, const pslbm_t* members, int32_t tile_x, int32_t tile_y,
                                 pslbm_batch_t* out);
 pslbm_status pslbm_batch_step(pslbm_batch_t b, int64_t n);

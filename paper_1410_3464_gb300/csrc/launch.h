@@ -5,6 +5,19 @@
 
 namespace pslbm {
 
+// SMs of the device (152 on a whole GB300).
+inline int device_sms() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) {
+      cudaGetLastError();
+      v = 152;
+    }
+    return v;
+  }();
+  return n;
+}
+
 struct Launchers {
   // work: the VOP chunks of a batch (null for one simulation); nwork: their number
   void (*vop)(cudaStream_t, const DevInst*, const Work* work, int nwork);

@@ -409,22 +409,25 @@ int list_warps(long long n, long long N, double turns) {
 
 // Turns a warp of the streaming kernels takes.  Several, because each saves a
 // start (descriptor, step count, list) and has the next turn's list entry in
-// flight.  One simulation up to 64 turns: one wave of 8 warps an SM (FP64: 16),
-// whose warps sweep the list together, so that what neighbours share is met in
-// L2: 1024x512 FP32 48.7 us a step, against 56.7 with 16 warps, 54.4 with 8 turns
-// in two waves and 66 with one turn; 2048x1024 161, 171, 169, 181; 1024x512 FP64
-// 209 with 16 warps, 214 with 8, 228 with 2 turns.  k_pot, with a third of the
-// loads in flight, takes 16 in either type (8: 2048x1024 177 us).  Longer lists: 8 turns
-// (4096x2048 601 us, one wave 619, one turn 619).  A batch, whose members' lists
-// do not join up: 8 turns (FP64 2), fewer where that leaves SMs idle (24 members
-// 384 us, one wave 405 to 450, one turn 428).
+// flight.  One simulation: one wave of 8 warps an SM (FP64: 16), whose warps sweep the
+// list together, so that what neighbours share is met in L2: 1024x512 FP32 48.7 us a
+// step, against 56.7 with 16 warps, 54.4 with 8 turns in two waves and 66 with one turn
+// (before the evict-first loads).  k_pot, with a third of the loads in flight, takes 16
+// in either type (8: 2048x1024 177 us, 16: 161).  Long lists: FP32 8 turns from 80 a
+// warp on (one wave and 8 turns: 2048x1024 165 and 179 us, 2896x1448, 65 a warp, 314 and
+// 324, 3072x2048, 97 a warp, 477 and 474, 8192x4096 2524 and 2456); FP64 2 turns from 5
+// a warp on (768x512 208 and 211, 1024x512, 4.1 a warp, 264 and 265, 1200x600, 5.6 a
+// warp, 342 and 336, 2048x1024 913 and 891, 4096x2048 3510 and 3426).  A batch, whose
+// members' lists do not join up: 8 turns (FP64 2), fewer where that leaves SMs idle (24
+// members 384 us, one wave 405 to 450, one turn 428).
 double stream_turns(const Stepper& st, bool pot) {
   if (st.fix_shape >= 0) return SHAPE_TX[st.fix_shape] * SHAPE_TY[st.fix_shape] / 64;
   double chunks = 0;
   for (int f : st.nfluid) chunks += (f + 31) / 32;
-  const double wave = 152.0 * (st.fp64 || (pot && st.mode == M_SINGLE) ? 16 : 8);
-  if (st.mode == M_SINGLE && chunks <= 64 * 152 * (st.fp64 ? 16 : 8)) return std::max(1.0, chunks / wave);
-  double turns = st.mode != M_SINGLE && st.fp64 ? 2 : 8;
+  const double sms = device_sms();
+  const double wave = sms * (st.fp64 || (pot && st.mode == M_SINGLE) ? 16 : 8);
+  if (st.mode == M_SINGLE && chunks <= sms * (st.fp64 ? 5 * 16 : 80 * 8)) return std::max(1.0, chunks / wave);
+  double turns = st.fp64 ? 2 : 8;
   while (turns > 1 && chunks / turns < wave) turns /= 2;
   return turns;
 }
