@@ -97,3 +97,31 @@ def test_a_long_run_stays_as_fast_as_a_fresh_one(pslbm):
     with simulation(pslbm, now, pslbm.FP32) as sim:
         fresh = us(sim)
     assert old <= 1.2 * fresh, (old, fresh)
+
+
+@pytest.mark.parametrize("members", [0, 2])
+def test_plans_follow_the_lists(pslbm, members):
+    """Nodes that dissolve fast: the list of minerals passes the length up to which VOP
+    and amendment are one launch and, made again, falls below it; the lists outgrow the
+    work laid out for them.  Each sync lets the host see their lengths.  One simulation,
+    and a batch, against steps that keep list and plan."""
+    sc = bank(200, 120, 80, 3.0)
+    with simulation(pslbm, sc, pslbm.FP32) as b:
+        sims = [simulation(pslbm, sc, pslbm.FP32) for _ in range(max(1, members))]
+        run = pslbm.Batch(sims) if members else sims[0]
+        gone = [0]
+        for n in (150, 150, 400, 400, 300, 200):
+            run.step(n)
+            run.sync()
+            b.profile_step(n)
+            ref = b.read()
+            for s in sims:
+                got = s.read()
+                for name in ref:
+                    np.testing.assert_array_equal(got[name], ref[name], err_msg=f"{n} {name}")
+            gone.append(int((sc["mask"] == 2).sum() - (ref["type"] == 2).sum()))
+        assert gone[2] > 300 and gone[-1] > 2300, gone
+        if members:
+            run.close()
+        for s in sims:
+            s.close()
