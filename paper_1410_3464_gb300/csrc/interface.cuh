@@ -430,8 +430,8 @@ __global__ void __launch_bounds__(NTHREADS) k_amend(const DevInst* __restrict__ 
 // k_vop and k_amend of an instance in one block, for lists that one block can take
 // at once (FUSE_FACE).  What the block's threads wrote they read back after a block
 // barrier; nothing passes between blocks.  Saves a dependent launch and its round
-// trip: 131x67 FP32 12.4 -> 11.8 us a step, 100x160 16.4 -> 15.9, 102x90 FP64 24.1 ->
-// 23.3, 201x201 FP64 32.8 -> 32.3.
+// trip: 131x67 FP32 12.0 -> 11.4 us a step, 100x160 15.3 -> 14.7, 102x90 FP64 24.0 ->
+// 23.4, 201x201 FP64 36.0 -> 35.3.
 template <class TF, class TG, class R, int NS>
 __global__ void __launch_bounds__(NTHREADS) k_vop_amend(const DevInst* __restrict__ insts) {
   step_begin();

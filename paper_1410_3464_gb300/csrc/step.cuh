@@ -244,7 +244,8 @@ __device__ __noinline__ void reservoir_pot(const DevInst* I, int cur, unsigned l
 // out; in FP64 by the equation of state and the exponentials.  A kernel of its own
 // because one that also collides had to hold or recompute the ring of neighbours:
 // 1,522 warp instructions and a block barrier per 32 nodes, 77 us at 1024x512 FP32
-// (FP64 460), where k_pot and k_move take 41 (FP64 213) together.
+// (FP64 460), where k_pot and k_move take 39 (FP64 254) together (between events, on a
+// lattice that the step before has left in L2 as far as it fits).
 template <class TF, class R, int MODE>
 __global__ void __launch_bounds__(ST_THREADS, sizeof(R) == 8 ? 4 : 8)
     k_pot(const Work* __restrict__ work, int nwork, int nstream, const DevInst* __restrict__ insts,
@@ -429,9 +430,11 @@ __device__ __noinline__ void reservoir_push(const DevInst* I, int cur, unsigned 
 // Bound by memory latency in FP32 (18 + 5 NS populations and nine potentials in, the
 // populations out; 128 registers, so 16 warps an SM at most, and more warps at fewer
 // registers measured slower), by the FP64 pipe in FP64, where an instruction of a warp
-// takes 64 cycles however many lanes are in: hence the regrouped collisions, few
-// comparisons, and lists without idle lanes (1024x512 FP64: 322 us a step before the
-// regrouping, 228 after).  The FP32 arithmetic keeps its order and rounding.
+// takes 64 cycles however many lanes are in: hence no BGK difference at tau = 1, the
+// density from k_pot, few comparisons, and lists without idle lanes (1024x512 FP64: 322 us
+// a step before, 265 now).  Forms with fewer roundings to share out between directions
+// were faster (228) and further from 64 bits: FP64 and FP32 keep the order and the
+// rounding of the equations.
 // Everything that depends on the node alone is loaded before the first use; the loop
 // stays within the instruction cache (nothing rare inline but the Step-2 amendment).
 template <class TF, class TG, class R, int NS, int MODE>
