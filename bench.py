@@ -409,7 +409,7 @@ def ours_arm(args):
         for _ in range(args.steps):
             r2.step(1)
             r2.monitor()
-            mon_bytes += 16 * len(sims2) if batch else 80
+            mon_bytes += 16 * len(sims2) if batch else 32
         if batch:
             r2.close()
         # every member's budget into one device buffer (no allocation per
